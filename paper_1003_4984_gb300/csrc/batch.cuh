@@ -24,7 +24,7 @@ __global__ void __launch_bounds__(256, 2) batch_kernel(const BatchHeader *__rest
     unsigned char *wbase = smem_raw + (size_t)warp * warp_smem_bytes<K, SPIN, MIXED>();
     const int nj = hdr->njobs[CLS];
     const int64_t total = hdr->total_tiles[CLS];
-    const int tile_pts = hdr->tile_pts;
+    const int tile_pts = hdr->tile_pts[CLS];
     const BatchJob *J = jobs + hdr->job_offset[CLS];
     if (nj <= 0) return;
     Counters ctr;

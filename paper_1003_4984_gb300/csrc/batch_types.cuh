@@ -20,8 +20,7 @@ struct BatchHeader {
     int njobs[BATCH_CLASSES];       // per class
     int job_offset[BATCH_CLASSES];  // index of the class's first job in the job array
     int64_t total_tiles[BATCH_CLASSES];
-    int tile_pts;
-    int pad;
+    int tile_pts[BATCH_CLASSES];    // targets per tile
 };
 
 }  // namespace flints

@@ -403,6 +403,30 @@ struct LaunchCfg {
     int warps_per_block, blocks_per_sm, tile_points;
 };
 
+// Targets per warp tile when the caller leaves the choice to the library.  A warp
+// works through its tile point by point (76 us per point at spin 2, K = 32 with 16
+// warps per SM), so a launch lasts about ceil(tiles / warps) rounds of a tile's
+// points plus its displacement pass, which costs about half a point whatever the
+// tile holds.  The size with the shortest such launch is taken, the largest one on
+// ties; past 8 rounds of full tiles the tail is within a few percent and the size
+// stays at its maximum, which displaces the most targets per pass.  Measured
+// (GB300, full tiles -> this rule): 1,009 targets (spin 0, K = 16) 389 -> 49 us,
+// 20,011 targets (spin 2, K = 32) 1222 -> 721 us.
+inline int auto_tile_points(int64_t count, int64_t warps) {
+    if (warps < 1 || count >= 8 * MAX_TILE_POINTS * warps) return MAX_TILE_POINTS;
+    int best = MAX_TILE_POINTS;
+    double best_cost = 0.0;
+    for (int t = MAX_TILE_POINTS; t >= 1; --t) {
+        const int64_t tiles = (count + t - 1) / t;
+        const double cost = (double)((tiles + warps - 1) / warps) * (t + 0.5);
+        if (t == MAX_TILE_POINTS || cost < best_cost) {
+            best = t;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+
 enum { CNT_POINTS = 0, CNT_NUGGET = 1, CNT_FALLBACK = 2, CNT_WINDOW = 3, CNT_FAILED = 4, CNT_N = 5 };
 
 // Correlation-table grid and stencil search disc of a K-nearest plan (host).

@@ -1560,7 +1560,6 @@ __global__ void __launch_bounds__(256, 2) lens_kernel(LensArgs a, int R_rings, i
 template <int K, int SPIN, int MIXED>
 cudaError_t launch_one(const LensArgs &a, int R_rings, const LaunchCfg &cfg, int num_sms, cudaStream_t st) {
     int wpb = cfg.warps_per_block > 0 ? cfg.warps_per_block : 4;
-    const int tile_pts = cfg.tile_points > 0 && cfg.tile_points < MAX_TILE_POINTS ? cfg.tile_points : MAX_TILE_POINTS;
     // the launch shape is a hint: keep the block within the opt-in shared memory
     const int fit = (int)(device_smem_optin() / warp_smem_bytes<K, SPIN, MIXED>());
     if (wpb > fit) wpb = fit > 0 ? fit : 1;
@@ -1573,8 +1572,10 @@ cudaError_t launch_one(const LensArgs &a, int R_rings, const LaunchCfg &cfg, int
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     if (cfg.blocks_per_sm > 0 && cfg.blocks_per_sm < per_sm) per_sm = cfg.blocks_per_sm;
-    const int64_t ntiles = (a.count + tile_pts - 1) / tile_pts;
     int64_t blocks = (int64_t)num_sms * per_sm;
+    const int tile_pts = cfg.tile_points > 0 ? (cfg.tile_points < MAX_TILE_POINTS ? cfg.tile_points : MAX_TILE_POINTS)
+                                             : auto_tile_points(a.count, blocks * wpb);
+    const int64_t ntiles = (a.count + tile_pts - 1) / tile_pts;
     const int64_t need = (ntiles + wpb - 1) / wpb;
     if (blocks > need) blocks = need;
     if (blocks < 1) blocks = 1;
