@@ -65,6 +65,8 @@ struct flints_plan_s {
     double *d_cl, *d_clbb, *d_f, *d_g, *d_fm, *d_gm;
     Coef64 *d_c64, *d_cm64;  // xi+ (spin 0: xi) and, spin 2, xi- interpolation coefficients
     float4 *d_c32, *d_cm32;
+    CoefFx *d_cfx;  // FP64 plans: the table of the fixed-point solve, used when `fixed`
+    bool fixed;
     unsigned long long *d_counters;
     unsigned long long *d_queue;  // QUEUE_SLOTS blocks of BATCH_CLASSES tile-queue counters, one block per call
     unsigned queue_next;
@@ -144,6 +146,16 @@ TableGrid table_grid(int64_t nside, int K, int lmax, const double *cl, const dou
     g.R_rings = (int)std::ceil(1.5 * g.r * (double)nside) + 1;
     return g;
 }
+bool fixed_table_ok(const TableGrid &g, int spin, int lmax, const double *cl, const double *cl_bb, double xi0) {
+    double x0 = 0.0, x1 = 0.0;
+    for (int l = 0; l <= lmax; ++l) {
+        const double a = (2.0 * l + 1.0) / (4.0 * PI) * (std::fabs(cl[l]) + (cl_bb ? std::fabs(cl_bb[l]) : 0.0));
+        x0 += a;
+        x1 += a * (double)l * (l + 1.0) / 4.0;
+    }
+    // c2 = 3D - 2 m0 - m1 and c3 = m0 + m1 - 2D, |D|, |m| <= h max|xi'|
+    return x0 <= 1.9 * xi0 && 6.0 * g.h * x1 <= 1.9 * xi0 && (spin == 0 || g.r2 <= 0.03125);
+}
 }  // namespace flints
 
 static void free_plan_memory(flints_plan_s *p) {
@@ -157,6 +169,7 @@ static void free_plan_memory(flints_plan_s *p) {
     cudaFree(p->d_c32);
     cudaFree(p->d_cm64);
     cudaFree(p->d_cm32);
+    cudaFree(p->d_cfx);
     cudaFree(p->d_counters);
     cudaFree(p->d_queue);
     cudaFree(p->d_jt);
@@ -201,16 +214,14 @@ int flints_plan(flints_plan_t *out, int64_t nside, int lmax, const double *cl, c
     p->flags = flags;
 
     // Table domain and size, and the search disc (the grid rule of table_grid).
-    {
-        const TableGrid tg = table_grid(nside, K, lmax, cl, spin != 0 ? cl_bb : nullptr);
-        p->r = tg.r;
-        p->r2 = tg.r2;
-        p->t_max = tg.t_max;
-        p->n = tg.n;
-        p->h = tg.h;
-        p->inv_h = tg.inv_h;
-        p->R_rings = tg.R_rings;
-    }
+    const TableGrid tg = table_grid(nside, K, lmax, cl, spin != 0 ? cl_bb : nullptr);
+    p->r = tg.r;
+    p->r2 = tg.r2;
+    p->t_max = tg.t_max;
+    p->n = tg.n;
+    p->h = tg.h;
+    p->inv_h = tg.inv_h;
+    p->R_rings = tg.R_rings;
     if (2 * p->R_rings + 2 > 32) {
         delete p;
         return fail(FLINTS_EINVAL, "flints_plan: search disc spans too many rings");
@@ -242,6 +253,9 @@ int flints_plan(flints_plan_t *out, int64_t nside, int lmax, const double *cl, c
     if (spin != 0) {
         ALLOC(p->d_cm64, (size_t)p->n * sizeof(Coef64));
         ALLOC(p->d_cm32, (size_t)p->n * 2 * sizeof(float4));
+    }
+    if (precision == FLINTS_FP64 && !(flags & FLINTS_SPIN2_AUGMENTED)) {
+        ALLOC(p->d_cfx, (size_t)p->n * sizeof(CoefFx));
     }
     ALLOC(p->d_counters, CNT_N * sizeof(unsigned long long));
     ALLOC(p->d_queue, (size_t)QUEUE_SLOTS * BATCH_CLASSES * sizeof(unsigned long long));
@@ -280,6 +294,9 @@ int flints_plan(flints_plan_t *out, int64_t nside, int lmax, const double *cl, c
         return bail(e, "flints_plan: table coefficients");
     if (spin != 0 && (e = finish_table(p->d_fm, p->d_gm, p->n, p->h, xi0, p->d_cm64, p->d_cm32, st)) != cudaSuccess)
         return bail(e, "flints_plan: xi- table");
+    p->fixed = p->d_cfx && fixed_table_ok(tg, spin, lmax, cl, spin != 0 ? cl_bb : nullptr, xi0);
+    if (p->fixed && (e = launch_fixed_table(p->d_c64, p->n, p->d_cfx, st)) != cudaSuccess)
+        return bail(e, "flints_plan: table coefficients");
     if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return bail(e, "flints_plan: table coefficients");
     *out = p;
     return FLINTS_OK;
@@ -342,11 +359,14 @@ static int run(flints_plan_t p, int64_t nside_tgt, int64_t first, int64_t count,
     a.tab.inv_h_hi = (float)p->inv_h;
     a.tab.inv_h_lo = (float)(p->inv_h - (double)a.tab.inv_h_hi);
     a.tab.n = p->n;
+    a.tab.cfx = p->fixed ? p->d_cfx : nullptr;
     a.tabm = a.tab;
     a.tabm.c64 = p->d_cm64;
     a.tabm.c32 = p->d_cm32;
     a.xi0 = p->xi0;
     a.r2 = p->r2;
+    a.two_r = 2.0 * p->r;
+    a.inv_2r = 0.5 / p->r;
     a.counters = p->d_counters;
     // this call's slot: its tile-queue counters (and one-job table), zeroed on the stream
     const unsigned slot = p->queue_next++ % QUEUE_SLOTS;
@@ -639,8 +659,11 @@ int flints_batch_stage(flints_batch_t b, const flints_job *jobs, int n, int tile
         a.tab.inv_h_hi = (float)p->inv_h;
         a.tab.inv_h_lo = (float)(p->inv_h - (double)a.tab.inv_h_hi);
         a.tab.n = p->n;
+        a.tab.cfx = p->fixed ? p->d_cfx : nullptr;
         a.xi0 = p->xi0;
         a.r2 = p->r2;
+        a.two_r = 2.0 * p->r;
+        a.inv_2r = 0.5 / p->r;
         a.counters = p->d_counters;
         bj.R_rings = p->R_rings;
         bj.K = p->K;

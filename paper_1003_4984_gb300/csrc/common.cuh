@@ -359,12 +359,18 @@ struct alignas(32) Coef64 {
     double f, m, c2, c3;
 };
 
+// The same coefficients as integers, units of 2^-58 (the fixed-point solve).
+struct alignas(32) CoefFx {
+    int64_t f, m, c2, c3;
+};
+
 struct TableDev {
     const Coef64 *c64;  // per interval: f_k, h g_k, c2, c3 (Horner in s)
     const float4 *c32;   // per interval, double-float: (f.hi, f.lo, m.hi, m.lo), (c2.hi, c2.lo, c3.hi, c3.lo)
     double t_max, inv_h;
     float inv_h_hi, inv_h_lo;  // inv_h as a double-float pair
     int n;
+    const CoefFx *cfx;         // FP64 plans whose table and search disc suit the fixed-point solve, else NULL
 };
 
 struct LensArgs {
@@ -378,6 +384,7 @@ struct LensArgs {
     TableDev tab;
     double xi0;
     double r2;  // squared search radius (chord^2)
+    double two_r, inv_2r;  // the search disc's diameter and its reciprocal (fixed-point solve)
     unsigned long long *counters;  // points, nugget, fallback, window, failed
     int force_fallback;            // discard double-float solves (testing aid)
     int64_t nside_tgt;             // > 0: targets are the pixel centres of this grid (no deflection)
@@ -451,6 +458,11 @@ cudaError_t launch_xi_table(int spin, int lmax, const double *cl_dev, const doub
                             cudaStream_t st);
 cudaError_t finish_table(double *f, double *g, int n, double h, double xi0, Coef64 *c64, float4 *c32,
                          cudaStream_t st);
+cudaError_t launch_fixed_table(const Coef64 *c64, int n, CoefFx *cfx, cudaStream_t st);
+// Whether a plan's table and disc fit the fixed-point solve: every coefficient below 2 in
+// size (bounded through sum |a_l| and sum |a_l| l(l+1)/4, the largest |xi| and |xi'|), and
+// for spin 1 and 2, whose pair phases are a series in r^2, r^2 <= 2^-5 (Nside >= 24 at K = 32).
+bool fixed_table_ok(const TableGrid &g, int spin, int lmax, const double *cl, const double *cl_bb, double xi0);
 int device_sm_count();
 size_t device_smem_optin();
 

@@ -21,7 +21,9 @@
 //      best_temperature_field, gaussvar, major_eq, gaussvar_pol).
 // Precision R = double (FP64 path) or df (double-float on the FP32 pipe, the
 // mixed path: FP64 geometry and selection, double-float assembly, factor and
-// solves, FP64 fallback for points whose double-float factor fails).
+// solves, FP64 fallback for points whose double-float factor fails).  The FP64
+// path runs steps 3 to 5 in 64-bit fixed point first (solve_point_fixed) and
+// takes the FP64 form for the points that form declines.
 #pragma once
 #include <cstddef>
 #include <type_traits>
@@ -80,7 +82,12 @@ struct WarpSmem {
     // spin 2: per-neighbour target phase Phi0_i = phase(n' -> X_i), tangent-plane
     // coordinates (u, v) of X_i - n' at n', and squared chords to n'
     typename Ops<R>::T p0r[K], p0i[K], pu[K], pv[K];
-    float ktf[K];  // squared chords to n' (FP32, for the spherical-excess correction)
+    // squared chords to n': FP32 for the spherical-excess correction of the mixed path; the
+    // fixed-point solve of spin 1 and 2 keeps them as integers (units of t_max 2^-62)
+    union {
+        float ktf[K];
+        int64_t tau[SPIN == 1 || SPIN == 2 ? K : K / 2];
+    };
     union U {
         struct Cand {
             RingRec rings[32];
@@ -759,8 +766,512 @@ __device__ __forceinline__ bool factor_bordered(Elem *mat, int lane) {
         return bordered_cholesky<N, NB, R>(mat, lane);
 }
 
+// ------------------------------------------------------- fixed-point solve
+// The FP64 solve in 64-bit fixed point.  This part's FP64 pipe takes 16 cycles of an
+// SM per warp instruction, its integer multiply-add IMAD.WIDE (32 x 32 + 64 bits) half
+// a cycle (measured: 1.9 against 58 lanes per cycle and SM), and every quantity of the
+// solve is bounded: entries of S + n I, of its factor and of L^-1 c by 1, squared
+// chords by the search disc.  A number is (hi 2^32 + lo) 2^-58 with a signed low word,
+// so a multiply-add is three IMAD.WIDE into two 64-bit sums (hi hi, and the two cross
+// products together; lo lo, below 2^-54 of a unit in the last place's square, is
+// dropped) with no rounding until the sum is used: absolute error 2^-57 per sum, where
+// FP64 rounds every term of these sums, which are near 1, to 2^-53.
+// Measured (GB300): 1,048,583 spin-0 targets (K = 32, Nside 2048) 52.4 -> 27.8 ms; 524,309
+// Q/U targets (K = 32, Nside 4096) 61.2 -> 26.9 ms.
 // Returns false when a pivot of S + nugget I is not positive.
+constexpr int FXB = 58;
 
+struct alignas(8) fx {
+    int hi, lo;
+};
+struct alignas(16) fxc {
+    fx re, im;
+};
+__device__ __forceinline__ int64_t fx_val(fx a) {
+    return (int64_t)(((uint64_t)(uint32_t)a.hi << 32) + (uint64_t)(int64_t)a.lo);
+}
+// The pair of v.  The lowest bit is set, so that the low word is never -2^31 and both
+// words can be negated.
+__device__ __forceinline__ fx fx_split(int64_t v) {
+    const uint32_t l = (uint32_t)v | 1u;
+    return {(int)((uint32_t)((uint64_t)v >> 32) + (l >> 31)), (int)l};
+}
+__device__ __forceinline__ fx fx_neg(fx a) { return {(int)(0u - (unsigned)a.hi), (int)(0u - (unsigned)a.lo)}; }
+__device__ __forceinline__ uint64_t mul_wide(int a, int b) { return (uint64_t)((int64_t)a * (int64_t)b); }
+
+// Sum of products hh 2^64 + cr 2^32.  With operands of at most 2^58 (the factor's rows,
+// |L_r| <= 1) the cross sum of n terms stays below sqrt(n) 2^58; the data row, kept below
+// 1/2 per entry, adds at most n 2^57 / sqrt(2): no overflow up to n = 96 terms.
+struct fxacc {
+    uint64_t hh, cr;
+};
+__device__ __forceinline__ void fx_mac(fxacc &a, fx x, fx y) {
+    a.hh += mul_wide(x.hi, y.hi);
+    a.cr += mul_wide(x.hi, y.lo);
+    a.cr += mul_wide(x.lo, y.hi);
+}
+// the sum divided by 2^DOWN, 32 < DOWN <= 64
+template <int DOWN>
+__device__ __forceinline__ int64_t fx_down(fxacc a) {
+    return (int64_t)((a.hh << (64 - DOWN)) + (uint64_t)((int64_t)a.cr >> (DOWN - 32)));
+}
+template <int DOWN>
+__device__ __forceinline__ int64_t fx_mul(fx x, fx y) {
+    fxacc a{0, (uint64_t)1 << (DOWN - 33)};
+    fx_mac(a, x, y);
+    return fx_down<DOWN>(a);
+}
+
+// x 2^sh rounded to an integer (|x| 2^sh < 2^62), by shifts of the significand
+__device__ __forceinline__ int64_t fx_of(double x, int sh) {
+    const uint64_t b = (uint64_t)__double_as_longlong(x);
+    const int e = (int)((b >> 52) & 0x7ff);
+    if (e == 0) return 0;
+    const uint64_t m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+    const int p = e - 1075 + sh;
+    const uint64_t v = p >= 0 ? m << (p & 15) : (p < -54 ? 0 : (m + ((uint64_t)1 << (-p - 1))) >> -p);
+    return (b >> 63) ? -(int64_t)v : (int64_t)v;
+}
+__device__ __forceinline__ double fx_scale2(double x, int e) {  // x 2^e, |e| <= 2000, in two exact steps
+    const int a = e / 2, c = e - a;
+    return x * __longlong_as_double((long long)(1023 + a) << 52) * __longlong_as_double((long long)(1023 + c) << 52);
+}
+__device__ __forceinline__ int fx_clz(uint64_t v) {
+    const uint32_t h = (uint32_t)(v >> 32);
+    return h ? __clz(h) : 32 + __clz((uint32_t)v);
+}
+// sums that wrap instead of overflowing: unused lanes carry arbitrary words
+__device__ __forceinline__ int64_t fx_add(int64_t a, int64_t b) { return (int64_t)((uint64_t)a + (uint64_t)b); }
+__device__ __forceinline__ int64_t fx_sub(int64_t a, int64_t b) { return (int64_t)((uint64_t)a - (uint64_t)b); }
+__device__ __forceinline__ int64_t fx_shfl(int64_t v, int src) { return __shfl_sync(FULL, v, src); }
+__device__ __forceinline__ fx fx_shfl(fx v, int src) {
+    return {__shfl_sync(FULL, v.hi, src), __shfl_sync(FULL, v.lo, src)};
+}
+
+// Reciprocal square root of a pivot d 2^-58: 1/sqrt(d) = rm 2^-61 2^(sh - 3), Newton's
+// third-order step on rsqrtf of the leading bits (within 2^-20.5, so the neglected term
+// is below 2^-63).  lim: 1.9 sqrt(d) in units of 2^-26, the high word of 2^-58.
+struct FxPivot {
+    fx rm;
+    int sh, lim;
+};
+__device__ __forceinline__ FxPivot fx_pivot(int64_t d) {
+    const int s = fx_clz((uint64_t)d) & ~1;  // even: the root's exponent is an integer
+    const uint64_t dp = (uint64_t)d << s;    // d = x 2^(6 - s), x = dp 2^-64 in [1/4, 1)
+    const uint32_t dh = (uint32_t)(dp >> 32), dl = (uint32_t)dp;
+    const float xf = (float)dh * 2.3283064365386963e-10f;
+    const float r0 = rsqrtf(xf);
+    const uint32_t R = (uint32_t)(r0 * 536870912.0f);  // 2^29
+    const uint64_t P = (uint64_t)R * R;
+    const uint32_t ph = (uint32_t)(P >> 32), pl = (uint32_t)P;
+    const uint64_t m = (uint64_t)dh * ph + (((uint64_t)dh * pl) >> 32) + (((uint64_t)dl * ph) >> 32);
+    const int64_t e = (int64_t)(((uint64_t)1 << 58) - m);  // 1 - x r0^2
+    const int e32 = (int)(e >> 7);
+    const int64_t corr = (e >> 1) + ((3 * (int64_t)(mul_wide(e32, e32) >> 44)) >> 3);
+    const int64_t rm = ((int64_t)R << 32) + ((int64_t)mul_wide((int)R, (int)(corr >> 16)) >> 10) +
+                       ((int64_t)mul_wide((int)R, (int)(corr & 0xffff)) >> 26);
+    FxPivot p;
+    p.rm = fx_split(rm);
+    p.sh = s >> 1;
+    p.lim = (int)(1.9f * xf * r0 * __uint_as_float((unsigned)(127 + 29 - p.sh) << 23)) + 1;
+    return p;
+}
+// v / sqrt(d): v is shifted up first, so the product keeps every bit
+__device__ __forceinline__ int64_t fx_over(int64_t v, const FxPivot &p) {
+    return fx_mul<64>(fx_split((int64_t)((uint64_t)v << p.sh)), p.rm);
+}
+__device__ __forceinline__ bool fx_beyond(int64_t v, int lim) {
+    const int h = (int)(v >> 32);
+    return (h < 0 ? ~h : h) > lim;
+}
+
+// Bordered Cholesky in fixed point, panels of four columns: the sums over earlier
+// columns of a row and four columns share the row's load (one 16-byte load per lane and
+// four broadcast ones per four complex multiply-adds; column by column the shared-memory
+// pipe would be the limit), lanes are dealt to rows, or s lanes to a row once few rows
+// are left, as in the floating-point forms; the panel's own columns follow in registers,
+// pivot rows passed by shuffles.  Only entries below the diagonal are written (the
+// diagonal is not read again).  Matrix rows beyond 1.9 (not a factor of a positive
+// matrix) end it: false, the caller's FP64 path decides.  The last bordered row holds the
+// data, scaled by its caller below 2^-6; its solve has no bound, and where an entry
+// passes 1/2 the row is shifted down by 6 bits (counted in ey) and the panel's slot redone.
+template <int N, int NB, class E>
+__device__ __forceinline__ bool factor_fixed(E *mat, int lane, int &ey) {
+    constexpr bool CPLX = std::is_same<E, fxc>::value;
+    constexpr int NROW = N + NB, PW = 4;
+    static_assert(N % PW == 0, "whole panels");
+    int grown = 0;
+    for (int j0 = 0; j0 < N; j0 += PW) {
+        const int nrows = NROW - j0;
+        const int cl2 = 32 - __clz(nrows - 1);
+        const int ls = cl2 < 5 ? 5 - cl2 : 0;
+        const int s = 1 << ls, g = 32 >> ls;
+        const int part = lane & (s - 1), grp = lane >> ls;
+        FxPivot piv[PW];
+        for (int base = j0; base < NROW; base += g) {
+            const bool first = base == j0;
+            const int r = base + grp;
+            const bool act = r < NROW, data = r == NROW - 1;
+            const E *Lr = mat + tri<N>(act ? r : j0, 0);
+            for (;;) {
+                int64_t vr[PW], vi[PW];
+                {
+                    fxacc ar[PW], ai[PW];
+#pragma unroll
+                    for (int c = 0; c < PW; ++c) ar[c] = ai[c] = fxacc{0, (uint64_t)1 << 25};
+                    const E *Lj = mat + tri<N>(j0, 0);
+#pragma unroll 1
+                    for (int k = part; k < j0; k += s) {
+                        const E a = Lr[k];
+                        if constexpr (CPLX) {
+                            const fx na = fx_neg(a.re);
+#pragma unroll
+                            for (int c = 0; c < PW; ++c) {  // row j0 + c starts c j0 + c(c+1)/2 after row j0
+                                const E b = Lj[c * j0 + c * (c + 1) / 2 + k];
+                                fx_mac(ar[c], a.re, b.re);
+                                fx_mac(ai[c], a.im, b.re);
+                                fx_mac(ar[c], a.im, b.im);
+                                fx_mac(ai[c], na, b.im);
+                            }
+                        } else {
+#pragma unroll
+                            for (int c = 0; c < PW; ++c) fx_mac(ar[c], a, Lj[c * j0 + c * (c + 1) / 2 + k]);
+                        }
+                    }
+#pragma unroll
+                    for (int c = 0; c < PW; ++c) {
+                        vr[c] = fx_down<FXB>(ar[c]);
+                        vi[c] = CPLX ? fx_down<FXB>(ai[c]) : 0;
+                    }
+                }
+                for (int o = 1; o < s; o <<= 1) {
+#pragma unroll
+                    for (int c = 0; c < PW; ++c) {
+                        vr[c] = fx_add(vr[c], __shfl_xor_sync(FULL, vr[c], o));
+                        if constexpr (CPLX) vi[c] = fx_add(vi[c], __shfl_xor_sync(FULL, vi[c], o));
+                    }
+                }
+                // (in a diagonal block the entries above the diagonal are read and carried along unused)
+#pragma unroll
+                for (int c = 0; c < PW; ++c) {
+                    if constexpr (CPLX) {
+                        vr[c] = fx_sub(fx_val(Lr[j0 + c].re), vr[c]);
+                        vi[c] = fx_sub(fx_val(Lr[j0 + c].im), vi[c]);
+                    } else {
+                        vr[c] = fx_sub(fx_val(Lr[j0 + c]), vr[c]);
+                    }
+                }
+                E l[PW];
+                bool bad = false, high = false;
+#pragma unroll
+                for (int c = 0; c < PW; ++c) {
+                    if (first) {
+                        const int64_t d = fx_shfl(vr[c], c << ls);
+                        if (d < ((int64_t)1 << (FXB - 30)) || d > ((int64_t)1 << (FXB + 1))) return false;
+                        piv[c] = fx_pivot(d);
+                    }
+                    if (act && r > j0 + c) {
+                        const int lim = data ? piv[c].lim >> 2 : piv[c].lim;
+                        const bool big = fx_beyond(vr[c], lim) || (CPLX && fx_beyond(vi[c], lim));
+                        bad |= big && !data;
+                        high |= big && data;
+                    }
+                    if constexpr (CPLX) {
+                        l[c] = E{fx_split(fx_over(vr[c], piv[c])), fx_split(fx_over(vi[c], piv[c]))};
+                    } else {
+                        l[c] = fx_split(fx_over(vr[c], piv[c]));
+                    }
+#pragma unroll
+                    for (int c2 = c + 1; c2 < PW; ++c2) {
+                        E b;
+                        if (first) {  // row j0 + c2 is held by lane c2 << ls
+                            if constexpr (CPLX) b = E{fx_shfl(l[c].re, c2 << ls), fx_shfl(l[c].im, c2 << ls)};
+                            else b = fx_shfl(l[c], c2 << ls);
+                        } else {
+                            b = mat[tri<N>(j0 + c2, j0 + c)];
+                        }
+                        fxacc ar{0, (uint64_t)1 << 25}, ai{0, (uint64_t)1 << 25};
+                        if constexpr (CPLX) {
+                            fx_mac(ar, l[c].re, b.re);
+                            fx_mac(ai, l[c].im, b.re);
+                            fx_mac(ar, l[c].im, b.im);
+                            fx_mac(ai, fx_neg(l[c].re), b.im);
+                            vi[c2] = fx_sub(vi[c2], fx_down<FXB>(ai));
+                        } else {
+                            fx_mac(ar, l[c], b);
+                        }
+                        vr[c2] = fx_sub(vr[c2], fx_down<FXB>(ar));
+                    }
+                }
+                if (__ballot_sync(FULL, bad)) return false;
+                if (__ballot_sync(FULL, high)) {
+                    if (++grown > 10) return false;
+                    ey += 6;
+                    for (int k = lane; k < N; k += 32) {
+                        E *y = mat + tri<N>(NROW - 1, k);
+                        if constexpr (CPLX) {
+                            *y = E{fx_split((fx_val(y->re) + 32) >> 6), fx_split((fx_val(y->im) + 32) >> 6)};
+                        } else {
+                            *y = fx_split((fx_val(*y) + 32) >> 6);
+                        }
+                    }
+                    __syncwarp();
+                    continue;
+                }
+                __syncwarp();  // the slot's entries have been read before they are overwritten
+                if (part == 0 && act) {
+#pragma unroll
+                    for (int c = 0; c < PW; ++c)
+                        if (r > j0 + c) mat[tri<N>(r, j0 + c)] = l[c];
+                }
+                __syncwarp();
+                break;
+            }
+        }
+    }
+    return true;
+}
+
+// Cubic of the xi table at t (in units of t_max 2^-62; the interval count is a power of
+// two, so interval and offset are the bits of t), 2^-58.
+__device__ __forceinline__ int64_t table_eval_fx(const TableDev &tab, int64_t t) {
+    const int lg = 31 - __clz(tab.n);
+    t = t < 0 ? 0 : (t > 0x3fffffffffffffffll ? 0x3fffffffffffffffll : t);
+    const int k = (int)((uint64_t)t >> (62 - lg));
+    const fx s = fx_split((int64_t)(((uint64_t)t << (2 + lg)) >> 2));  // 2^-62
+    const double2 c01 = __ldg(reinterpret_cast<const double2 *>(tab.cfx + k));
+    const double2 c23 = __ldg(reinterpret_cast<const double2 *>(tab.cfx + k) + 1);
+    int64_t v = __double_as_longlong(c23.y);
+    v = __double_as_longlong(c23.x) + fx_mul<62>(s, fx_split(v));
+    v = __double_as_longlong(c01.y) + fx_mul<62>(s, fx_split(v));
+    return __double_as_longlong(c01.x) + fx_mul<62>(s, fx_split(v));
+}
+
+// conj(a) b exp(-iSE) for the triangle (n', X_i, X_j): the pair phase through the target
+// (as holonomy32 and transported_phase), to 2^-55.  q = (u_i v_j - v_i u_j) / (4 r^2) and
+// tt = (t_i + t_j + t_ij) / (4 r^2), both 2^-62; hr = r^2 / 2 (2^-64), r2 = r^2 (2^-62), r^2 <= 2^-5.
+// tan(E/2) = x = r^2 q / (1 - eps), eps = (r^2 / 2) tt <= 2^-5.4; with z = x^2 <= 2^-13.9,
+//   S = 2: exp(-2iE) - 1 = -8z + 8z^2 (2 - 3z + 4z^2) - 4ix (1 - 3z + z^2 (5 - 7z))
+//   S = 1: exp(-iE) - 1 = -2z + 2z^2 (1 - z + z^2) - 2ix (1 - z + z^2 (1 - z)).
+template <int S>
+__device__ __forceinline__ void phase_fx(fxc a, fxc b, int64_t q, int64_t tt, fx hr, fx r2, int64_t &pr, int64_t &pi) {
+    const int64_t eps = fx_mul<62>(fx_split(tt), hr);  // 2^-64
+    // 1 / (1 - eps) = 1 + eps w, w = 1 + eps w2, w2 to 2^-30
+    const int e31 = (int)(eps >> 33);
+    int w2 = 1 << 30;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) w2 = (1 << 30) + (int)((int64_t)mul_wide(e31, w2) >> 31);
+    const fx es = fx_split(eps);
+    const int64_t w = ((int64_t)1 << 62) + (int64_t)mul_wide(es.hi, w2) + ((int64_t)mul_wide(es.lo, w2) >> 32);  // 2^-62
+    const fx ew = fx_split(fx_mul<64>(es, fx_split(w)));                                                         // 2^-62
+    const fx x = fx_split(fx_mul<60>(fx_split(q + fx_mul<62>(fx_split(q), ew)), r2));                             // 2^-64
+    const int64_t xv = fx_val(x);
+    const int64_t z = fx_mul<64>(x, x);          // 2^-64
+    const int z44 = (int)(z >> 20);              // 2^-44
+    const int zz = (int)((int64_t)mul_wide(z44, z44) >> 30);  // z^2, 2^-58
+    int64_t u, dr, di;
+    if constexpr (S == 1) {
+        const int t1 = (1 << 28) - (z44 >> 16), t3 = t1 + (zz >> 30);
+        u = z - ((int64_t)mul_wide(zz, t1) >> 22);
+        dr = -(z + z) + ((int64_t)mul_wide(zz, t3) >> 21);
+    } else {
+        const int t1 = (5 << 28) - 7 * (z44 >> 16), t3 = (2 << 28) - 3 * (z44 >> 16) + (zz >> 28);
+        u = 3 * z - ((int64_t)mul_wide(zz, t1) >> 22);
+        dr = -8 * z + ((int64_t)mul_wide(zz, t3) >> 19);
+    }
+    di = xv - fx_mul<64>(x, fx_split(u));
+    di *= S == 1 ? -2 : -4;
+    // conj(a) b
+    fxacc cr{0, (uint64_t)1 << 25}, ci{0, (uint64_t)1 << 25};
+    fx_mac(cr, a.re, b.re);
+    fx_mac(ci, a.re, b.im);
+    fx_mac(cr, a.im, b.im);
+    fx_mac(ci, fx_neg(a.im), b.re);
+    const int64_t br = fx_down<FXB>(cr), bi = fx_down<FXB>(ci);
+    const fx bre = fx_split(br), bim = fx_split(bi), fdr = fx_split(dr), fdi = fx_split(di);
+    fxacc er{0, (uint64_t)1 << 31}, ei{0, (uint64_t)1 << 31};
+    fx_mac(er, bre, fdr);
+    fx_mac(ei, bre, fdi);
+    fx_mac(er, fx_neg(bim), fdi);
+    fx_mac(ei, bim, fdr);
+    pr = br + fx_down<64>(er);
+    pi = bi + fx_down<64>(ei);
+}
+
+// The estimate of solve_point<double> (nugget NUGGET_EPS) in fixed point.  Neighbour
+// offsets become integers in units of the disc's diameter (in place: gx, gy, gz, the
+// phases and tangent coordinates; fx_restore gives gx, gy, gz back), chords, table
+// lookups, pair phases, factor and final sums stay integers; FP64 serves the one phase
+// per neighbour.  False (nothing solved): a data value that is not finite, or a matrix
+// that is not safely positive.
+template <int K, int SPIN, class SM>
+__device__ bool solve_point_fixed(SM &sm, const PointA &P, int lane, const LensArgs &a,
+                                  const double (&keyd)[Shape<K>::RPL], const double (&yre)[Shape<K>::RPL],
+                                  const double (&yim)[Shape<K>::RPL], double &val_re, double &val_im,
+                                  double &var_rel) {
+    using E = typename std::conditional<SPIN == 0, fx, fxc>::type;
+    static_assert(offsetof(SM, u) % 16 == 0, "16-byte elements");
+    constexpr int RPL = Shape<K>::RPL, NTRI = Shape<K>::NTRI;
+    E *mat = reinterpret_cast<E *>(&sm.u);
+    auto put = [](double &slot, int64_t v) { slot = __longlong_as_double((long long)v); };
+    auto get = [](const double &slot) { return (int64_t)__double_as_longlong(slot); };
+    auto put_fx = [](double &slot, fx v) {
+        slot = __longlong_as_double((long long)(((uint64_t)(uint32_t)v.hi << 32) | (uint32_t)v.lo));
+    };
+    auto get_fx = [](const double &slot) {
+        const uint64_t b = (uint64_t)__double_as_longlong(slot);
+        return fx{(int)(b >> 32), (int)(uint32_t)b};
+    };
+    // data exponent: the largest |y| of the stencil is scaled into [2^-7, 2^-6)
+    int ymax = 0;
+    int64_t tau[RPL];
+#pragma unroll
+    for (int r = 0; r < RPL; ++r) {
+        const int i = lane + 32 * r;
+        tau[r] = 0;
+        if (i < K) {
+            const int e0 = (int)((uint64_t)__double_as_longlong(yre[r]) >> 52 & 0x7ff);
+            const int e1 = SPIN == 0 ? 0 : (int)((uint64_t)__double_as_longlong(yim[r]) >> 52 & 0x7ff);
+            ymax = e0 > ymax ? e0 : ymax;
+            ymax = e1 > ymax ? e1 : ymax;
+            tau[r] = fx_of(keyd[r] * (a.inv_2r * a.inv_2r), 62);
+            if constexpr (SPIN != 0) {
+                double u, v;
+                const Cx<double> ph = pair_phase_uv<double, SPIN>(sm.gx[i], sm.gy[i], sm.gz[i], P.z, P.s, P.cph, P.sph,
+                                                                  sm.gnz[i], sm.gns[i], sm.gnc[i], sm.gnsn[i], u, v);
+                put_fx(sm.p0r[i], fx_split(fx_of(ph.re, FXB)));
+                put_fx(sm.p0i[i], fx_split(fx_of(ph.im, FXB)));
+                put_fx(sm.pu[i], fx_split(fx_of(u * a.inv_2r, 60)));
+                put_fx(sm.pv[i], fx_split(fx_of(v * a.inv_2r, 60)));
+                sm.tau[i] = tau[r];
+            }
+            put(sm.gx[i], fx_of(sm.gx[i] * a.inv_2r, 60));
+            put(sm.gy[i], fx_of(sm.gy[i] * a.inv_2r, 60));
+            put(sm.gz[i], fx_of(sm.gz[i] * a.inv_2r, 60));
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const int v = __shfl_xor_sync(FULL, ymax, o);
+        ymax = v > ymax ? v : ymax;
+    }
+    __syncwarp();
+    if (ymax == 0x7ff) return false;
+    int ey = ymax - 1022 + 6;  // |y| < 2^(ey - 6)
+
+    const fx hr = fx_split(fx_of(0.5 * a.r2, 64)), r2 = fx_split(fx_of(a.r2, 62));
+    constexpr int64_t DIAG = (int64_t)((1.0 + NUGGET_EPS) * 288230376151711744.0);  // 2^58
+    {
+        int i = 0, j = lane;
+        while (j > i) {
+            j -= i + 1;
+            ++i;
+        }
+        for (int q = lane; q < NTRI; q += 32) {
+            E e;
+            if (i == j) {
+                if constexpr (SPIN == 0) e = fx_split(DIAG);
+                else e = E{fx_split(DIAG), fx{0, 0}};
+            } else {
+                fxacc t{0, (uint64_t)1 << 24};
+                const fx dx = fx_split(get(sm.gx[j]) - get(sm.gx[i]));
+                const fx dy = fx_split(get(sm.gy[j]) - get(sm.gy[i]));
+                const fx dz = fx_split(get(sm.gz[j]) - get(sm.gz[i]));
+                t.hh += mul_wide(dx.hi, dx.hi);
+                t.cr += mul_wide(dx.hi, dx.lo);
+                t.hh += mul_wide(dy.hi, dy.hi);
+                t.cr += mul_wide(dy.hi, dy.lo);
+                t.hh += mul_wide(dz.hi, dz.hi);
+                t.cr += mul_wide(dz.hi, dz.lo);  // 2 hi lo, the factor 2 in the shift
+                const int64_t tij = (int64_t)((t.hh << 6) + (uint64_t)((int64_t)t.cr >> 25));  // 2^-62
+                const int64_t f = table_eval_fx(a.tab, tij);
+                if constexpr (SPIN == 0) {
+                    e = fx_split(f);
+                } else {
+                    const fx ui = get_fx(sm.pu[i]), vi = get_fx(sm.pv[i]), uj = get_fx(sm.pu[j]), vj = get_fx(sm.pv[j]);
+                    fxacc c{0, (uint64_t)1 << 25};
+                    fx_mac(c, ui, vj);
+                    fx_mac(c, fx_neg(vi), uj);
+                    int64_t pr, pi;
+                    phase_fx<SPIN == 1 ? 1 : 2>(fxc{get_fx(sm.p0r[i]), get_fx(sm.p0i[i])},
+                                                fxc{get_fx(sm.p0r[j]), get_fx(sm.p0i[j])}, fx_down<58>(c),
+                                                sm.tau[i] + sm.tau[j] + tij, hr, r2, pr, pi);
+                    const fx fs = fx_split(f);
+                    e = E{fx_split(fx_mul<FXB>(fs, fx_split(pr))), fx_split(fx_mul<FXB>(fs, fx_split(pi)))};
+                }
+            }
+            mat[q] = e;
+            j += 32;
+            while (j > i) {
+                j -= i + 1;
+                ++i;
+            }
+        }
+    }
+    // bordered rows: K = c (spin 1, 2: <P(n') P_i^*>), K + 1 = conj(y)
+#pragma unroll
+    for (int r = 0; r < RPL; ++r) {
+        const int i = lane + 32 * r;
+        if (i < K) {
+            const fx f = fx_split(table_eval_fx(a.tab, tau[r]));
+            if constexpr (SPIN == 0) {
+                mat[tri<K>(K, i)] = f;
+                mat[tri<K>(K + 1, i)] = fx_split(fx_of(yre[r], FXB - ey));
+            } else {
+                mat[tri<K>(K, i)] = E{fx_split(fx_mul<FXB>(f, get_fx(sm.p0r[i]))), fx_split(fx_mul<FXB>(f, get_fx(sm.p0i[i])))};
+                mat[tri<K>(K + 1, i)] = E{fx_split(fx_of(yre[r], FXB - ey)), fx_split(-fx_of(yim[r], FXB - ey))};
+            }
+        }
+    }
+    __syncwarp();
+    if (!factor_fixed<K, 2>(mat, lane, ey)) return false;
+
+    fxacc sr{0, (uint64_t)1 << 25}, si{0, (uint64_t)1 << 25}, sn{0, (uint64_t)1 << 25};
+#pragma unroll
+    for (int r = 0; r < RPL; ++r) {
+        const int k = lane + 32 * r;
+        if (k < K) {
+            const E c = mat[tri<K>(K, k)], y = mat[tri<K>(K + 1, k)];
+            if constexpr (SPIN == 0) {
+                fx_mac(sr, c, y);
+                fx_mac(sn, c, c);
+            } else {  // (cr + i ci)(yr - i yi)
+                fx_mac(sr, c.re, y.re);
+                fx_mac(sr, c.im, y.im);
+                fx_mac(si, c.im, y.re);
+                fx_mac(si, fx_neg(c.re), y.im);
+                fx_mac(sn, c.re, c.re);
+                fx_mac(sn, c.im, c.im);
+            }
+        }
+    }
+    int64_t v = fx_down<FXB>(sr), w = fx_down<FXB>(si), n = fx_down<FXB>(sn);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        v += __shfl_xor_sync(FULL, v, o);
+        if constexpr (SPIN != 0) w += __shfl_xor_sync(FULL, w, o);
+        n += __shfl_xor_sync(FULL, n, o);
+    }
+    val_re = fx_scale2((double)v, ey - FXB);
+    val_im = SPIN == 0 ? 0.0 : fx_scale2((double)w, ey - FXB);
+    var_rel = (double)(((int64_t)1 << FXB) - n) * 3.469446951953614e-18;  // 2^-58
+    return true;
+}
+
+// The FP64 offsets back from solve_point_fixed's integers (its phases are recomputed by solve_point).
+template <int K, class SM>
+__device__ __forceinline__ void fx_restore(SM &sm, int lane, double two_r) {
+    for (int i = lane; i < K; i += 32) {
+        const double q = two_r * 8.673617379884035e-19;  // 2^-60
+        sm.gx[i] = (double)__double_as_longlong(sm.gx[i]) * q;
+        sm.gy[i] = (double)__double_as_longlong(sm.gy[i]) * q;
+        sm.gz[i] = (double)__double_as_longlong(sm.gz[i]) * q;
+    }
+    __syncwarp();
+}
+
+// Assembly, factor and solves of one point in precision R; false when a pivot of
+// S + nugget I is not positive.
 //
 // Factorisation: left-looking Cholesky of the matrix bordered by the two
 // right-hand-side rows (row K holds c (spin 2: c0 = <P(n') P_i^*>), row K+1
@@ -1497,6 +2008,13 @@ __device__ __forceinline__ void process_tile(const LensArgs &a, int R_rings, int
                         sm.gnsn[i] = g[6];
                     }
                     __syncwarp();
+                }
+            }
+            if constexpr (!MIXED && SPIN != SPIN2_AUG) {
+                if (a.tab.cfx) {
+                    solved = solve_point_fixed<K, SPIN>(sm, P, lane, a, keyd, yre, yim, vre, vim, vrel);
+                    __syncwarp();
+                    if (!solved) fx_restore<K>(sm, lane, a.two_r);
                 }
             }
             double nug = NUGGET_EPS;

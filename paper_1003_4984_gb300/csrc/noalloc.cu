@@ -39,6 +39,10 @@ constexpr size_t OFF_GM = OFF_FM + al(sizeof(double) * (NA_MAX_INTERVALS + 1));
 constexpr size_t OFF_C64 = OFF_GM + al(sizeof(double) * (NA_MAX_INTERVALS + 1));
 constexpr size_t OFF_C32 = OFF_C64 + al(sizeof(Coef64) * NA_MAX_INTERVALS);
 constexpr size_t OFF_CNT = OFF_C32 + al(sizeof(float4) * 2 * NA_MAX_INTERVALS);
+// the fixed-point table replaces the spectrum and the nodes once the interval
+// coefficients have been formed from them
+constexpr size_t OFF_CFX = OFF_CL;
+static_assert(OFF_CFX + sizeof(CoefFx) * NA_MAX_INTERVALS <= OFF_C64, "the fixed-point table fits what it replaces");
 constexpr size_t OFF_QUEUE = OFF_CNT + al(sizeof(unsigned long long) * CNT_N);
 constexpr size_t SCRATCH_BYTES = OFF_QUEUE + al(sizeof(unsigned long long));
 
@@ -155,6 +159,12 @@ extern "C" int flints_lens_noalloc(int64_t nside, int lmax, const double *cl, co
         return na_fail(FLINTS_EINVAL, "flints_lens_noalloc: xi(0) = %g is not positive", xi0);
     NA_CK(finish_table(d_f, d_g, n, tg.h, xi0, d_c64, d_c32, st), "table coefficients");
 
+    CoefFx *d_cfx = nullptr;
+    if (precision == FLINTS_FP64 && fixed_table_ok(tg, spin, lmax, cl, spin == 2 ? cl_bb : nullptr, xi0)) {
+        d_cfx = reinterpret_cast<CoefFx *>(base + OFF_CFX);
+        NA_CK(launch_fixed_table(d_c64, n, d_cfx, st), "fixed-point table");
+    }
+
     LensArgs a{};
     a.nside = nside;
     a.first = first;
@@ -172,8 +182,11 @@ extern "C" int flints_lens_noalloc(int64_t nside, int lmax, const double *cl, co
     a.tab.inv_h_hi = (float)a.tab.inv_h;
     a.tab.inv_h_lo = (float)(a.tab.inv_h - (double)a.tab.inv_h_hi);
     a.tab.n = n;
+    a.tab.cfx = d_cfx;
     a.xi0 = xi0;
     a.r2 = tg.r2;
+    a.two_r = 2.0 * tg.r;
+    a.inv_2r = 0.5 / tg.r;
     a.counters = d_cnt;
     a.queue = d_queue;
     NA_CK(launch_lens(spin, K, precision, a, R_rings, LaunchCfg{0, 0, 0}, st), "lens kernel launch");

@@ -131,6 +131,15 @@ __global__ void normalise_kernel(double *f, double *g, int n, double xi0) {
     g[k] /= xi0;
 }
 
+// The interval coefficients rounded to units of 2^-58 (all of them below 2 in size, see fixed_table_ok).
+__global__ void fixed_table_kernel(const Coef64 *__restrict__ c64, int n, CoefFx *__restrict__ cfx) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    const double u = 288230376151711744.0;  // 2^58
+    const Coef64 c = c64[k];
+    cfx[k] = CoefFx{(int64_t)(c.f * u), (int64_t)(c.m * u), (int64_t)(c.c2 * u), (int64_t)(c.c3 * u)};
+}
+
 cudaError_t launch_xi_table(int spin, int lmax, const double *cl_dev, const double *clbb_dev, double t_max,
                             int n, double *f_out, double *g_out, double *fm_out, double *gm_out,
                             cudaStream_t st) {
@@ -152,6 +161,12 @@ cudaError_t finish_table(double *f, double *g, int n, double h, double xi0, Coef
         if (e != cudaSuccess) return e;
     }
     normalise_kernel<<<(n + 1 + threads - 1) / threads, threads, 0, st>>>(f, g, n, xi0);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fixed_table(const Coef64 *c64, int n, CoefFx *cfx, cudaStream_t st) {
+    const int threads = 128;
+    fixed_table_kernel<<<(n + threads - 1) / threads, threads, 0, st>>>(c64, n, cfx);
     return cudaGetLastError();
 }
 
