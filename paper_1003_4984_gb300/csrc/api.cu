@@ -146,16 +146,6 @@ TableGrid table_grid(int64_t nside, int K, int lmax, const double *cl, const dou
     g.R_rings = (int)std::ceil(1.5 * g.r * (double)nside) + 1;
     return g;
 }
-bool fixed_table_ok(const TableGrid &g, int spin, int lmax, const double *cl, const double *cl_bb, double xi0) {
-    double x0 = 0.0, x1 = 0.0;
-    for (int l = 0; l <= lmax; ++l) {
-        const double a = (2.0 * l + 1.0) / (4.0 * PI) * (std::fabs(cl[l]) + (cl_bb ? std::fabs(cl_bb[l]) : 0.0));
-        x0 += a;
-        x1 += a * (double)l * (l + 1.0) / 4.0;
-    }
-    // c2 = 3D - 2 m0 - m1 and c3 = m0 + m1 - 2D, |D|, |m| <= h max|xi'|
-    return x0 <= 1.9 * xi0 && 6.0 * g.h * x1 <= 1.9 * xi0 && (spin == 0 || g.r2 <= 0.03125);
-}
 }  // namespace flints
 
 static void free_plan_memory(flints_plan_s *p) {

@@ -359,7 +359,7 @@ struct alignas(32) Coef64 {
     double f, m, c2, c3;
 };
 
-// The same coefficients as integers, units of 2^-58 (the fixed-point solve).
+// The same coefficients as integers, units of 2^-59 (the fixed-point solve).
 struct alignas(32) CoefFx {
     int64_t f, m, c2, c3;
 };

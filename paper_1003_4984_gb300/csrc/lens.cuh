@@ -771,15 +771,15 @@ __device__ __forceinline__ bool factor_bordered(Elem *mat, int lane) {
 // SM per warp instruction, its integer multiply-add IMAD.WIDE (32 x 32 + 64 bits) half
 // a cycle (measured: 1.9 against 58 lanes per cycle and SM), and every quantity of the
 // solve is bounded: entries of S + n I, of its factor and of L^-1 c by 1, squared
-// chords by the search disc.  A number is (hi 2^32 + lo) 2^-58 with a signed low word,
+// chords by the search disc.  A number is (hi 2^32 + lo) 2^-59 with a signed low word,
 // so a multiply-add is three IMAD.WIDE into two 64-bit sums (hi hi, and the two cross
-// products together; lo lo, below 2^-54 of a unit in the last place's square, is
-// dropped) with no rounding until the sum is used: absolute error 2^-57 per sum, where
-// FP64 rounds every term of these sums, which are near 1, to 2^-53.
+// products together).  The low words' product is dropped: at most 2^-56 a term and
+// without bias, 2^-58 rms, where FP64 rounds every term of these sums, which are near 1,
+// to 2^-54; where a word meets itself (pivots, the variance) its mean is put back.
 // Measured (GB300): 1,048,583 spin-0 targets (K = 32, Nside 2048) 52.4 -> 27.8 ms; 524,309
 // Q/U targets (K = 32, Nside 4096) 61.2 -> 26.9 ms.
 // Returns false when a pivot of S + nugget I is not positive.
-constexpr int FXB = 58;
+constexpr int FXB = 59;
 
 struct alignas(8) fx {
     int hi, lo;
@@ -799,9 +799,9 @@ __device__ __forceinline__ fx fx_split(int64_t v) {
 __device__ __forceinline__ fx fx_neg(fx a) { return {(int)(0u - (unsigned)a.hi), (int)(0u - (unsigned)a.lo)}; }
 __device__ __forceinline__ uint64_t mul_wide(int a, int b) { return (uint64_t)((int64_t)a * (int64_t)b); }
 
-// Sum of products hh 2^64 + cr 2^32.  With operands of at most 2^58 (the factor's rows,
-// |L_r| <= 1) the cross sum of n terms stays below sqrt(n) 2^58; the data row, kept below
-// 1/2 per entry, adds at most n 2^57 / sqrt(2): no overflow up to n = 96 terms.
+// Sum of products hh 2^64 + cr 2^32.  With rows of at most unit length (the factor's,
+// |L_r| <= 1) the cross sum of n terms stays below 2 sqrt(n) 2^58, with the data row, kept
+// below 1/8 per entry, below 2.3 sqrt(n) 2^58: no overflow up to n = 96 terms.
 struct fxacc {
     uint64_t hh, cr;
 };
@@ -809,6 +809,10 @@ __device__ __forceinline__ void fx_mac(fxacc &a, fx x, fx y) {
     a.hh += mul_wide(x.hi, y.hi);
     a.cr += mul_wide(x.hi, y.lo);
     a.cr += mul_wide(x.lo, y.hi);
+}
+__device__ __forceinline__ void fx_sqr(fxacc &a, fx x) {  // + x^2, all of it
+    fx_mac(a, x, x);
+    a.cr += mul_wide(x.lo, x.lo) >> 32;
 }
 // the sum divided by 2^DOWN, 32 < DOWN <= 64
 template <int DOWN>
@@ -848,16 +852,16 @@ __device__ __forceinline__ fx fx_shfl(fx v, int src) {
     return {__shfl_sync(FULL, v.hi, src), __shfl_sync(FULL, v.lo, src)};
 }
 
-// Reciprocal square root of a pivot d 2^-58: 1/sqrt(d) = rm 2^-61 2^(sh - 3), Newton's
+// Reciprocal square root of a pivot d 2^-59: 1/sqrt(d) = rm 2^-61 2^(sh - 1), Newton's
 // third-order step on rsqrtf of the leading bits (within 2^-20.5, so the neglected term
-// is below 2^-63).  lim: 1.9 sqrt(d) in units of 2^-26, the high word of 2^-58.
+// is below 2^-63).  lim: 1.9 sqrt(d) in units of 2^-27, the high word of 2^-59.
 struct FxPivot {
     fx rm;
     int sh, lim;
 };
 __device__ __forceinline__ FxPivot fx_pivot(int64_t d) {
-    const int s = fx_clz((uint64_t)d) & ~1;  // even: the root's exponent is an integer
-    const uint64_t dp = (uint64_t)d << s;    // d = x 2^(6 - s), x = dp 2^-64 in [1/4, 1)
+    const int s = (fx_clz((uint64_t)d) - 1) | 1;  // odd: the root's exponent is an integer
+    const uint64_t dp = (uint64_t)d << s;         // d = x 2^(5 - s), x = dp 2^-64 in [1/4, 1)
     const uint32_t dh = (uint32_t)(dp >> 32), dl = (uint32_t)dp;
     const float xf = (float)dh * 2.3283064365386963e-10f;
     const float r0 = rsqrtf(xf);
@@ -872,13 +876,13 @@ __device__ __forceinline__ FxPivot fx_pivot(int64_t d) {
                        ((int64_t)mul_wide((int)R, (int)(corr & 0xffff)) >> 26);
     FxPivot p;
     p.rm = fx_split(rm);
-    p.sh = s >> 1;
-    p.lim = (int)(1.9f * xf * r0 * __uint_as_float((unsigned)(127 + 29 - p.sh) << 23)) + 1;
+    p.sh = (s - 3) >> 1;
+    p.lim = (int)(1.9f * xf * r0 * __uint_as_float((unsigned)(127 + 28 - p.sh) << 23)) + 1;
     return p;
 }
 // v / sqrt(d): v is shifted up first, so the product keeps every bit
 __device__ __forceinline__ int64_t fx_over(int64_t v, const FxPivot &p) {
-    return fx_mul<64>(fx_split((int64_t)((uint64_t)v << p.sh)), p.rm);
+    return fx_mul<62>(fx_split((int64_t)((uint64_t)v << p.sh)), p.rm);
 }
 __device__ __forceinline__ bool fx_beyond(int64_t v, int lim) {
     const int h = (int)(v >> 32);
@@ -893,8 +897,8 @@ __device__ __forceinline__ bool fx_beyond(int64_t v, int lim) {
 // pivot rows passed by shuffles.  Only entries below the diagonal are written (the
 // diagonal is not read again).  Matrix rows beyond 1.9 (not a factor of a positive
 // matrix) end it: false, the caller's FP64 path decides.  The last bordered row holds the
-// data, scaled by its caller below 2^-6; its solve has no bound, and where an entry
-// passes 1/2 the row is shifted down by 6 bits (counted in ey) and the panel's slot redone.
+// data, scaled by its caller below 2^-8; its solve has no bound, and where an entry
+// passes 1/8 the row is shifted down by 6 bits (counted in ey) and the panel's slot redone.
 template <int N, int NB, class E>
 __device__ __forceinline__ bool factor_fixed(E *mat, int lane, int &ey) {
     constexpr bool CPLX = std::is_same<E, fxc>::value;
@@ -918,7 +922,7 @@ __device__ __forceinline__ bool factor_fixed(E *mat, int lane, int &ey) {
                 {
                     fxacc ar[PW], ai[PW];
 #pragma unroll
-                    for (int c = 0; c < PW; ++c) ar[c] = ai[c] = fxacc{0, (uint64_t)1 << 25};
+                    for (int c = 0; c < PW; ++c) ar[c] = ai[c] = fxacc{0, (uint64_t)1 << (FXB - 33)};
                     const E *Lj = mat + tri<N>(j0, 0);
 #pragma unroll 1
                     for (int k = part; k < j0; k += s) {
@@ -966,12 +970,13 @@ __device__ __forceinline__ bool factor_fixed(E *mat, int lane, int &ey) {
 #pragma unroll
                 for (int c = 0; c < PW; ++c) {
                     if (first) {
-                        const int64_t d = fx_shfl(vr[c], c << ls);
+                        // 8/3 units: the mean square of the dropped low words, one per real term
+                        const int64_t d = fx_shfl(vr[c], c << ls) - (8 * (j0 + c) * (CPLX ? 2 : 1)) / 3;
                         if (d < ((int64_t)1 << (FXB - 30)) || d > ((int64_t)1 << (FXB + 1))) return false;
                         piv[c] = fx_pivot(d);
                     }
                     if (act && r > j0 + c) {
-                        const int lim = data ? piv[c].lim >> 2 : piv[c].lim;
+                        const int lim = data ? piv[c].lim >> 4 : piv[c].lim;
                         const bool big = fx_beyond(vr[c], lim) || (CPLX && fx_beyond(vi[c], lim));
                         bad |= big && !data;
                         high |= big && data;
@@ -990,7 +995,7 @@ __device__ __forceinline__ bool factor_fixed(E *mat, int lane, int &ey) {
                         } else {
                             b = mat[tri<N>(j0 + c2, j0 + c)];
                         }
-                        fxacc ar{0, (uint64_t)1 << 25}, ai{0, (uint64_t)1 << 25};
+                        fxacc ar{0, (uint64_t)1 << (FXB - 33)}, ai{0, (uint64_t)1 << (FXB - 33)};
                         if constexpr (CPLX) {
                             fx_mac(ar, l[c].re, b.re);
                             fx_mac(ai, l[c].im, b.re);
@@ -1033,7 +1038,7 @@ __device__ __forceinline__ bool factor_fixed(E *mat, int lane, int &ey) {
 }
 
 // Cubic of the xi table at t (in units of t_max 2^-62; the interval count is a power of
-// two, so interval and offset are the bits of t), 2^-58.
+// two, so interval and offset are the bits of t), 2^-59.
 __device__ __forceinline__ int64_t table_eval_fx(const TableDev &tab, int64_t t) {
     const int lg = 31 - __clz(tab.n);
     t = t < 0 ? 0 : (t > 0x3fffffffffffffffll ? 0x3fffffffffffffffll : t);
@@ -1047,6 +1052,18 @@ __device__ __forceinline__ int64_t table_eval_fx(const TableDev &tab, int64_t t)
     return __double_as_longlong(c01.x) + fx_mul<62>(s, fx_split(v));
 }
 
+// 1 / (1 - eps) - 1 in units of 2^-62, to 2^-55 for eps (2^-64) <= 2^-5.4: eps w with
+// w = 1 + eps w2 and w2 = 1 + eps + .. + eps^5 to 2^-30.
+__device__ __forceinline__ fx fx_recip1m(int64_t eps) {
+    const int e31 = (int)(eps >> 33);
+    int w2 = 1 << 30;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) w2 = (1 << 30) + (int)((int64_t)mul_wide(e31, w2) >> 31);
+    const fx es = fx_split(eps);
+    const int64_t w = ((int64_t)1 << 62) + (int64_t)mul_wide(es.hi, w2) + ((int64_t)mul_wide(es.lo, w2) >> 32);  // 2^-62
+    return fx_split(fx_mul<64>(es, fx_split(w)));
+}
+
 // conj(a) b exp(-iSE) for the triangle (n', X_i, X_j): the pair phase through the target
 // (as holonomy32 and transported_phase), to 2^-55.  q = (u_i v_j - v_i u_j) / (4 r^2) and
 // tt = (t_i + t_j + t_ij) / (4 r^2), both 2^-62; hr = r^2 / 2 (2^-64), r2 = r^2 (2^-62), r^2 <= 2^-5.
@@ -1055,15 +1072,7 @@ __device__ __forceinline__ int64_t table_eval_fx(const TableDev &tab, int64_t t)
 //   S = 1: exp(-iE) - 1 = -2z + 2z^2 (1 - z + z^2) - 2ix (1 - z + z^2 (1 - z)).
 template <int S>
 __device__ __forceinline__ void phase_fx(fxc a, fxc b, int64_t q, int64_t tt, fx hr, fx r2, int64_t &pr, int64_t &pi) {
-    const int64_t eps = fx_mul<62>(fx_split(tt), hr);  // 2^-64
-    // 1 / (1 - eps) = 1 + eps w, w = 1 + eps w2, w2 to 2^-30
-    const int e31 = (int)(eps >> 33);
-    int w2 = 1 << 30;
-#pragma unroll
-    for (int i = 0; i < 5; ++i) w2 = (1 << 30) + (int)((int64_t)mul_wide(e31, w2) >> 31);
-    const fx es = fx_split(eps);
-    const int64_t w = ((int64_t)1 << 62) + (int64_t)mul_wide(es.hi, w2) + ((int64_t)mul_wide(es.lo, w2) >> 32);  // 2^-62
-    const fx ew = fx_split(fx_mul<64>(es, fx_split(w)));                                                         // 2^-62
+    const fx ew = fx_recip1m(fx_mul<62>(fx_split(tt), hr));  // 1 / (1 - eps) = 1 + ew
     const fx x = fx_split(fx_mul<60>(fx_split(q + fx_mul<62>(fx_split(q), ew)), r2));                             // 2^-64
     const int64_t xv = fx_val(x);
     const int64_t z = fx_mul<64>(x, x);          // 2^-64
@@ -1082,7 +1091,7 @@ __device__ __forceinline__ void phase_fx(fxc a, fxc b, int64_t q, int64_t tt, fx
     di = xv - fx_mul<64>(x, fx_split(u));
     di *= S == 1 ? -2 : -4;
     // conj(a) b
-    fxacc cr{0, (uint64_t)1 << 25}, ci{0, (uint64_t)1 << 25};
+    fxacc cr{0, (uint64_t)1 << (FXB - 33)}, ci{0, (uint64_t)1 << (FXB - 33)};
     fx_mac(cr, a.re, b.re);
     fx_mac(ci, a.re, b.im);
     fx_mac(cr, a.im, b.im);
@@ -1122,7 +1131,7 @@ __device__ bool solve_point_fixed(SM &sm, const PointA &P, int lane, const LensA
         const uint64_t b = (uint64_t)__double_as_longlong(slot);
         return fx{(int)(b >> 32), (int)(uint32_t)b};
     };
-    // data exponent: the largest |y| of the stencil is scaled into [2^-7, 2^-6)
+    // data exponent: the largest |y| of the stencil is scaled into [2^-9, 2^-8)
     int ymax = 0;
     int64_t tau[RPL];
 #pragma unroll
@@ -1157,10 +1166,10 @@ __device__ bool solve_point_fixed(SM &sm, const PointA &P, int lane, const LensA
     }
     __syncwarp();
     if (ymax == 0x7ff) return false;
-    int ey = ymax - 1022 + 6;  // |y| < 2^(ey - 6)
+    int ey = ymax - 1022 + 8;  // |y| < 2^(ey - 8)
 
     const fx hr = fx_split(fx_of(0.5 * a.r2, 64)), r2 = fx_split(fx_of(a.r2, 62));
-    constexpr int64_t DIAG = (int64_t)((1.0 + NUGGET_EPS) * 288230376151711744.0);  // 2^58
+    constexpr int64_t DIAG = (int64_t)((1.0 + NUGGET_EPS) * 576460752303423488.0);  // 2^59
     {
         int i = 0, j = lane;
         while (j > i) {
@@ -1189,7 +1198,7 @@ __device__ bool solve_point_fixed(SM &sm, const PointA &P, int lane, const LensA
                     e = fx_split(f);
                 } else {
                     const fx ui = get_fx(sm.pu[i]), vi = get_fx(sm.pv[i]), uj = get_fx(sm.pu[j]), vj = get_fx(sm.pv[j]);
-                    fxacc c{0, (uint64_t)1 << 25};
+                    fxacc c{0, (uint64_t)1 << (FXB - 33)};
                     fx_mac(c, ui, vj);
                     fx_mac(c, fx_neg(vi), uj);
                     int64_t pr, pi;
@@ -1226,7 +1235,7 @@ __device__ bool solve_point_fixed(SM &sm, const PointA &P, int lane, const LensA
     __syncwarp();
     if (!factor_fixed<K, 2>(mat, lane, ey)) return false;
 
-    fxacc sr{0, (uint64_t)1 << 25}, si{0, (uint64_t)1 << 25}, sn{0, (uint64_t)1 << 25};
+    fxacc sr{0, (uint64_t)1 << (FXB - 33)}, si{0, (uint64_t)1 << (FXB - 33)}, sn{0, (uint64_t)1 << (FXB - 33)};
 #pragma unroll
     for (int r = 0; r < RPL; ++r) {
         const int k = lane + 32 * r;
@@ -1234,14 +1243,14 @@ __device__ bool solve_point_fixed(SM &sm, const PointA &P, int lane, const LensA
             const E c = mat[tri<K>(K, k)], y = mat[tri<K>(K + 1, k)];
             if constexpr (SPIN == 0) {
                 fx_mac(sr, c, y);
-                fx_mac(sn, c, c);
+                fx_sqr(sn, c);
             } else {  // (cr + i ci)(yr - i yi)
                 fx_mac(sr, c.re, y.re);
                 fx_mac(sr, c.im, y.im);
                 fx_mac(si, c.im, y.re);
                 fx_mac(si, fx_neg(c.re), y.im);
-                fx_mac(sn, c.re, c.re);
-                fx_mac(sn, c.im, c.im);
+                fx_sqr(sn, c.re);
+                fx_sqr(sn, c.im);
             }
         }
     }
@@ -1254,7 +1263,7 @@ __device__ bool solve_point_fixed(SM &sm, const PointA &P, int lane, const LensA
     }
     val_re = fx_scale2((double)v, ey - FXB);
     val_im = SPIN == 0 ? 0.0 : fx_scale2((double)w, ey - FXB);
-    var_rel = (double)(((int64_t)1 << FXB) - n) * 3.469446951953614e-18;  // 2^-58
+    var_rel = (double)(((int64_t)1 << FXB) - n) * 1.734723475976807e-18;  // 2^-59
     return true;
 }
 

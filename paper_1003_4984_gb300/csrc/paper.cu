@@ -39,6 +39,7 @@ namespace flints {
 namespace paper {
 
 constexpr int SINV_THREADS = 64;
+constexpr int ROW_EXP_MIN = -6, ROW_EXP_MAX = 24;  // what the fixed-point kernel takes: 2^24 is above 1/sqrt(n)
 
 // offset of column j of a K x K lower-triangular matrix packed by columns
 __host__ __device__ constexpr int col_start(int K, int j) { return j * K - j * (j - 1) / 2; }
@@ -155,6 +156,17 @@ __global__ void stencil_kernel(int64_t Nc, int k, int K, int32_t *members, int32
     slot[c] = (int32_t)slot_of(Nc, i, j);
 }
 
+__device__ __forceinline__ int expo_of(double x) {
+    return (int)(((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ff);
+}
+
+// the exponent stored for a row whose largest biased exponent is ex: |entry| < 2^(ex - 1022)
+// (rows of L^-1 lie between 1/sqrt(1 + n) and 1/sqrt(n) in size; 0 for absent rows)
+__device__ __forceinline__ int8_t row_exponent(int ex) {
+    const int e = ex == 0 ? 0 : ex - 1022;
+    return (int8_t)(e < ROW_EXP_MIN ? ROW_EXP_MIN : e);
+}
+
 struct LinvArgs {
     int64_t Nc, N, nslot;
     int K;
@@ -162,6 +174,7 @@ struct LinvArgs {
     TableDev tab;
     double *linv;                  // [nslot][K (K + 1) / 2], L^-1 packed by columns
     int *slot_steps;               // [nslot]: nugget doublings, -1 = no factor found
+    int8_t *row_exp;               // [nslot][K]: the entries of a row are below 2^row_exp in size (NULL: not wanted)
     unsigned long long *max_t;     // bits of the largest member-pair chord^2
     int *counts;                   // [0]: slots with a raised nugget, [1]: failed slots
 };
@@ -247,6 +260,13 @@ __global__ void __launch_bounds__(SINV_THREADS) linv_kernel(LinvArgs a) {
                 const bool v = lanestep_entry(e, i, j);
                 dst[e] = (ok && v && i < n && j < n) ? Li[i * LDS + j] : 0.0;
             }
+            if (a.row_exp)
+                for (int i = tid; i < K; i += nt) {
+                    int ex = 0;
+                    if (ok && i < n)
+                        for (int j = 0; j <= i; ++j) ex = max(ex, expo_of(Li[i * LDS + j]));
+                    a.row_exp[sl * K + i] = row_exponent(ex);
+                }
         } else {
             for (int j = 0; j < K; ++j) {
                 for (int i = j + tid; i < K; i += nt)
@@ -399,6 +419,13 @@ __global__ void __launch_bounds__(SINV_THREADS) linv_kernel_c(LinvArgs a, double
                 const bool in = ok && v && i < n && j < n;
                 dst[e] = make_double2(in ? Lr[i * LDS + j] : 0.0, in ? Lim[i * LDS + j] : 0.0);
             }
+            if (a.row_exp)
+                for (int i = tid; i < K; i += nt) {
+                    int ex = 0;
+                    if (ok && i < n)
+                        for (int j = 0; j <= i; ++j) ex = max(ex, max(expo_of(Lr[i * LDS + j]), expo_of(Lim[i * LDS + j])));
+                    a.row_exp[sl * K + i] = row_exponent(ex);
+                }
         } else {
             for (int j = 0; j < K; ++j) {
                 for (int i = j + tid; i < K; i += nt) {
@@ -429,6 +456,7 @@ struct ApplyArgs {
     const float4 *pvf;             // [12 N^2][2]: double-float (x, y), (z, 0) (mixed plans)
     const float2 *linvf;           // double-float L^-1 blocks (mixed plans)
     const int *slot_steps;
+    const int8_t *row_exp;
     TableDev tab;
     TableDev tabm;                 // augmented plans: xi-/xi+(0) on the same grid
     double xi0;
@@ -1229,6 +1257,415 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32) apply_kernel_aug(ApplyArgs a
     }
 }
 
+// ------------------------------------------- y = 2 apply in fixed point (FP64 plans)
+// The per-target work of an FP64 plan at K = 36 on the integer pipe, in the pairs of
+// lens.cuh (three IMAD.WIDE per multiply-add; the FP64 kernels were 91 %
+// FP64-pipe bound).  Offsets from the target are formed in
+// FP64 (exact differences) and become integers; chords, correlation lookup, phases and the triangular products are
+// integer sums.  L^-1 blocks stay FP64 in memory and are shifted to integers as they are
+// loaded, in units of 2^(e - 57) with 2^e the power of two above the row's largest entry
+// (row_exp): 2^-3 of the rounding of that entry's products in FP64, and the cross sums of a
+// row's 72 products stay below 2^63.
+// z_y = L^-1 y has no bound of its own: its two 64-bit sums are kept and shifted by what
+// the largest row of the target needs.
+// Member terms are formed for FX_G = 8 targets at a time, flattened over the lanes (288
+// terms, nine full passes; member by member a target needs two, the second with four
+// lanes).  Measured (GB300, 2,097,169 Q/U targets, Nside 1024): 40.5 -> 15.2 ms.
+constexpr int FX_G = 8, FX_K = 36, FXA = 58;  // FXA: units of c, y and their products, 2^-58
+
+constexpr int FX_FP64 = 1 << 20;
+
+template <int S>
+struct FxApplyWarp {
+    using E = typename std::conditional<S == 0, fx, fxc>::type;
+    using Y = typename std::conditional<S == 0, double, double2>::type;
+    E x[FX_G * FX_K];      // conj(c)
+    Y y[FX_G * FX_K];      // data, FP64 until the target's turn, then integers in the same place
+    double tx[32], ty[32], tz[32];  // target position
+    fx fz[S ? 32 : 1], fs[S ? 32 : 1], fc[S ? 32 : 1], fn[S ? 32 : 1];  // its frame: z, sin(theta), cos and sin(phi)
+    int64_t cp[32];        // coarse pixel
+    int64_t vr[32], vi[32], q[32];
+    int ve[32];            // exponent of the value; FX_FP64: the three words are FP64 bits
+    int32_t sl[32];
+    int win[32];
+};
+
+// lane-step position of entry (row, col) of a K = 36 block (the inverse of lanestep_entry)
+__device__ __forceinline__ int lanestep_index(int row, int col) {
+    if (row >= 32) return (LS_STEPS + (col >> 3)) * 32 + ((row - 32) | ((col & 7) << 2));
+    const int p = row < 16 ? row : 31 - row, t = row < 16 ? col : p + 1 + col;
+    return t < LS_STEPS ? t * 32 + 2 * p : (t - LS_STEPS) * 32 + 2 * p + 1;
+}
+
+// a double below 2^e in size in units of 2^(e - 57), truncated with the lowest bit set (which
+// leaves no bias); flip: the sign bit is inverted
+__device__ __forceinline__ fx fx_entry(double v, int e, unsigned flip) {
+    const uint64_t b = (uint64_t)__double_as_longlong(v);
+    const uint32_t h = (uint32_t)(b >> 32);
+    const int r = e + 1022 - (int)((h >> 20) & 0x7ffu);  // >= 0
+    const uint64_t m = (((uint64_t)((h & 0xfffffu) | 0x100000u) << 32) | (uint32_t)b) << 4;
+    const uint64_t a = (m >> (r < 63 ? r : 63)) | 1;
+    const int64_t neg = (int64_t)(int)(h ^ flip) >> 63;
+    return fx_split((int64_t)((a ^ (uint64_t)neg) - (uint64_t)neg));
+}
+
+// Sum of products of L^-1 entries with the low words' products kept: entries grow to
+// 2^row_exp and cancel, so what fx_mac drops would be some three times the FP64 kernel's
+// rounding.  The top 13 bits of both low words are enough (2^-12 of what they replace),
+// 72 products of them stay below 2^31.
+struct fxacc3 {
+    uint64_t hh, cr;
+    int ll;
+};
+__device__ __forceinline__ void fx_mac3(fxacc3 &a, fx x, int xl, fx y, int yl) {
+    a.hh += mul_wide(x.hi, y.hi);
+    a.cr += mul_wide(x.hi, y.lo);
+    a.cr += mul_wide(x.lo, y.hi);
+    a.ll += xl * yl;
+}
+__device__ __forceinline__ fxacc fx_fold(fxacc3 a) { return {a.hh, a.cr + (uint64_t)((int64_t)a.ll * 64)}; }
+
+// FP64 form of one target (rows per lane): data that is not finite, classes with a raised nugget
+template <int S>
+__device__ __attribute__((noinline)) void target_fp64(const double *linv, bool mir, const FxApplyWarp<S> &sm, int g, int lane,
+                                         double &vr, double &vi, double &qc) {
+    const double u = 3.469446951953614e-18;  // 2^-58
+    vr = vi = qc = 0.0;
+    for (int row = lane; row < FX_K; row += 32) {
+        double zc0 = 0.0, zc1 = 0.0, zy0 = 0.0, zy1 = 0.0;
+        for (int j = 0; j <= row; ++j) {
+            const int at = lanestep_index(row, j);
+            if constexpr (S == 0) {
+                const double e = linv[at];
+                zc0 = fma(e, (double)fx_val(sm.x[g * FX_K + j]) * u, zc0);
+                zy0 = fma(e, sm.y[g * FX_K + j], zy0);
+            } else {
+                const double2 e = reinterpret_cast<const double2 *>(linv)[at];
+                const double ei = mir ? -e.y : e.y;
+                const double xr = (double)fx_val(sm.x[g * FX_K + j].re) * u, xi = (double)fx_val(sm.x[g * FX_K + j].im) * u;
+                const double2 y = sm.y[g * FX_K + j];
+                zc0 += e.x * xr - ei * xi;
+                zc1 += e.x * xi + ei * xr;
+                zy0 += e.x * y.x - ei * y.y;
+                zy1 += e.x * y.y + ei * y.x;
+            }
+        }
+        vr += zc0 * zy0 + zc1 * zy1;
+        vi += zc0 * zy1 - zc1 * zy0;
+        qc += zc0 * zc0 + zc1 * zc1;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        vr += __shfl_xor_sync(FULL, vr, o);
+        vi += __shfl_xor_sync(FULL, vi, o);
+        qc += __shfl_xor_sync(FULL, qc, o);
+    }
+}
+
+struct FxChord {
+    int k;        // chords are shifted up by k bits: t_max 4^k in (1/4, 1]
+    fx scale;     // 1 / (t_max 4^k), 2^-60
+};
+
+template <int S>
+__global__ void __launch_bounds__(APPLY_WARPS * 32, 4) apply_kernel_fx(ApplyArgs a, FxChord ch) {
+    extern __shared__ __align__(16) unsigned char fx_smem[];
+    using W = FxApplyWarp<S>;
+    using E = typename W::E;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    W &sm = reinterpret_cast<W *>(fx_smem)[wid];
+    const int64_t ntiles = (a.count + 31) / 32;
+    const int64_t mirror_from = 6 * a.Nc * a.Nc + 2 * a.Nc;  // first pixel of coarse ring 2 Nc + 1
+    unsigned long long n_win = 0, n_nug = 0, n_fail = 0;
+    for (int64_t tile = (int64_t)blockIdx.x * APPLY_WARPS + wid; tile < ntiles;
+         tile += (int64_t)gridDim.x * APPLY_WARPS) {
+        {
+            double x = 0.0, y = 0.0, z = 1.0;
+            int64_t c = 0;
+            target_of(a, tile * 32 + lane, x, y, z, c);
+            if (!(z == z)) {  // not finite: NaN outputs whatever is computed (finish_point)
+                x = y = 0.0;
+                z = 1.0;
+            }
+            sm.cp[lane] = c;
+            sm.tx[lane] = x;
+            sm.ty[lane] = y;
+            sm.tz[lane] = z;
+            if constexpr (S != 0) {
+                const double sn = sqrt(x * x + y * y);
+                sm.fz[lane] = fx_split(fx_of(z, FXB));
+                sm.fs[lane] = fx_split(fx_of(sn, FXB));
+                sm.fc[lane] = fx_split(fx_of(sn > 1e-12 ? x / sn : 1.0, FXB));
+                sm.fn[lane] = fx_split(fx_of(sn > 1e-12 ? y / sn : 0.0, FXB));
+            }
+            sm.sl[lane] = __ldg(a.slot + c);
+            sm.win[lane] = 0;
+        }
+        __syncwarp();
+        const int npt = a.count - tile * 32 < 32 ? (int)(a.count - tile * 32) : 32;
+        for (int q0 = 0; q0 < npt; q0 += FX_G) {
+            // ---- member terms of targets q0 .. q0 + 7
+#pragma unroll 1
+            for (int it = lane; it < FX_G * FX_K; it += 32) {
+                const int g = it / FX_K, q = q0 + g;
+                E xc{};
+                typename W::Y yv{};
+                const int64_t c = sm.cp[q];
+                const int32_t m = q < npt ? __ldg(a.members + c * FX_K + (it - g * FX_K)) : -1;
+                if (m >= 0) {
+                    const double2 p0 = __ldg(a.pv + 2 * (int64_t)m), p1 = __ldg(a.pv + 2 * (int64_t)m + 1);
+                    double dx, dy;  // as the FP64 kernels form them (spin 1, 2: the product is not rounded)
+                    if constexpr (S == 0) {  // (x, y), (z, 0)
+                        dx = p0.x - sm.tx[q];
+                        dy = p0.y - sm.ty[q];
+                        yv = __ldg(a.map + m);
+                    } else {  // (cos, sin phi), (z, s)
+                        dx = fma(p1.y, p0.x, -sm.tx[q]);
+                        dy = fma(p1.y, p0.y, -sm.ty[q]);
+                        yv = __ldg(reinterpret_cast<const double2 *>(a.map) + m);
+                    }
+                    const fx ex = fx_split(fx_of(dx, 60 + ch.k)), ey = fx_split(fx_of(dy, 60 + ch.k));
+                    const fx ez = fx_split(fx_of(p1.x - sm.tz[q], 60 + ch.k));
+                    fxacc t2{0, (uint64_t)1 << 24};
+                    t2.hh += mul_wide(ex.hi, ex.hi);
+                    t2.cr += mul_wide(ex.hi, ex.lo);
+                    t2.hh += mul_wide(ey.hi, ey.hi);
+                    t2.cr += mul_wide(ey.hi, ey.lo);
+                    t2.hh += mul_wide(ez.hi, ez.hi);
+                    t2.cr += mul_wide(ez.hi, ez.lo);
+                    const int64_t tk = (int64_t)((t2.hh << 6) + (uint64_t)((int64_t)t2.cr >> 25));  // 4^k chord^2, 2^-62
+                    const int64_t tau = fx_mul<60>(fx_split(tk), ch.scale);                          // of t_max, 2^-62
+                    if (tau > ((int64_t)1 << 62)) atomicAdd(&sm.win[q], 1);
+                    const int64_t f = table_eval_fx(a.tab, tau);
+                    if constexpr (S == 0) {
+                        xc = fx_split(f >> (FXB - FXA));
+                    } else {
+                        // phase of the transport between the two frames: with D = phi_m - phi_t,
+                        // (1 + cos b) exp(i psi) = cos D (1 + z z') + s s' + i (z + z') sin D and
+                        // 1 + cos b = 2 (1 - t/4)
+                        const fx mc = fx_split(fx_of(p0.x, FXB)), mn = fx_split(fx_of(p0.y, FXB));
+                        const fx mz = fx_split(fx_of(p1.x, FXB)), ms = fx_split(fx_of(p1.y, FXB));
+                        const fx tc = sm.fc[q], tn = sm.fn[q], tz = sm.fz[q];
+                        fxacc cd{0, (uint64_t)1 << (FXB - 33)}, sd{0, (uint64_t)1 << (FXB - 33)};
+                        fx_mac(cd, tc, mc);
+                        fx_mac(cd, tn, mn);
+                        fx_mac(sd, tc, mn);
+                        fx_mac(sd, fx_neg(tn), mc);
+                        const fx h = fx_split(((int64_t)1 << (FXB - 1)) + fx_mul<FXB + 1>(tz, mz));
+                        const fx hz = fx_split((fx_val(tz) + fx_val(mz)) >> 1);
+                        const int64_t pr = fx_mul<FXB>(fx_split(fx_down<FXB>(cd)), h) + fx_mul<FXB + 1>(sm.fs[q], ms);
+                        const int64_t pi = fx_mul<FXB>(fx_split(fx_down<FXB>(sd)), hz);
+                        fx er = fx_split(pr), ei = fx_split(pi);
+                        int64_t ur, ui, eps;  // before the division by 1 - eps (2^-64)
+                        if constexpr (S == 2) {
+                            // the square over the squared size, which takes out the frames' own
+                            // rounding (it would scale all of c)
+                            const int64_t rr = fx_mul<FXB>(er, er), ii = fx_mul<FXB>(ei, ei);
+                            ur = rr - ii;
+                            ui = fx_mul<FXB - 1>(er, ei);
+                            eps = (((int64_t)1 << FXB) - rr - ii) * 32;
+                        } else {
+                            ur = pr;
+                            ui = pi;
+                            eps = tk >> (2 * ch.k);
+                        }
+                        const fx ew = fx_recip1m(eps);
+                        er = fx_split(ur + fx_mul<62>(fx_split(ur), ew));
+                        ei = fx_split(ui + fx_mul<62>(fx_split(ui), ew));
+                        const fx fs = fx_split(f);
+                        xc = E{fx_split(fx_mul<2 * FXB - FXA>(fs, er)), fx_split(fx_mul<2 * FXB - FXA>(fs, fx_neg(ei)))};
+                    }
+                }
+                sm.x[it] = xc;
+                sm.y[it] = yv;
+            }
+            __syncwarp();
+            // ---- triangular products and sums, target by target
+            for (int g = 0; g < FX_G && q0 + g < npt; ++g) {
+                const int q = q0 + g;
+                const int32_t sl = sm.sl[q];
+                const bool mir = S != 0 && sm.cp[q] >= mirror_from;  // conj(L^-1)
+                const unsigned flip = mir ? 0x80000000u : 0u;
+                const int pp = lane >> 1, odd = lane & 1;
+                const int8_t *re = a.row_exp + (int64_t)sl * FX_K;
+                const int ep = __ldg(re + pp), eq = __ldg(re + 31 - pp), et = __ldg(re + 32 + (lane & 3));
+                // data to integers: the largest of the target into [2^-3, 2^-2)
+                typename W::Y y0 = sm.y[g * FX_K + lane], y1{};
+                if (lane < FX_K - 32) y1 = sm.y[g * FX_K + 32 + lane];
+                auto expo = [](double v) { return (int)((uint64_t)__double_as_longlong(v) >> 52 & 0x7ff); };
+                int ymax;
+                if constexpr (S == 0) {
+                    ymax = max(expo(y0), expo(y1));
+                } else {
+                    ymax = max(max(expo(y0.x), expo(y0.y)), max(expo(y1.x), expo(y1.y)));
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) ymax = max(ymax, __shfl_xor_sync(FULL, ymax, o));
+                if (ymax == 0x7ff || __ldg(a.slot_steps + sl) != 0) {  // warp-uniform
+                    double vr, vi, qc;
+                    target_fp64<S>(a.linv + (int64_t)sl * linv_len(FX_K) * (S ? 2 : 1), mir, sm, g, lane, vr, vi, qc);
+                    if (lane == 0) {
+                        sm.vr[q] = __double_as_longlong(vr);
+                        sm.vi[q] = __double_as_longlong(vi);
+                        sm.q[q] = __double_as_longlong(qc);
+                        sm.ve[q] = FX_FP64;
+                    }
+                    continue;
+                }
+                const int ey = ymax - 1022 + 2;  // |y| < 2^(ey - 2)
+                fx *yf = reinterpret_cast<fx *>(sm.y);
+                __syncwarp();
+                if constexpr (S == 0) {
+                    yf[g * FX_K + lane] = fx_split(fx_of(y0, FXA - ey));
+                    if (lane < FX_K - 32) yf[g * FX_K + 32 + lane] = fx_split(fx_of(y1, FXA - ey));
+                } else {
+                    reinterpret_cast<fxc *>(yf)[g * FX_K + lane] =
+                        fxc{fx_split(fx_of(y0.x, FXA - ey)), fx_split(fx_of(y0.y, FXA - ey))};
+                    if (lane < FX_K - 32)
+                        reinterpret_cast<fxc *>(yf)[g * FX_K + 32 + lane] =
+                            fxc{fx_split(fx_of(y1.x, FXA - ey)), fx_split(fx_of(y1.y, FXA - ey))};
+                }
+                __syncwarp();
+                const E *X = sm.x + g * FX_K, *Y = reinterpret_cast<const E *>(yf) + g * FX_K;
+                // sums of L^-1 conj(c) and L^-1 y, real and imaginary parts
+                constexpr int NC = S == 0 ? 2 : 4;
+                fxacc3 z[NC], zp[NC], zt[NC];
+#pragma unroll
+                for (int i = 0; i < NC; ++i) z[i] = zp[i] = zt[i] = fxacc3{0, 0, 0};
+                auto mac = [&](fxacc3(&s)[NC], int at, int j, int e) {
+                    if constexpr (S == 0) {
+                        const fx l = fx_entry(__ldg(a.linv + (int64_t)sl * linv_len(FX_K) + at), e, 0u);
+                        const int ll = l.lo >> 19;
+                        fx_mac3(s[0], l, ll, X[j], X[j].lo >> 19);
+                        fx_mac3(s[1], l, ll, Y[j], Y[j].lo >> 19);
+                    } else {
+                        const double2 l = __ldg(reinterpret_cast<const double2 *>(a.linv) + (int64_t)sl * linv_len(FX_K) + at);
+                        const fx lr = fx_entry(l.x, e, 0u), li = fx_entry(l.y, e, flip), nl = fx_neg(li);
+                        const int rl = lr.lo >> 19, il = li.lo >> 19;
+                        const E x = X[j], y = Y[j];
+                        const int x0 = x.re.lo >> 19, x1 = x.im.lo >> 19, y0 = y.re.lo >> 19, y1 = y.im.lo >> 19;
+                        fx_mac3(s[0], lr, rl, x.re, x0);
+                        fx_mac3(s[1], lr, rl, x.im, x1);
+                        fx_mac3(s[2], lr, rl, y.re, y0);
+                        fx_mac3(s[3], lr, rl, y.im, y1);
+                        fx_mac3(s[0], nl, -il, x.im, x1);
+                        fx_mac3(s[1], li, il, x.re, x0);
+                        fx_mac3(s[2], nl, -il, y.im, y1);
+                        fx_mac3(s[3], li, il, y.re, y0);
+                    }
+                };
+                // rows p and 31 - p on lanes 2p and 2p + 1 (the lane-step layout): lane 2p notes its
+                // sums after column p of row p and goes on into row 31 - p
+#pragma unroll 1
+                for (int u = 0; u < LS_STEPS; ++u) {
+                    const int t = odd ? LS_STEPS + u : u;
+                    const int j = t <= pp ? t : t - pp - 1;
+                    mac(z, u * 32 + lane, j < FX_K ? j : FX_K - 1, t <= pp ? ep : eq);  // (the zero pad)
+                    if (!odd && u == pp) {
+#pragma unroll
+                        for (int i = 0; i < NC; ++i) zp[i] = z[i];
+                    }
+                }
+#pragma unroll 1
+                for (int t = 0; t < LS_TAIL; ++t) {  // rows 32 .. 35: zero entries past the diagonal
+                    const int j = (lane >> 2) + 8 * t;
+                    mac(zt, (LS_STEPS + t) * 32 + lane, j < FX_K ? j : FX_K - 1, et);
+                }
+                fxacc f0[NC], f1[NC], f2[NC];  // row p, this lane's part of row 31 - p, of row 32 + (lane & 3)
+#pragma unroll
+                for (int i = 0; i < NC; ++i) {
+                    f0[i] = fx_fold(zp[i]);
+                    f1[i] = fx_fold(z[i]);
+                    f2[i] = fx_fold(zt[i]);
+                    f1[i].hh -= f0[i].hh;  // (zero on odd lanes)
+                    f1[i].cr -= f0[i].cr;
+                }
+                // shift of z_y: by the bits its largest partial sum takes, rows on their own units
+                int top = 0;
+#pragma unroll
+                for (int i = NC / 2; i < NC; ++i) {
+                    auto bits = [](fxacc s) {
+                        const int64_t h = (int64_t)(s.hh + (uint64_t)((int64_t)s.cr >> 32));
+                        return 64 - fx_clz((uint64_t)(h ^ (h >> 63)) | 1);
+                    };
+                    top = max(max(top, bits(f0[i]) + ep), max(bits(f1[i]) + eq, bits(f2[i]) + et));
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(FULL, top, o));
+                const int D = top + 6 > 33 + ROW_EXP_MAX ? top + 6 : 33 + ROW_EXP_MAX;  // |z_y| < 2^58 units
+                auto down = [](fxacc s, int d) {
+                    if (d > 64) return (int64_t)(s.hh + (uint64_t)((int64_t)s.cr >> 32)) >> (d - 64);
+                    return (int64_t)((s.hh << (64 - d)) + (uint64_t)((int64_t)s.cr >> (d - 32)));
+                };
+                auto shfl_add = [](int64_t v, int o) { return fx_add(v, __shfl_xor_sync(FULL, v, o)); };
+                fx w0[NC], w1[NC], w2[NC];
+#pragma unroll
+                for (int i = 0; i < NC; ++i) {
+                    const int d = i < NC / 2 ? 57 : D;
+                    w0[i] = fx_split(down(f0[i], d - ep));
+                    w1[i] = fx_split(shfl_add(down(f1[i], d - eq), 1));
+                    int64_t t = down(f2[i], d - et);
+#pragma unroll
+                    for (int o = 4; o < 32; o <<= 1) t = shfl_add(t, o);
+                    w2[i] = fx_split(t);
+                }
+                // even lanes count rows p and 31 - p, lanes 0..3 rows 32..35, each once
+                fxacc sr{0, (uint64_t)1 << (FXA - 33)}, si{0, (uint64_t)1 << (FXA - 33)}, sq{0, (uint64_t)1 << (FXA - 33)};
+                auto dots = [&](const fx(&w)[NC]) {
+                    if constexpr (S == 0) {
+                        fx_mac(sr, w[0], w[1]);
+                        fx_sqr(sq, w[0]);
+                    } else {  // conj(z_c) z_y, |z_c|^2
+                        fx_mac(sr, w[0], w[2]);
+                        fx_mac(sr, w[1], w[3]);
+                        fx_mac(si, w[0], w[3]);
+                        fx_mac(si, fx_neg(w[1]), w[2]);
+                        fx_sqr(sq, w[0]);
+                        fx_sqr(sq, w[1]);
+                    }
+                };
+                if (!odd) {
+                    dots(w0);
+                    dots(w1);
+                }
+                if (lane < FX_K - 32) dots(w2);
+                int64_t vr = fx_down<FXA>(sr), vi = fx_down<FXA>(si), vq = fx_down<FXA>(sq);
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    vr = shfl_add(vr, o);
+                    if constexpr (S != 0) vi = shfl_add(vi, o);
+                    vq = shfl_add(vq, o);
+                }
+                if (lane == 0) {
+                    sm.vr[q] = vr;
+                    sm.vi[q] = vi;
+                    sm.q[q] = vq;
+                    sm.ve[q] = D - 115 + ey;  // z_y counts 2^(D - e - (57 - e) - (58 - ey))
+                }
+            }
+            __syncwarp();
+        }
+        if (lane < npt) {
+            const int ve = sm.ve[lane];
+            const bool f64 = ve == FX_FP64;
+            const double vr = f64 ? __longlong_as_double(sm.vr[lane]) : fx_scale2((double)sm.vr[lane], ve);
+            const double vi = f64 ? __longlong_as_double(sm.vi[lane]) : fx_scale2((double)sm.vi[lane], ve);
+            const double qc = f64 ? __longlong_as_double(sm.q[lane]) : (double)sm.q[lane] * 3.469446951953614e-18;
+            const int64_t p = tile * 32 + lane;
+            if constexpr (S == 0) finish_point(a, p, sm.sl[lane], vr, qc, sm.win[lane] != 0, n_win, n_nug, n_fail);
+            else finish_point_s2(a, p, sm.sl[lane], vr, vi, qc, sm.win[lane] != 0, n_win, n_nug, n_fail);
+        }
+        __syncwarp();
+    }
+    const unsigned w_win = __reduce_add_sync(FULL, (unsigned)n_win);
+    const unsigned w_nug = __reduce_add_sync(FULL, (unsigned)n_nug);
+    const unsigned w_fail = __reduce_add_sync(FULL, (unsigned)n_fail);
+    if (lane == 0 && a.counters) {
+        if (w_win) atomicAdd(a.counters + CNT_WINDOW, (unsigned long long)w_win);
+        if (w_nug) atomicAdd(a.counters + CNT_NUGGET, (unsigned long long)w_nug);
+        if (w_fail) atomicAdd(a.counters + CNT_FAILED, (unsigned long long)w_fail);
+    }
+}
+
 // ------------------------------------------------------- mixed precision
 // The same route with the per-target arithmetic in double-float (pairs of FP32,
 // about 2^-44 relative per operation) on the FP32 pipe: member positions from a
@@ -1799,6 +2236,9 @@ struct flints_paper_s {
     double *d_clbb;
     Coef64 *d_cm64;
     float4 *d_cm32;
+    CoefFx *d_cfx;      // FP64 plans at y = 2: the integer table and the exponents of the class
+    int8_t *d_row_exp;  // blocks' rows for the fixed-point kernel, which runs when `fixed`
+    bool fixed;
     unsigned long long *d_counters, *d_maxt;
     int64_t points;
     int64_t device_bytes;  // sum of the plan's device allocations
@@ -1835,6 +2275,8 @@ static void paper_release(flints_paper_s *p) {
     cudaFree(p->d_clbb);
     cudaFree(p->d_cm64);
     cudaFree(p->d_cm32);
+    cudaFree(p->d_cfx);
+    cudaFree(p->d_row_exp);
     cudaFree(p->d_pvf);
     cudaFree(p->d_linvf);
     cudaFree(p->d_counters);
@@ -1857,6 +2299,21 @@ static int table_intervals(const double *cl, const double *cl_bb, int lmax, doub
     const double h = std::pow(384.0 * 1e-11 / b4, 0.25);
     const double want = std::ceil(std::log2(t_max / h));
     return want > 16 ? 65536 : (want < 6 ? 64 : (1 << (int)want));
+}
+
+template <int S>
+static cudaError_t launch_fx(const ApplyArgs &a, double t_max, unsigned grid, cudaStream_t st) {
+    FxChord ch;
+    ch.k = (int)std::floor(-0.5 * std::log2(t_max));  // t_max 4^k in (1/4, 1]
+    ch.k = ch.k < 0 ? 0 : ch.k;
+    const int64_t c = (int64_t)std::llround(std::ldexp(1.0 / std::ldexp(t_max, 2 * ch.k), 60)) | 1;
+    ch.scale.lo = (int)(uint32_t)c;
+    ch.scale.hi = (int)((c - ch.scale.lo) / 4294967296);
+    const size_t smem = APPLY_WARPS * sizeof(FxApplyWarp<S>);
+    const cudaError_t e = cudaFuncSetAttribute(apply_kernel_fx<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    apply_kernel_fx<S><<<grid, APPLY_WARPS * 32, smem, st>>>(a, ch);
+    return cudaGetLastError();
 }
 
 extern "C" {
@@ -1941,6 +2398,10 @@ int flints_paper_plan(flints_paper_t *out, int64_t nside, int lmax, const double
     } else {
         PALLOC(p->d_pv, (size_t)12 * nside * nside * 2 * sizeof(double2));
     }
+    if (precision == FLINTS_FP64 && !aug && p->K == FX_K) {
+        PALLOC(p->d_cfx, (size_t)p->n * sizeof(CoefFx));
+        PALLOC(p->d_row_exp, (size_t)p->nslot * p->K);
+    }
     PALLOC(p->d_counters, CNT_N * sizeof(unsigned long long));
     PALLOC(p->d_maxt, sizeof(unsigned long long));
 #undef PALLOC
@@ -1974,6 +2435,14 @@ int flints_paper_plan(flints_paper_t *out, int64_t nside, int lmax, const double
         return bail(e, "flints_paper_plan: table coefficients");
     if (aug && (e = finish_table(p->d_fm, p->d_gm, p->n, p->h, xi0, p->d_cm64, p->d_cm32, st)) != cudaSuccess)
         return bail(e, "flints_paper_plan: xi- table coefficients");
+    if (p->d_cfx) {
+        TableGrid tg{};
+        tg.h = p->h;
+        tg.r2 = p->t_max / 1.533;  // the phases' series run in t/2 (spin 2), at most 0.0239 like the other solve's
+        p->fixed = p->t_max <= 1.0 && fixed_table_ok(tg, spin, lmax, cl, cl_bb, xi0);  // Nside_c >= 7 (spin 0), 32
+        if (p->fixed && (e = launch_fixed_table(p->d_c64, p->n, p->d_cfx, st)) != cudaSuccess)
+            return bail(e, "flints_paper_plan: table coefficients");
+    }
     if (precision == FLINTS_MIXED && spin != 0)
         pixframe_df_kernel<<<(unsigned)((12 * nside * nside + 255) / 256), 256, 0, st>>>(nside, p->d_pvf);
     else if (precision == FLINTS_MIXED)
@@ -2001,6 +2470,7 @@ int flints_paper_plan(flints_paper_t *out, int64_t nside, int lmax, const double
     sa.tab.n = p->n;
     sa.linv = p->d_linv;
     sa.slot_steps = p->d_steps;
+    sa.row_exp = p->d_row_exp;
     sa.max_t = p->d_maxt;
     sa.counts = p->d_scratch;
     const int64_t grid = p->nslot < 152 * 16 ? p->nslot : 152 * 16;
@@ -2107,6 +2577,7 @@ static int paper_run(flints_paper_t p, int64_t nside_tgt, int64_t first, int64_t
     a.pvf = p->d_pvf;
     a.linvf = p->d_linvf;
     a.slot_steps = p->d_steps;
+    a.row_exp = p->d_row_exp;
     a.tab.c64 = p->d_c64;
     a.tab.c32 = p->d_c32;
     a.tab.t_max = p->t_max;
@@ -2125,7 +2596,13 @@ static int paper_run(flints_paper_t p, int64_t nside_tgt, int64_t first, int64_t
     const unsigned grid = (unsigned)(want < cap ? want : cap);
     cudaStream_t st = (cudaStream_t)stream;
     const bool mixed = p->precision == FLINTS_MIXED;
-    if (p->flags & FLINTS_SPIN2_AUGMENTED) {
+    if (p->fixed) {
+        a.tab.cfx = p->d_cfx;
+        const cudaError_t ef = p->spin == 0 ? launch_fx<0>(a, p->t_max, grid, st)
+                               : p->spin == 1 ? launch_fx<1>(a, p->t_max, grid, st)
+                                              : launch_fx<2>(a, p->t_max, grid, st);
+        if (ef != cudaSuccess) return pcuda(ef, "paper apply kernel launch");
+    } else if (p->flags & FLINTS_SPIN2_AUGMENTED) {
         if (p->K == 9)
             apply_kernel_aug<9><<<grid, APPLY_WARPS * 32, 0, st>>>(a);
         else

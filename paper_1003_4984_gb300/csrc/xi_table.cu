@@ -19,6 +19,8 @@
 //     D_{l+1} = e_l D_l - a_l b_l u d_l,
 // the same cancellation-free form as for spin 0.  x-derivatives follow by
 // differentiating the recurrence; d/dt = -1/2 d/dx.
+#include <cmath>
+
 #include "common.cuh"
 
 namespace flints {
@@ -131,11 +133,11 @@ __global__ void normalise_kernel(double *f, double *g, int n, double xi0) {
     g[k] /= xi0;
 }
 
-// The interval coefficients rounded to units of 2^-58 (all of them below 2 in size, see fixed_table_ok).
+// The interval coefficients in units of 2^-59 (all of them below 2 in size, see fixed_table_ok).
 __global__ void fixed_table_kernel(const Coef64 *__restrict__ c64, int n, CoefFx *__restrict__ cfx) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
-    const double u = 288230376151711744.0;  // 2^58
+    const double u = 576460752303423488.0;  // 2^59
     const Coef64 c = c64[k];
     cfx[k] = CoefFx{(int64_t)(c.f * u), (int64_t)(c.m * u), (int64_t)(c.c2 * u), (int64_t)(c.c3 * u)};
 }
@@ -168,6 +170,17 @@ cudaError_t launch_fixed_table(const Coef64 *c64, int n, CoefFx *cfx, cudaStream
     const int threads = 128;
     fixed_table_kernel<<<(n + threads - 1) / threads, threads, 0, st>>>(c64, n, cfx);
     return cudaGetLastError();
+}
+
+bool fixed_table_ok(const TableGrid &g, int spin, int lmax, const double *cl, const double *cl_bb, double xi0) {
+    double x0 = 0.0, x1 = 0.0;
+    for (int l = 0; l <= lmax; ++l) {
+        const double a = (2.0 * l + 1.0) / (4.0 * PI) * (std::fabs(cl[l]) + (cl_bb ? std::fabs(cl_bb[l]) : 0.0));
+        x0 += a;
+        x1 += a * (double)l * (l + 1.0) / 4.0;
+    }
+    // c2 = 3D - 2 m0 - m1 and c3 = m0 + m1 - 2D, |D|, |m| <= h max|xi'|
+    return x0 <= 1.9 * xi0 && 6.0 * g.h * x1 <= 1.9 * xi0 && (spin == 0 || g.r2 <= 0.03125);
 }
 
 }  // namespace flints
