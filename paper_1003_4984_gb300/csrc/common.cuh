@@ -450,6 +450,84 @@ struct TableGrid {
 };
 TableGrid table_grid(int64_t nside, int K, int lmax, const double *cl, const double *cl_bb);
 
+// ---------------------------------------------------------------------------
+// 64-bit fixed-point numbers as pairs hi 2^32 + lo with a signed low word, in units
+// that each use states; a multiply-add is three IMAD.WIDE (32 x 32 + 64 bits), which
+// run at 58 lanes per cycle and SM here against 1.9 for an FP64 multiply-add.
+// ---------------------------------------------------------------------------
+struct alignas(8) fx {
+    int hi, lo;
+};
+struct alignas(16) fxc {
+    fx re, im;
+};
+__device__ __forceinline__ int64_t fx_val(fx a) {
+    return (int64_t)(((uint64_t)(uint32_t)a.hi << 32) + (uint64_t)(int64_t)a.lo);
+}
+// The pair of v.  The lowest bit is set, so that the low word is never -2^31 and both
+// words can be negated.
+__device__ __forceinline__ fx fx_split(int64_t v) {
+    const uint32_t l = (uint32_t)v | 1u;
+    return {(int)((uint32_t)((uint64_t)v >> 32) + (l >> 31)), (int)l};
+}
+__device__ __forceinline__ fx fx_neg(fx a) { return {(int)(0u - (unsigned)a.hi), (int)(0u - (unsigned)a.lo)}; }
+__device__ __forceinline__ uint64_t mul_wide(int a, int b) { return (uint64_t)((int64_t)a * (int64_t)b); }
+// s + a b in one instruction
+__device__ __forceinline__ void mad_wide(uint64_t &s, int a, int b) {
+#ifdef __CUDA_ARCH__
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(s) : "r"(a), "r"(b));
+#else
+    s += mul_wide(a, b);
+#endif
+}
+
+// Sum of products hh 2^64 + cr 2^32; the low words' product is dropped.
+struct fxacc {
+    uint64_t hh, cr;
+};
+__device__ __forceinline__ void fx_mac(fxacc &a, fx x, fx y) {
+    mad_wide(a.hh, x.hi, y.hi);
+    mad_wide(a.cr, x.hi, y.lo);
+    mad_wide(a.cr, x.lo, y.hi);
+}
+__device__ __forceinline__ void fx_sqr(fxacc &a, fx x) {  // + x^2, all of it
+    fx_mac(a, x, x);
+    a.cr += mul_wide(x.lo, x.lo) >> 32;
+}
+// the sum divided by 2^DOWN, 32 < DOWN <= 64
+template <int DOWN>
+__device__ __forceinline__ int64_t fx_down(fxacc a) {
+    return (int64_t)((a.hh << (64 - DOWN)) + (uint64_t)((int64_t)a.cr >> (DOWN - 32)));
+}
+template <int DOWN>
+__device__ __forceinline__ int64_t fx_mul(fx x, fx y) {
+    fxacc a{0, (uint64_t)1 << (DOWN - 33)};
+    fx_mac(a, x, y);
+    return fx_down<DOWN>(a);
+}
+
+// x 2^sh rounded to an integer (|x| 2^sh < 2^62), by shifts of the significand
+__device__ __forceinline__ int64_t fx_of(double x, int sh) {
+    const uint64_t b = (uint64_t)__double_as_longlong(x);
+    const int e = (int)((b >> 52) & 0x7ff);
+    if (e == 0) return 0;
+    const uint64_t m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
+    const int p = e - 1075 + sh;
+    const uint64_t v = p >= 0 ? m << (p & 15) : (p < -54 ? 0 : (m + ((uint64_t)1 << (-p - 1))) >> -p);
+    return (b >> 63) ? -(int64_t)v : (int64_t)v;
+}
+__device__ __forceinline__ double fx_scale2(double x, int e) {  // x 2^e, |e| <= 2000, in two exact steps
+    const int a = e / 2, c = e - a;
+    return x * __longlong_as_double((long long)(1023 + a) << 52) * __longlong_as_double((long long)(1023 + c) << 52);
+}
+__device__ __forceinline__ int fx_clz(uint64_t v) {
+    const uint32_t h = (uint32_t)(v >> 32);
+    return h ? __clz(h) : 32 + __clz((uint32_t)v);
+}
+// sums that wrap instead of overflowing: unused lanes carry arbitrary words
+__device__ __forceinline__ int64_t fx_add(int64_t a, int64_t b) { return (int64_t)((uint64_t)a + (uint64_t)b); }
+__device__ __forceinline__ int64_t fx_sub(int64_t a, int64_t b) { return (int64_t)((uint64_t)a - (uint64_t)b); }
+
 // Host-side launchers (lens_spin0.cu, lens_spin2.cu, xi_table.cu).
 cudaError_t launch_lens(int spin, int K, int precision, const LensArgs &a, int R_rings, const LaunchCfg &cfg,
                         cudaStream_t st);

@@ -781,72 +781,6 @@ __device__ __forceinline__ bool factor_bordered(Elem *mat, int lane) {
 // Returns false when a pivot of S + nugget I is not positive.
 constexpr int FXB = 59;
 
-struct alignas(8) fx {
-    int hi, lo;
-};
-struct alignas(16) fxc {
-    fx re, im;
-};
-__device__ __forceinline__ int64_t fx_val(fx a) {
-    return (int64_t)(((uint64_t)(uint32_t)a.hi << 32) + (uint64_t)(int64_t)a.lo);
-}
-// The pair of v.  The lowest bit is set, so that the low word is never -2^31 and both
-// words can be negated.
-__device__ __forceinline__ fx fx_split(int64_t v) {
-    const uint32_t l = (uint32_t)v | 1u;
-    return {(int)((uint32_t)((uint64_t)v >> 32) + (l >> 31)), (int)l};
-}
-__device__ __forceinline__ fx fx_neg(fx a) { return {(int)(0u - (unsigned)a.hi), (int)(0u - (unsigned)a.lo)}; }
-__device__ __forceinline__ uint64_t mul_wide(int a, int b) { return (uint64_t)((int64_t)a * (int64_t)b); }
-
-// Sum of products hh 2^64 + cr 2^32.  With rows of at most unit length (the factor's,
-// |L_r| <= 1) the cross sum of n terms stays below 2 sqrt(n) 2^58, with the data row, kept
-// below 1/8 per entry, below 2.3 sqrt(n) 2^58: no overflow up to n = 96 terms.
-struct fxacc {
-    uint64_t hh, cr;
-};
-__device__ __forceinline__ void fx_mac(fxacc &a, fx x, fx y) {
-    a.hh += mul_wide(x.hi, y.hi);
-    a.cr += mul_wide(x.hi, y.lo);
-    a.cr += mul_wide(x.lo, y.hi);
-}
-__device__ __forceinline__ void fx_sqr(fxacc &a, fx x) {  // + x^2, all of it
-    fx_mac(a, x, x);
-    a.cr += mul_wide(x.lo, x.lo) >> 32;
-}
-// the sum divided by 2^DOWN, 32 < DOWN <= 64
-template <int DOWN>
-__device__ __forceinline__ int64_t fx_down(fxacc a) {
-    return (int64_t)((a.hh << (64 - DOWN)) + (uint64_t)((int64_t)a.cr >> (DOWN - 32)));
-}
-template <int DOWN>
-__device__ __forceinline__ int64_t fx_mul(fx x, fx y) {
-    fxacc a{0, (uint64_t)1 << (DOWN - 33)};
-    fx_mac(a, x, y);
-    return fx_down<DOWN>(a);
-}
-
-// x 2^sh rounded to an integer (|x| 2^sh < 2^62), by shifts of the significand
-__device__ __forceinline__ int64_t fx_of(double x, int sh) {
-    const uint64_t b = (uint64_t)__double_as_longlong(x);
-    const int e = (int)((b >> 52) & 0x7ff);
-    if (e == 0) return 0;
-    const uint64_t m = (b & 0xfffffffffffffull) | 0x10000000000000ull;
-    const int p = e - 1075 + sh;
-    const uint64_t v = p >= 0 ? m << (p & 15) : (p < -54 ? 0 : (m + ((uint64_t)1 << (-p - 1))) >> -p);
-    return (b >> 63) ? -(int64_t)v : (int64_t)v;
-}
-__device__ __forceinline__ double fx_scale2(double x, int e) {  // x 2^e, |e| <= 2000, in two exact steps
-    const int a = e / 2, c = e - a;
-    return x * __longlong_as_double((long long)(1023 + a) << 52) * __longlong_as_double((long long)(1023 + c) << 52);
-}
-__device__ __forceinline__ int fx_clz(uint64_t v) {
-    const uint32_t h = (uint32_t)(v >> 32);
-    return h ? __clz(h) : 32 + __clz((uint32_t)v);
-}
-// sums that wrap instead of overflowing: unused lanes carry arbitrary words
-__device__ __forceinline__ int64_t fx_add(int64_t a, int64_t b) { return (int64_t)((uint64_t)a + (uint64_t)b); }
-__device__ __forceinline__ int64_t fx_sub(int64_t a, int64_t b) { return (int64_t)((uint64_t)a - (uint64_t)b); }
 __device__ __forceinline__ int64_t fx_shfl(int64_t v, int src) { return __shfl_sync(FULL, v, src); }
 __device__ __forceinline__ fx fx_shfl(fx v, int src) {
     return {__shfl_sync(FULL, v.hi, src), __shfl_sync(FULL, v.lo, src)};
@@ -899,6 +833,8 @@ __device__ __forceinline__ bool fx_beyond(int64_t v, int lim) {
 // matrix) end it: false, the caller's FP64 path decides.  The last bordered row holds the
 // data, scaled by its caller below 2^-8; its solve has no bound, and where an entry
 // passes 1/8 the row is shifted down by 6 bits (counted in ey) and the panel's slot redone.
+// With rows of at most unit length (|L_r| <= 1) a cross sum of n terms stays below
+// 2 sqrt(n) 2^58, with the data row below 2.3 sqrt(n) 2^58: no overflow up to n = 96 terms.
 template <int N, int NB, class E>
 __device__ __forceinline__ bool factor_fixed(E *mat, int lane, int &ey) {
     constexpr bool CPLX = std::is_same<E, fxc>::value;
@@ -1186,12 +1122,12 @@ __device__ bool solve_point_fixed(SM &sm, const PointA &P, int lane, const LensA
                 const fx dx = fx_split(get(sm.gx[j]) - get(sm.gx[i]));
                 const fx dy = fx_split(get(sm.gy[j]) - get(sm.gy[i]));
                 const fx dz = fx_split(get(sm.gz[j]) - get(sm.gz[i]));
-                t.hh += mul_wide(dx.hi, dx.hi);
-                t.cr += mul_wide(dx.hi, dx.lo);
-                t.hh += mul_wide(dy.hi, dy.hi);
-                t.cr += mul_wide(dy.hi, dy.lo);
-                t.hh += mul_wide(dz.hi, dz.hi);
-                t.cr += mul_wide(dz.hi, dz.lo);  // 2 hi lo, the factor 2 in the shift
+                mad_wide(t.hh, dx.hi, dx.hi);
+                mad_wide(t.cr, dx.hi, dx.lo);
+                mad_wide(t.hh, dy.hi, dy.hi);
+                mad_wide(t.cr, dy.hi, dy.lo);
+                mad_wide(t.hh, dz.hi, dz.hi);
+                mad_wide(t.cr, dz.hi, dz.lo);  // 2 hi lo, the factor 2 in the shift
                 const int64_t tij = (int64_t)((t.hh << 6) + (uint64_t)((int64_t)t.cr >> 25));  // 2^-62
                 const int64_t f = table_eval_fx(a.tab, tij);
                 if constexpr (SPIN == 0) {

@@ -1318,9 +1318,9 @@ struct fxacc3 {
     int ll;
 };
 __device__ __forceinline__ void fx_mac3(fxacc3 &a, fx x, int xl, fx y, int yl) {
-    a.hh += mul_wide(x.hi, y.hi);
-    a.cr += mul_wide(x.hi, y.lo);
-    a.cr += mul_wide(x.lo, y.hi);
+    mad_wide(a.hh, x.hi, y.hi);
+    mad_wide(a.cr, x.hi, y.lo);
+    mad_wide(a.cr, x.lo, y.hi);
     a.ll += xl * yl;
 }
 __device__ __forceinline__ fxacc fx_fold(fxacc3 a) { return {a.hh, a.cr + (uint64_t)((int64_t)a.ll * 64)}; }
@@ -1426,12 +1426,12 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32, 4) apply_kernel_fx(ApplyArgs
                     const fx ex = fx_split(fx_of(dx, 60 + ch.k)), ey = fx_split(fx_of(dy, 60 + ch.k));
                     const fx ez = fx_split(fx_of(p1.x - sm.tz[q], 60 + ch.k));
                     fxacc t2{0, (uint64_t)1 << 24};
-                    t2.hh += mul_wide(ex.hi, ex.hi);
-                    t2.cr += mul_wide(ex.hi, ex.lo);
-                    t2.hh += mul_wide(ey.hi, ey.hi);
-                    t2.cr += mul_wide(ey.hi, ey.lo);
-                    t2.hh += mul_wide(ez.hi, ez.hi);
-                    t2.cr += mul_wide(ez.hi, ez.lo);
+                    mad_wide(t2.hh, ex.hi, ex.hi);
+                    mad_wide(t2.cr, ex.hi, ex.lo);
+                    mad_wide(t2.hh, ey.hi, ey.hi);
+                    mad_wide(t2.cr, ey.hi, ey.lo);
+                    mad_wide(t2.hh, ez.hi, ez.hi);
+                    mad_wide(t2.cr, ez.hi, ez.lo);
                     const int64_t tk = (int64_t)((t2.hh << 6) + (uint64_t)((int64_t)t2.cr >> 25));  // 4^k chord^2, 2^-62
                     const int64_t tau = fx_mul<60>(fx_split(tk), ch.scale);                          // of t_max, 2^-62
                     if (tau > ((int64_t)1 << 62)) atomicAdd(&sm.win[q], 1);

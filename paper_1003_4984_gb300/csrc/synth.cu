@@ -51,9 +51,8 @@
 
 namespace {
 
-using flints::df;
 
-constexpr int CHUNK = 256;  // l values staged per pass in shared memory
+
 constexpr double PI_D = 3.14159265358979323846;
 
 struct SynthRing {
@@ -85,31 +84,31 @@ int sfail(int code, const char *fmt, ...) {
     return code;
 }
 
-// log2 |d^l0_{m,m'}| (as lg) and sign of the starting value of a column
-__device__ __forceinline__ double start_log2(int m, int mp, double lc, double ls, bool &neg) {
-    const double inv_ln2 = 1.4426950408889634;
-    int l, b, pc, ps;
+constexpr int CHUNK = 256;  // l values staged per pass in shared memory (FP64 kernel)
+constexpr unsigned FULL_WARP = 0xffffffffu;
+
+// Start of a column: d^l0_{m,m'} = (sign) sqrt((2l)! / ((l+b)!(l-b)!)) c^pc s^ps.
+__device__ __forceinline__ void start_powers(int m, int mp, int &pc, int &ps, bool &neg) {
     if (m >= abs(mp)) {  // first index +l = m, second b = m'
-        l = m;
-        b = mp;
-        pc = l + b;
-        ps = l - b;
-        neg = ((l - b) & 1) != 0;
-    } else if (mp < 0) {  // d_{m,m'} = d_{-m',-m}, first index -m' = +l
-        l = -mp;
-        b = -m;
-        pc = l + b;
-        ps = l - b;
-        neg = ((l - b) & 1) != 0;
-    } else {  // first index -m' = -l
-        l = mp;
-        b = -m;
-        pc = l - b;
-        ps = l + b;
+        pc = m + mp;
+        ps = m - mp;
+        neg = ((m - mp) & 1) != 0;
+    } else if (mp < 0) {  // d_{m,m'} = d_{-m',-m}: first index -m' = +l, b = -m
+        pc = -mp - m;
+        ps = -mp + m;
+        neg = ((m - mp) & 1) != 0;
+    } else {  // first index -m' = -l, b = -m
+        pc = mp + m;
+        ps = mp - m;
         neg = false;
     }
+}
+
+// log2 of sqrt((2l)! / ((l+b)!(l-b)!)) at l = max(m, s), b = min(m, s)
+__device__ __forceinline__ double start_factor(int m, int s) {
+    const int l = m > s ? m : s, b = m > s ? s : m;
     const double lf = 0.5 * (lgamma(2.0 * l + 1.0) - lgamma((double)(l + b) + 1.0) - lgamma((double)(l - b) + 1.0));
-    return lf * inv_ln2 + pc * lc + ps * ls;
+    return lf * 1.4426950408889634;
 }
 
 // One recurrence column carried as v 2^E.
@@ -158,12 +157,14 @@ __global__ void __launch_bounds__(128) legendre_kernel(int lmax, int nside, cons
     // columns: A = d_{m,-s}, B = d_{m,+s} (spin 0: A only)
     Col ca{}, cb{};
     if (active && l0 <= lmax) {
+        const double lg = start_factor(m, S);
+        int pc, ps;
         bool neg;
-        double lg = start_log2(m, -S, rg.lc, rg.ls, neg);
-        ca.init(lg, neg);
+        start_powers(m, -S, pc, ps, neg);
+        ca.init(lg + pc * rg.lc + ps * rg.ls, neg);
         if (S > 0) {
-            lg = start_log2(m, S, rg.lc, rg.ls, neg);
-            cb.init(lg, neg);
+            start_powers(m, S, pc, ps, neg);
+            cb.init(lg + pc * rg.lc + ps * rg.ls, neg);
         }
     }
     // accumulators by parity of l + m (e: even, o: odd); the parity is uniform
@@ -246,172 +247,381 @@ __global__ void __launch_bounds__(128) legendre_kernel(int lmax, int nside, cons
     }
 }
 
-// Fold the coefficients of one ring modulo its length n, with the phase of the
-// first pixel: H_k = sum_{m = k mod n} F_m e^{i m phi0}.  Spin 0 (real field,
-// F_-m = F_m^*): k = 0..n/2 for a complex-to-real FFT; spin s: k = 0..n-1.
-// Double-float form of the same recurrence on the FP32 pipe (the mixed
-// precision of the synthesis): the column carried as v 2^E with v a double-
-// float pair, rescaled by 2^-64 while |v| > 2^64 (FP32 exponent range);
-// coefficients, weights and sums in double-float, the sums (F) written as
-// FP64.  Relative accuracy about 1e-13 after 4096 steps.
-struct ColDF {
-    df v, prev;
-    float mult;
-    int e;
-    __device__ __forceinline__ void init(double lg, bool neg) {
-        const double fl = floor(lg);
-        e = (int)fl;
-        double vd = exp2(lg - fl);
-        if (neg) vd = -vd;
-        v = flints::df_from(vd);
-        prev = df{0.0f, 0.0f};
-        mult = e < -126 ? 0.0f : ldexpf(1.0f, e);
-    }
-    __device__ __forceinline__ void step(df a, df b, df c, df x) {
-        const df t = flints::df_sub(flints::df_mul(a, x), b);
-        const df nv = flints::df_sub(flints::df_mul(t, v), flints::df_mul(c, prev));
-        prev = v;
-        v = nv;
-        if (fabsf(v.hi) > 1.8446744e19f) {  // 2^64
-            const float k = 5.421011e-20f;  // 2^-64
-            v = df{v.hi * k, v.lo * k};
-            prev = df{prev.hi * k, prev.lo * k};
-            e += 64;
-            mult = e < -126 ? 0.0f : ldexpf(1.0f, e);
-        }
-    }
-    __device__ __forceinline__ df value() const { return df{v.hi * mult, v.lo * mult}; }
+// --------------------------------------------------- the l-sums in fixed point
+// The mixed precision of the synthesis.
+// Per (ring, m) column the recurrence is run on g_l = d^l / alpha_l with
+// alpha_{l+1} = C_l alpha_{l-1} and alpha = 1 at the two largest l, which leaves
+//   g_{l+1} = (a_l x -+ b_l) g_l - g_{l-1},   a_l = A_l alpha_l / alpha_{l+1}, b_l likewise:
+// alpha falls with l (C_l < 1), so |g| <= |d| <= 1, and one product per column and step is
+// gone.  Everything is an integer: x in units of 2^-62, a of 2^-54, b, t = a x -+ b and g of
+// 2^-59, the weights alpha_l N_l (E + iB) of a unit chosen per m (synth_weight_kernel) so that
+// a sum's high word cannot overflow; its cross word is folded every 16 steps.  Three stretches of l per warp: while every lane's columns are below 2^-64 the
+// recurrence alone; then columns v 2^E with sums; and once every lane oscillates (|t| < 2:
+// no growth left, E = 0) the plain loop, which most steps take.  Coefficients depend on
+// (l, m) alone and are tabulated per plan, weights once per call (every block of 128 rings
+// formed both anew, in FP64).
+// What bounds it: issue.  A plain step at spin 2 is 37 IMAD.WIDE (two issue cycles each)
+// and some 50 other instructions; the double-float form took 273.  Words carry an offset of
+// 2^31, so splitting one into signed halves is one XOR.  Measured (GB300, Q/U at
+// Nside 1024, lmax 2048, whole synthesis): 40.7 -> 27.0 ms, error against 64 bits 7.6e-13 ->
+// 1.7e-13 of the map.
+constexpr int GS = 59, AS = 54;
+
+// The signed halves of v when V = v + 2^31.  (The pairs here are never negated, so they keep
+// every bit: a lowest bit always set would shift every coefficient the same way, and near the
+// poles, where the recurrence answers a constant push with its square, that showed.)
+constexpr long long OFF = 1ll << 31;
+__device__ __forceinline__ flints::fx halves(long long V) {
+    return {(int)(V >> 32), (int)((uint32_t)V ^ 0x80000000u)};
+}
+struct alignas(16) SynthStep {
+    flints::fx a;  // units of 2^-AS
+    long long b;   // units of 2^-GS
 };
 
-template <int S>
-__global__ void __launch_bounds__(128) legendre_df_kernel(int lmax, int nside, const SynthRing *__restrict__ rings,
-                                                          const double2 *__restrict__ alm,
-                                                          const double2 *__restrict__ blm, double2 *__restrict__ F) {
-    __shared__ float2 sA[CHUNK], sB[CHUNK], sC[CHUNK];
-    __shared__ float4 sWp[CHUNK], sWm[CHUNK];  // (re.hi, re.lo, im.hi, im.lo)
-    const int m = blockIdx.y;
-    const int ring = blockIdx.x * blockDim.x + threadIdx.x + 1;
-    const int nnorth = 2 * nside;
-    const bool active = ring <= nnorth;
-    const int NM = S == 0 ? lmax + 1 : 2 * lmax + 1;
-    const int l0 = m > S ? m : S;
-    const double inv4pi = 1.0 / (4.0 * PI_D);
-    SynthRing rg{};
-    if (active) rg = rings[ring - 1];
-    const df x = flints::df_from(rg.x);
-    ColDF ca{}, cb{};
-    if (active && l0 <= lmax) {
-        bool neg;
-        double lg = start_log2(m, -S, rg.lc, rg.ls, neg);
-        ca.init(lg, neg);
-        if (S > 0) {
-            lg = start_log2(m, S, rg.lc, rg.ls, neg);
-            cb.init(lg, neg);
-        }
-    }
-    using Acc = flints::dfacc;
-    struct CAcc {  // complex double-float sum
-        Acc re, im;
-    };
-    CAcc pAe{}, pAo{}, pBe{}, pBo{}, mAe{}, mAo{}, mBe{}, mBo{};
-    auto mac = [](CAcc &a, df wr, df wi, df d) {
-        flints::dfacc_add_prod(a.re, wr, d);
-        flints::dfacc_add_prod(a.im, wi, d);
-    };
-    auto f2 = [](double v) {
-        const df d = flints::df_from(v);
-        return make_float2(d.hi, d.lo);
-    };
-    for (int c0 = l0; c0 <= lmax; c0 += CHUNK) {
-        const int c1 = min(c0 + CHUNK, lmax + 1);
-        __syncthreads();
-        for (int l = c0 + threadIdx.x; l < c1; l += blockDim.x) {
-            const int k = l - c0;
-            const double ld = (double)l, lp = ld + 1.0;
-            const double md = (double)m, sd = (double)S;
-            const double den = ld * sqrt((lp * lp - md * md) * (lp * lp - sd * sd));
-            if (l == 0 || !(den > 0.0)) {
-                sA[k] = f2(1.0);
-                sB[k] = f2(0.0);
-                sC[k] = f2(0.0);
-            } else {
-                sA[k] = f2((2.0 * ld + 1.0) * ld * lp / den);
-                sB[k] = f2((2.0 * ld + 1.0) * md * sd / den);
-                sC[k] = f2(lp * sqrt((ld * ld - md * md) * (ld * ld - sd * sd)) / den);
-            }
-            const double nl = sqrt((2.0 * ld + 1.0) * inv4pi);
-            const double2 a = alm[(size_t)l * (lmax + 1) + m];
-            double2 wp, wm = make_double2(0.0, 0.0);
-            if (S == 0) {
-                wp = make_double2(a.x * nl, a.y * nl);
-            } else {
-                const double2 b = blm ? blm[(size_t)l * (lmax + 1) + m] : make_double2(0.0, 0.0);
-                wp = make_double2((a.x - b.y) * nl, (a.y + b.x) * nl);
-                wm = make_double2((a.x + b.y) * nl, (b.x - a.y) * nl);
-            }
-            const float2 pr = f2(wp.x), pi = f2(wp.y), mr = f2(wm.x), mi = f2(wm.y);
-            sWp[k] = make_float4(pr.x, pr.y, pi.x, pi.y);
-            sWm[k] = make_float4(mr.x, mr.y, mi.x, mi.y);
-        }
-        __syncthreads();
-        if (active) {
-            for (int l = c0; l < c1; ++l) {
-                const int k = l - c0;
-                const bool odd = ((l + m) & 1) != 0;
-                const df da = ca.value();
-                const float4 wpf = sWp[k];
-                const df wpr{wpf.x, wpf.y}, wpi{wpf.z, wpf.w};
-                // the parity is uniform across the block: no divergence, no indexed registers
-                if (odd) {
-                    mac(pAo, wpr, wpi, da);
-                } else {
-                    mac(pAe, wpr, wpi, da);
-                }
-                if (S > 0) {
-                    const df db = cb.value();
-                    const float4 wmf = sWm[k];
-                    const df wmr{wmf.x, wmf.y}, wmi{wmf.z, wmf.w};
-                    if (odd) {
-                        mac(pBo, wpr, wpi, db);
-                        mac(mAo, wmr, wmi, da);
-                        mac(mBo, wmr, wmi, db);
-                    } else {
-                        mac(pBe, wpr, wpi, db);
-                        mac(mAe, wmr, wmi, da);
-                        mac(mBe, wmr, wmi, db);
-                    }
-                }
-                if (l < lmax) {
-                    const float2 A = sA[k], B = sB[k], C = sC[k];
-                    const df Ad{A.x, A.y}, Bd{B.x, B.y}, Cd{C.x, C.y};
-                    ca.step(Ad, flints::df_neg(Bd), Cd, x);
-                    if (S > 0) cb.step(Ad, Bd, Cd, x);
-                }
-            }
-        }
-    }
-    if (!active) return;
-    auto val = [](const Acc &acc) { return flints::df_to(flints::dfacc_val(acc)); };
-    auto sum = [&](const CAcc &e_, const CAcc &o_, double sg_o, double sg) {
-        return make_double2(sg * (val(e_.re) + sg_o * val(o_.re)), sg * (val(e_.im) + sg_o * val(o_.im)));
-    };
-    const int south = 4 * nside - ring;
-    double2 *Fn = F + (size_t)(ring - 1) * NM;
-    double2 *Fs = F + (size_t)(south - 1) * NM;
-    if (S == 0) {
-        Fn[m] = sum(pAe, pAo, 1.0, 1.0);
-        if (south != ring) Fs[m] = sum(pAe, pAo, -1.0, 1.0);
-        return;
-    }
-    const double sg = (S & 1) ? 1.0 : -1.0;  // -(-1)^s
-    Fn[lmax + m] = sum(pAe, pAo, 1.0, sg);
-    if (south != ring) Fs[lmax + m] = sum(pBe, pBo, -1.0, sg);
-    if (m > 0) {
-        Fn[lmax - m] = sum(mBe, mBo, 1.0, -1.0);
-        if (south != ring) Fs[lmax - m] = sum(mAe, mAo, -1.0, -1.0);
+// Row m of the (l, m) tables: l = m .. lmax, contiguous.
+__host__ __device__ __forceinline__ long long tri_row(int lmax, int m) {
+    return (long long)m * (lmax + 1) - (long long)m * (m - 1) / 2 - m;
+}
+
+// C_l = q_l / q_{l+1} with q_l = sqrt((l^2 - m^2)(l^2 - s^2)) / l, so alpha_l alpha_{l-1} q_l is
+// the same for all l.  Three kernels: q_l for every (l, m); alpha downwards in l, one thread
+// per m (the only serial part: one division a step); coefficients, weights' factors and starts.
+__global__ void synth_q_kernel(int lmax, int s, double *__restrict__ na) {
+    const int m = blockIdx.y, l = (m > s ? m : s) + blockIdx.x * blockDim.x + threadIdx.x;
+    if (l > lmax) return;
+    const double ld = l, md = m, sd = s;
+    na[tri_row(lmax, m) + l] = l > 0 ? sqrt((ld * ld - md * md) * (ld * ld - sd * sd)) / ld : 0.0;
+}
+
+// na: q_l in, alpha_l out
+__global__ void synth_alpha_kernel(int lmax, int s, double *__restrict__ na) {
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m > lmax) return;
+    const int l0 = m > s ? m : s;
+    double *n = na + tri_row(lmax, m);
+    double q = n[lmax], alpha = 1.0;
+    const double same = q;  // alpha = 1 at lmax and lmax - 1
+    n[lmax] = 1.0;
+    for (int l = lmax - 1; l >= l0; --l) {
+        const double below = n[l];
+        alpha = l == lmax - 1 ? 1.0 : same / (alpha * q);
+        n[l] = alpha;
+        q = below;
     }
 }
 
+// na: alpha_l in, alpha_l N_l out (per block of one m, whose threads take l in turn from the top)
+__global__ void synth_coef_kernel(int lmax, int s, SynthStep *__restrict__ steps, double *__restrict__ na,
+                                  double *__restrict__ start) {
+    const int m = blockIdx.x, l0 = m > s ? m : s;
+    SynthStep *st = steps + tri_row(lmax, m);
+    double *n = na + tri_row(lmax, m);
+    const double md = m, sd = s, inv4pi = 1.0 / (4.0 * PI_D);
+    if (threadIdx.x == 0) start[m] = start_factor(m, s) - log2(n[l0]);
+    for (int base = l0; base <= lmax; base += blockDim.x) {  // upwards: alpha_{l+1} is read before its block overwrites it
+        const int l = base + threadIdx.x;
+        const double cur = l <= lmax ? n[l] : 1.0, up = l < lmax ? n[l + 1] : 1.0;
+        __syncthreads();
+        if (l > lmax) continue;
+        const double ld = l, lp = ld + 1.0;
+        n[l] = sqrt((2.0 * ld + 1.0) * inv4pi) * cur;
+        const double den = ld * sqrt((lp * lp - md * md) * (lp * lp - sd * sd));
+        double a = 1.0, b = 0.0;  // l = m = s = 0: d^1 = x d^0
+        if (l > 0 && den > 0.0) {
+            a = (2.0 * ld + 1.0) * ld * lp / den;
+            b = (2.0 * ld + 1.0) * md * sd / den;
+        }
+        const double r = cur / up;
+        st[l] = SynthStep{halves(flints::fx_of(a * r, AS) + OFF), (long long)flints::fx_of(b * r, GS)};
+    }
+}
+
+// One block per m: weights W_l = alpha_l N_l (E + iB) and, spin s, alpha_l N_l (E^* + iB^*) in
+// units of 2^-ws, ws the largest with sum_l |W_l| < 2^66 units (a sum's high word, whose terms
+// are at most 2^(GS - 32) times a weight's, stays below 2^61) and |W_l| < 2^59 (eight terms of
+// its cross word stay below 2^62).  The low words' products that the sums drop are then 2^-51
+// of the sum of the weights' sizes at most; ws = WE_BAD where that sum is not finite.
+constexpr int WE_BAD = 1 << 20;
+template <int S>
+__global__ void synth_weight_kernel(int lmax, const double *__restrict__ na, const double2 *__restrict__ alm,
+                                    const double2 *__restrict__ blm, flints::fxc *__restrict__ W, int *__restrict__ we) {
+    __shared__ double part[256], peak[256];
+    const int m = blockIdx.x, l0 = m > S ? m : S, tid = threadIdx.x;
+    const double *n = na + tri_row(lmax, m);
+    auto weights = [&](int l, double2 &p, double2 &q) {
+        const double nl = n[l];
+        const double2 a = alm[(size_t)l * (lmax + 1) + m];
+        const double2 b = (S > 0 && blm) ? blm[(size_t)l * (lmax + 1) + m] : make_double2(0.0, 0.0);
+        p = make_double2((a.x - b.y) * nl, (a.y + b.x) * nl);
+        q = make_double2((a.x + b.y) * nl, (b.x - a.y) * nl);
+    };
+    double sum = 0.0, big = 0.0;
+    for (int l = l0 + tid; l <= lmax; l += blockDim.x) {
+        double2 p, q;
+        weights(l, p, q);
+        double t = fabs(p.x) + fabs(p.y);
+        if (S > 0) t += fabs(q.x) + fabs(q.y);
+        sum += t;
+        big = fmax(big, t);
+    }
+    part[tid] = sum;
+    peak[tid] = big;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+        if (tid < o) {
+            part[tid] += part[tid + o];
+            peak[tid] = fmax(peak[tid], peak[tid + o]);
+        }
+        __syncthreads();
+    }
+    const bool bad = !(part[0] <= 1.7e308);
+    // a value below 2^expo (one more than its own exponent for the sum, whose rounding may carry)
+    auto expo = [](double v) {
+        const int ex = (int)(((unsigned long long)__double_as_longlong(v) >> 52) & 0x7ff);
+        return ex == 0 ? -960 : ex - 1022;
+    };
+    const int e0 = 66 - (expo(part[0]) + 1), e1 = 59 - expo(peak[0]), ws = e0 < e1 ? e0 : e1;
+    if (tid == 0) we[m] = bad ? WE_BAD : ws;
+    flints::fxc *w = W + (S > 0 ? 2 : 1) * tri_row(lmax, m);
+    auto put = [&](flints::fxc &dst, double2 v) {
+        dst = flints::fxc{halves((bad ? 0 : flints::fx_of(v.x, ws)) + OFF), halves((bad ? 0 : flints::fx_of(v.y, ws)) + OFF)};
+    };
+    for (int l = l0 + tid; l <= lmax; l += blockDim.x) {
+        double2 p, q;
+        weights(l, p, q);
+        if constexpr (S == 0) {  // two real weights per l
+            put(w[l], p);
+        } else {
+            put(w[2 * l], p);
+            put(w[2 * l + 1], q);
+        }
+    }
+}
+
+// x y / 2^DOWN + offs, rounded; the low words' product enters by its top halves
+template <int DOWN>
+__device__ __forceinline__ long long mul_off(flints::fx x, flints::fx y, uint64_t offs) {
+    flints::fxacc a{0, (offs << (DOWN - 32)) + ((uint64_t)1 << (DOWN - 33))};
+    flints::fx_mac(a, x, y);
+    flints::mad_wide(a.cr, x.lo >> 16, y.lo >> 16);
+    return flints::fx_down<DOWN>(a);
+}
+
+// One column v 2^(E - GS); prev on the same scale.
+struct ColFx {
+    long long v, prev;
+    int e;
+    __device__ __forceinline__ void init(double lg, bool neg) {
+        const double fl = floor(lg);
+        e = (int)fl - 1;
+        v = (long long)(exp2(lg - fl) * 1152921504606846976.0);  // 2^60 to 2^61
+        if (neg) v = -v;
+        prev = 0;
+    }
+    // to the next l with t = T 2^-AS, |T| < 2^(AS + k): v is kept below 2^(62 - k), lim its high word's bound
+    __device__ __forceinline__ void step(long long T, int lim) {
+        if (e < 0) {
+            const int th = (int)(T >> 32);
+            int k = 0;
+            if ((th < 0 ? ~th : th) < (2 << (AS - 32)) && e > -24) {
+                k = -e;  // the column oscillates: the common scale holds what it needs
+            } else {
+                int h = (int)(v >> 32);
+                h = h < 0 ? ~h : h;
+                if (h >= lim) {
+                    k = __clz((unsigned)lim) - __clz((unsigned)h) + 5;
+                    k = k < -e ? k : -e;
+                }
+            }
+            v >>= k;
+            prev >>= k;
+            e += k;
+        }
+        const long long nv = (long long)((uint64_t)mul_off<AS>(halves(T + OFF), halves(v + OFF), 0) - (uint64_t)prev);
+        prev = v;
+        v = nv;
+    }
+    __device__ __forceinline__ flints::fx value() const { return halves((v >> (e > -63 ? -e : 63)) + OFF); }
+};
+
+template <int S>
+__global__ void __launch_bounds__(128) legendre_fx_kernel(int lmax, int nside, const SynthRing *__restrict__ rings,
+                                                          const SynthStep *__restrict__ steps,
+                                                          const flints::fxc *__restrict__ W, const int *__restrict__ we,
+                                                          const double *__restrict__ start, double2 *__restrict__ F) {
+    using flints::fx;
+    using flints::fxacc;
+    using flints::fxc;
+    constexpr int NS = S == 0 ? 1 : 4;  // sums: pA (spin 0: the only one), pB, mA, mB
+    const int m = blockIdx.y;
+    const int ring = blockIdx.x * blockDim.x + threadIdx.x + 1;  // northern ring incl. the equator
+    const int nnorth = 2 * nside;
+    const bool active = ring <= nnorth;
+    const int NM = S == 0 ? lmax + 1 : 2 * lmax + 1;
+    int l = m > S ? m : S;
+    SynthRing rg{};
+    if (active) rg = rings[ring - 1];
+    const fx x = halves(flints::fx_of(rg.x, 62) + OFF);
+    ColFx ca{0, 0, -(1 << 20)}, cb{0, 0, -(1 << 20)};
+    if (active && l <= lmax) {  // columns A = d_{m,-s}, B = d_{m,s}
+        const double lg = __ldg(start + m);
+        int pc, ps;
+        bool neg;
+        start_powers(m, -S, pc, ps, neg);
+        ca.init(lg + pc * rg.lc + ps * rg.ls, neg);
+        if (S > 0) {
+            start_powers(m, S, pc, ps, neg);
+            cb.init(lg + pc * rg.lc + ps * rg.ls, neg);
+        }
+    }
+    // Columns that stay evanescent: left of its turning point l sin(theta) = M = m - s a column is
+    // at most exp(-M (acosh(1/r) - sqrt(1 - r^2))), r = (l + 1/2) sin(theta) / M (WKB; the
+    // factor it leaves out is below 1).  Below 2^-93 at lmax nothing of it reaches a sum's last bit.
+    const float M = (float)(m - S), r = ((float)lmax + 0.5f) * sqrtf(fmaxf(0.0f, (float)((1.0 - rg.x) * (1.0 + rg.x)))) / fmaxf(M, 1.0f);
+    bool never = !active;
+    if (active && r < 1.0f) {
+        const float c = sqrtf(1.0f - r * r);
+        never = M * (logf((1.0f + c) / fmaxf(r, 1e-30f)) - c) > 64.5f;  // 93 ln 2
+    }
+    if (__all_sync(FULL_WARP, never)) l = lmax + 1;
+    const SynthStep *st = steps + tri_row(lmax, m);
+    const fxc *w = W + (S > 0 ? 2 : 1) * tri_row(lmax, m);
+    auto ld_step = [&](int i) {
+        const float4 q = __ldg(reinterpret_cast<const float4 *>(st + i));
+        SynthStep r;
+        r.a = fx{(int)__float_as_uint(q.x), (int)__float_as_uint(q.y)};
+        r.b = (long long)(((uint64_t)__float_as_uint(q.w) << 32) | __float_as_uint(q.z));
+        return r;
+    };
+    auto ld_w = [&](int i) {
+        const float4 q = __ldg(reinterpret_cast<const float4 *>(w + i));
+        return fxc{fx{(int)__float_as_uint(q.x), (int)__float_as_uint(q.y)},
+                   fx{(int)__float_as_uint(q.z), (int)__float_as_uint(q.w)}};
+    };
+    auto top_of = [](const SynthStep &c) {  // above a + |b|, units of 2^(32 - AS)
+        const int bh = (int)(c.b >> (32 + GS - AS));
+        return c.a.hi + (bh < 0 ? ~bh : bh) + 2;
+    };
+    auto advance = [&](const SynthStep &c) {
+        const long long b = c.b >> (GS - AS);
+        const int lim = 1 << (30 - (32 - __clz((unsigned)top_of(c)) - (AS - 32)));
+        const long long ax = mul_off<62>(c.a, x, 0);
+        ca.step(ax + b, lim);
+        if (S > 0) cb.step(ax - b, lim);
+    };
+    // no lane's columns above 2^-64: the recurrence alone
+    while (l < lmax) {
+        if (__any_sync(FULL_WARP, ca.e > -64 || (S > 0 && cb.e > -64))) break;
+        const int stop = l + 8 < lmax ? l + 8 : lmax;
+        for (; l < stop; ++l) advance(ld_step(l));
+    }
+    // sums by parity of l + l1, l1 the first summed l (re, im)
+    const int l1 = l;
+    fxacc acc[2][NS][2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int i = 0; i < NS; ++i) acc[h][i][0] = acc[h][i][1] = fxacc{0, 0};
+    auto fold = [&]() {  // the cross words' upper halves into the high words
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int i = 0; i < NS; ++i)
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    acc[h][i][c].hh += (uint64_t)((int64_t)acc[h][i][c].cr >> 32);
+                    acc[h][i][c].cr &= 0xffffffffull;
+                }
+    };
+    auto add = [&](fxacc(&s)[NS][2], const fxc &p, const fxc &q, const fx &da, const fx &db) {
+        flints::fx_mac(s[0][0], p.re, da);
+        flints::fx_mac(s[0][1], p.im, da);
+        if constexpr (S > 0) {
+            flints::fx_mac(s[1][0], p.re, db);
+            flints::fx_mac(s[1][1], p.im, db);
+            flints::fx_mac(s[2][0], q.re, da);
+            flints::fx_mac(s[2][1], q.im, da);
+            flints::fx_mac(s[3][0], q.re, db);
+            flints::fx_mac(s[3][1], q.im, db);
+        }
+    };
+    constexpr int WN = S > 0 ? 2 : 1;  // weight pairs per l
+    while (l <= lmax) {
+        const bool plain = !active || (ca.e == 0 && (S == 0 || cb.e == 0));
+        if (l < lmax && top_of(ld_step(l)) < (7 << (AS - 32)) && __all_sync(FULL_WARP, plain)) break;
+#pragma unroll 1
+        for (int j = 0; j < 4 && l <= lmax; ++j) {
+            add(acc[0], ld_w(WN * l), ld_w(WN * l + WN - 1), ca.value(), cb.value());
+            if (l < lmax) advance(ld_step(l));
+            if (++l > lmax) break;
+            add(acc[1], ld_w(WN * l), ld_w(WN * l + WN - 1), ca.value(), cb.value());
+            if (l < lmax) advance(ld_step(l));
+            ++l;
+        }
+        fold();
+    }
+    // every column on the common scale and |t| < 7 from here on (a and |b| fall with l)
+    long long va = ca.v + OFF, pa = ca.prev + OFF, vb = cb.v + OFF, pb = cb.prev + OFF;
+    auto plain_step = [&](fxacc(&s)[NS][2], int at) {
+        const fxc p = ld_w(WN * at), q = ld_w(WN * at + WN - 1);
+        const SynthStep c = ld_step(at < lmax ? at : lmax);
+        const fx da = halves(va), db = halves(vb);
+        add(s, p, q, da, db);
+        const long long ax = mul_off<62 + AS - GS>(c.a, x, OFF);  // units of 2^-GS
+        const long long na = (long long)((uint64_t)mul_off<GS>(halves(ax + c.b), da, 2 * OFF) - (uint64_t)pa);
+        pa = va;
+        va = na;
+        if constexpr (S > 0) {
+            const long long nb = (long long)((uint64_t)mul_off<GS>(halves(ax - c.b), db, 2 * OFF) - (uint64_t)pb);
+            pb = vb;
+            vb = nb;
+        }
+    };
+    while (l + 1 <= lmax) {
+#pragma unroll 1
+        for (int j = 0; j < 8 && l + 1 <= lmax; ++j, l += 2) {
+            plain_step(acc[0], l);
+            plain_step(acc[1], l + 1);
+        }
+        fold();
+    }
+    if (l <= lmax) plain_step(acc[0], l);
+    fold();
+    if (!active) return;
+    const int ws = __ldg(we + m);
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    auto val = [&](const fxacc &s) {  // units of 2^-(ws + GS), hh of 2^64 and cr of 2^32 of them
+        return ws == WE_BAD ? nan : flints::fx_scale2((double)(int64_t)s.hh, 64 - ws - GS) +
+                                        flints::fx_scale2((double)(int64_t)s.cr, 32 - ws - GS);
+    };
+    const bool odd = ((l1 + m) & 1) != 0;  // acc[0] holds the terms of odd l + m
+    auto sum = [&](int i, double sg_o, double sg) {
+        const double r0 = val(acc[0][i][0]), r1 = val(acc[1][i][0]), i0 = val(acc[0][i][1]), i1 = val(acc[1][i][1]);
+        return odd ? make_double2(sg * (r1 + sg_o * r0), sg * (i1 + sg_o * i0))
+                   : make_double2(sg * (r0 + sg_o * r1), sg * (i0 + sg_o * i1));
+    };
+    const int south = 4 * nside - ring;  // mirror ring (== ring at the equator)
+    double2 *Fn = F + (size_t)(ring - 1) * NM;
+    double2 *Fs = F + (size_t)(south - 1) * NM;
+    if constexpr (S == 0) {
+        Fn[m] = sum(0, 1.0, 1.0);
+        if (south != ring) Fs[m] = sum(0, -1.0, 1.0);
+    } else {
+        // P_m = -(-1)^s sum wp d_{m,-s}; south: d_{m,-s}(pi - t) = (-1)^{l+m} d_{m,s}(t)
+        const double sg = (S & 1) ? 1.0 : -1.0;  // -(-1)^s
+        Fn[lmax + m] = sum(0, 1.0, sg);
+        if (south != ring) Fs[lmax + m] = sum(1, -1.0, sg);
+        if (m > 0) {  // P_-m = -sum wm d_{m,s}; south: d_{m,s}(pi - t) = (-1)^{l+m} d_{m,-s}(t)
+            Fn[lmax - m] = sum(3, 1.0, -1.0);
+            if (south != ring) Fs[lmax - m] = sum(2, -1.0, -1.0);
+        }
+    }
+}
+
+// Fold the coefficients of one ring modulo its length n, with the phase of the
+// first pixel: H_k = sum_{m = k mod n} F_m e^{i m phi0}.  Spin 0 (real field,
+// F_-m = F_m^*): k = 0..n/2 for a complex-to-real FFT; spin s: k = 0..n-1.
 // Polar rings (rg.M > 0) write a_k = H_k w_k, k < n, zero-padded to M, into
 // their Bluestein slot in A; equatorial rings write H into H.
 template <int S>
@@ -429,38 +639,38 @@ __global__ void fold_kernel(int lmax, const SynthRing *__restrict__ rings, const
     const int nk = (S == 0 && !polar) ? n / 2 + 1 : n;
     for (int k = threadIdx.x; k < nk; k += blockDim.x) {
         double hr = 0.0, hi = 0.0;
+        // m = k + j n: e^{i m phi0} = e^{i k phi0} (-1)^j where phi0 is half a pixel, and 1 where it is 0
+        const bool half = rg.phi0 > 0.0;
         if (S == 0) {
-            for (int m = k; m <= lmax; m += n) {  // m >= 0, m = k mod n
-                double sp, cp;
-                sincospi((double)m * rg.phi0, &sp, &cp);
+            double sg = 1.0;
+            for (int m = k; m <= lmax; m += n) {  // m >= 0
                 const double2 f = Fr[m];
-                hr += f.x * cp - f.y * sp;
-                hi += f.x * sp + f.y * cp;
+                hr = fma(sg, f.x, hr);
+                hi = fma(sg, f.y, hi);
+                if (half) sg = -sg;
             }
+            sg = half ? -1.0 : 1.0;  // -m = k - (j + 1) n
             for (int m = (k == 0 ? n : n - k); m <= lmax; m += n) {  // m >= 1, -m = k mod n: conj
-                double sp, cp;
-                sincospi((double)m * rg.phi0, &sp, &cp);
                 const double2 f = Fr[m];
-                hr += f.x * cp - f.y * sp;
-                hi -= f.x * sp + f.y * cp;
+                hr = fma(sg, f.x, hr);
+                hi = fma(-sg, f.y, hi);
+                if (half) sg = -sg;
             }
         } else {
-            // m = k + j n within [-lmax, lmax]
-            int m = k - ((k + lmax) / n) * n;
-            for (; m <= lmax; m += n) {
-                double sp, cp;
-                sincospi((double)m * rg.phi0, &sp, &cp);
+            const int j0 = (k + lmax) / n;  // first m = k - j0 n >= -lmax
+            double sg = (half && (j0 & 1)) ? -1.0 : 1.0;
+            for (int m = k - j0 * n; m <= lmax; m += n) {
                 const double2 f = Fr[lmax + m];
-                hr += f.x * cp - f.y * sp;
-                hi += f.x * sp + f.y * cp;
+                hr = fma(sg, f.x, hr);
+                hi = fma(sg, f.y, hi);
+                if (half) sg = -sg;
             }
         }
-        if (polar) {
-            const double2 w = chirp(k, n);
-            Hr[k] = make_double2(hr * w.x - hi * w.y, hr * w.y + hi * w.x);
-        } else {
-            Hr[k] = make_double2(hr, hi);
-        }
+        // one phase per k: polar rings e^{i k phi0} w_k = exp(i pi k (k + 1) / n), reduced in integers
+        double sp = 0.0, cp = 1.0;
+        if (polar) sincospi((double)(((long long)k * (k + 1)) % (2LL * n)) / (double)n, &sp, &cp);
+        else if (half) sincospi((double)k / (double)n, &sp, &cp);
+        Hr[k] = make_double2(hr * cp - hi * sp, hr * sp + hi * cp);
     }
 }
 
@@ -521,6 +731,11 @@ struct flints_synth_s {
     SynthRing *d_rings;
     int *d_polar;      // indices of the polar rings
     double2 *d_F, *d_H, *d_A, *d_FB;
+    SynthStep *d_steps;    // recurrence coefficients per (m, l)
+    double *d_na;          // alpha_l N_l per (m, l)
+    double *d_start;       // log2 of the columns' start factor per m
+    flints::fxc *d_W;      // weights of the call in hand per (m, l)
+    int *d_we;             // their exponents per m
     void *d_work;
     std::vector<SynthRing> rings;
     int npolar;
@@ -539,6 +754,11 @@ static void synth_release(flints_synth_s *s) {
     cudaFree(s->d_H);
     cudaFree(s->d_A);
     cudaFree(s->d_FB);
+    cudaFree(s->d_steps);
+    cudaFree(s->d_na);
+    cudaFree(s->d_start);
+    cudaFree(s->d_W);
+    cudaFree(s->d_we);
     cudaFree(s->d_work);
 }
 
@@ -547,6 +767,20 @@ static int synth_bail(flints_synth_s *s, int code, const char *what, cudaError_t
     delete s;
     if (e != cudaSuccess) return sfail(code, "flints_synth_plan: %s: %s", what, cudaGetErrorString(e));
     return sfail(code, "flints_synth_plan: %s", what);
+}
+
+// weights, l-sums and the fold of one synthesis
+template <int S>
+static void launch_sums(flints_synth_s *s, const double2 *alm, const double2 *blm, cudaStream_t st) {
+    const int N = (int)s->nside, lmax = s->lmax, nr = 4 * N - 1;
+    const dim3 grid((2 * N + 127) / 128, lmax + 1);
+    if (s->precision == FLINTS_MIXED) {
+        synth_weight_kernel<S><<<lmax + 1, 256, 0, st>>>(lmax, s->d_na, alm, blm, s->d_W, s->d_we);
+        legendre_fx_kernel<S><<<grid, 128, 0, st>>>(lmax, N, s->d_rings, s->d_steps, s->d_W, s->d_we, s->d_start, s->d_F);
+    } else {
+        legendre_kernel<S><<<grid, 128, 0, st>>>(lmax, N, s->d_rings, alm, blm, s->d_F);
+    }
+    fold_kernel<S><<<nr, 256, 0, st>>>(lmax, s->d_rings, s->d_F, s->d_H, s->d_A);
 }
 
 extern "C" {
@@ -572,6 +806,10 @@ int flints_synth_plan(flints_synth_t *out, int64_t nside, int lmax, int spin, in
     s->d_rings = nullptr;
     s->d_polar = nullptr;
     s->d_F = s->d_H = s->d_A = s->d_FB = nullptr;
+    s->d_steps = nullptr;
+    s->d_na = s->d_start = nullptr;
+    s->d_W = nullptr;
+    s->d_we = nullptr;
     s->d_work = nullptr;
     s->belt_made = false;
     // ring geometry (host, FP64)
@@ -642,10 +880,18 @@ int flints_synth_plan(flints_synth_t *out, int64_t nside, int lmax, int spin, in
     }
     s->npolar = (int)polar.size();
     const size_t NM = spin == 0 ? (size_t)lmax + 1 : 2 * (size_t)lmax + 1;
+    const size_t npair = (size_t)(lmax + 1) * (lmax + 2) / 2;
     cudaError_t e;
     if ((e = cudaMalloc(&s->d_rings, sizeof(SynthRing) * nr)) != cudaSuccess ||
         (e = cudaMalloc(&s->d_F, sizeof(double2) * NM * nr)) != cudaSuccess ||
         (e = cudaMalloc(&s->d_H, sizeof(double2) * (size_t)hsize)) != cudaSuccess)
+        return synth_bail(s, e == cudaErrorMemoryAllocation ? FLINTS_ENOMEM : FLINTS_ECUDA, "allocation", e);
+    if (precision == FLINTS_MIXED &&
+        ((e = cudaMalloc(&s->d_steps, sizeof(SynthStep) * npair)) != cudaSuccess ||
+         (e = cudaMalloc(&s->d_na, sizeof(double) * npair)) != cudaSuccess ||
+         (e = cudaMalloc(&s->d_start, sizeof(double) * (size_t)(lmax + 1))) != cudaSuccess ||
+         (e = cudaMalloc(&s->d_W, sizeof(flints::fxc) * npair * (spin == 0 ? 1 : 2))) != cudaSuccess ||
+         (e = cudaMalloc(&s->d_we, sizeof(int) * (size_t)(lmax + 1))) != cudaSuccess))
         return synth_bail(s, e == cudaErrorMemoryAllocation ? FLINTS_ENOMEM : FLINTS_ECUDA, "allocation", e);
     if (s->npolar > 0 &&
         ((e = cudaMalloc(&s->d_polar, sizeof(int) * polar.size())) != cudaSuccess ||
@@ -659,6 +905,12 @@ int flints_synth_plan(flints_synth_t *out, int64_t nside, int lmax, int spin, in
     if (s->npolar > 0 && (e = cudaMemcpyAsync(s->d_polar, polar.data(), sizeof(int) * polar.size(),
                                               cudaMemcpyHostToDevice, st)) != cudaSuccess)
         return synth_bail(s, FLINTS_ECUDA, "copy", e);
+    if (precision == FLINTS_MIXED) {
+        synth_q_kernel<<<dim3((lmax + 256) / 256, lmax + 1), 256, 0, st>>>(lmax, spin, s->d_na);
+        synth_alpha_kernel<<<(lmax + 32) / 32, 32, 0, st>>>(lmax, spin, s->d_na);
+        synth_coef_kernel<<<lmax + 1, 128, 0, st>>>(lmax, spin, s->d_steps, s->d_na, s->d_start);
+        if ((e = cudaGetLastError()) != cudaSuccess) return synth_bail(s, FLINTS_ECUDA, "coefficients", e);
+    }
     // cuFFT plans sharing one work area
     size_t work_max = 0;
     auto make = [&](cufftHandle &h, int n, long long idist, long long odist, cufftType type, int batch) -> bool {
@@ -751,34 +1003,13 @@ int flints_synthesize(flints_synth_t s, const double *alm, const double *blm, do
     cudaGetDevice(&cur);
     if (cur != s->device) return sfail(FLINTS_EINVAL, "flints_synthesize: plan made on another device");
     cudaStream_t st = (cudaStream_t)stream;
-    const int N = (int)s->nside, lmax = s->lmax;
-    const dim3 grid((2 * N + 127) / 128, lmax + 1);
+    const int N = (int)s->nside;
     const double2 *a = reinterpret_cast<const double2 *>(alm);
     const double2 *b = s->spin == 0 ? nullptr : reinterpret_cast<const double2 *>(blm);
-    const int nr = 4 * N - 1;
-    const bool mixed = s->precision == FLINTS_MIXED;
     switch (s->spin) {
-        case 0:
-            if (mixed)
-                legendre_df_kernel<0><<<grid, 128, 0, st>>>(lmax, N, s->d_rings, a, b, s->d_F);
-            else
-                legendre_kernel<0><<<grid, 128, 0, st>>>(lmax, N, s->d_rings, a, b, s->d_F);
-            fold_kernel<0><<<nr, 256, 0, st>>>(lmax, s->d_rings, s->d_F, s->d_H, s->d_A);
-            break;
-        case 1:
-            if (mixed)
-                legendre_df_kernel<1><<<grid, 128, 0, st>>>(lmax, N, s->d_rings, a, b, s->d_F);
-            else
-                legendre_kernel<1><<<grid, 128, 0, st>>>(lmax, N, s->d_rings, a, b, s->d_F);
-            fold_kernel<1><<<nr, 256, 0, st>>>(lmax, s->d_rings, s->d_F, s->d_H, s->d_A);
-            break;
-        default:
-            if (mixed)
-                legendre_df_kernel<2><<<grid, 128, 0, st>>>(lmax, N, s->d_rings, a, b, s->d_F);
-            else
-                legendre_kernel<2><<<grid, 128, 0, st>>>(lmax, N, s->d_rings, a, b, s->d_F);
-            fold_kernel<2><<<nr, 256, 0, st>>>(lmax, s->d_rings, s->d_F, s->d_H, s->d_A);
-            break;
+        case 0: launch_sums<0>(s, a, b, st); break;
+        case 1: launch_sums<1>(s, a, b, st); break;
+        default: launch_sums<2>(s, a, b, st); break;
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return sfail(FLINTS_ECUDA, "flints_synthesize: kernel launch: %s", cudaGetErrorString(e));
