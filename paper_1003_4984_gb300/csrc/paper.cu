@@ -549,7 +549,7 @@ template <int K>
 __global__ void __launch_bounds__(APPLY_WARPS * 32) apply_kernel(ApplyArgs a) {
     __shared__ double stx[APPLY_WARPS][32], sty[APPLY_WARPS][32], stz[APPLY_WARPS][32];
     __shared__ int64_t scp[APPLY_WARPS][32];
-    __shared__ double sc[APPLY_WARPS][K > GROUP ? K : 1], sy[APPLY_WARPS][K > GROUP ? K : 1];
+    __shared__ double sc[APPLY_WARPS][K], sy[APPLY_WARPS][K];
     // per target of the tile: w . y, w . c, class and window flag, finished one
     // target per lane after the tile
     __shared__ double rv[APPLY_WARPS][32], rq[APPLY_WARPS][32];
@@ -572,183 +572,121 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32) apply_kernel(ApplyArgs a) {
         }
         __syncwarp();
         const int npt = a.count - tile * 32 < 32 ? (int)(a.count - tile * 32) : 32;
-        if constexpr (K <= GROUP) {
-            // three targets at a time, one per group of GROUP lanes (lanes 30, 31 idle)
-            const int g = lane / GROUP, l = lane - g * GROUP, base = g * GROUP;
-            for (int q0 = 0; q0 < npt; q0 += 3) {
-                const int q = q0 + g;
-                const bool has = g < 3 && q < npt;
-                double tx = 0.0, ty = 0.0, tz = 0.0;
-                int64_t c = 0;
-                if (has) {
-                    tx = stx[wid][q];
-                    ty = sty[wid][q];
-                    tz = stz[wid][q];
-                    c = scp[wid][q];
-                }
-                const int32_t sl = has ? __ldg(a.slot + c) : 0;
-                double cv = 0.0, yv = 0.0;
-                bool win = false;
-                if (has && l < K) {
-                    const int32_t m = __ldg(a.members + c * K + l);
-                    if (m >= 0) {
-                        double mx, my, mz;
-                        member_vec(a.pv, m, mx, my, mz);
-                        const double dx = tx - mx, dy = ty - my, dz = tz - mz;
-                        const double t = dx * dx + dy * dy + dz * dz;
-                        win = t > a.tab.t_max;
-                        cv = table_eval<double>(a.tab, t);
-                        yv = __ldg(a.map + m);
-                    }
-                }
-                // z_c = L^-1 c, z_y = L^-1 y: lane l of the group accumulates row l
-                const double *Lr = a.linv + (int64_t)sl * linv_len(K);
-                double zc = 0.0, zy = 0.0;
+                    // one target at a time; lanes own members l and l + 32.  Consecutive
+                    // targets in one coarse pixel reuse the members' positions and data.
+                    int64_t prev = -1;
+                    double m0x = 0.0, m0y = 0.0, m0z = 0.0, y0 = 0.0, m1x = 0.0, m1y = 0.0, m1z = 0.0, y1 = 0.0;
+                    bool v0 = false, v1 = false;
+                    for (int q = 0; q < npt; ++q) {
+                        const double tx = stx[wid][q], ty = sty[wid][q], tz = stz[wid][q];
+                        const int64_t c = scp[wid][q];
+                        const int32_t sl = __ldg(a.slot + c);
+                        if (c != prev) {
+                            prev = c;
+                            const int32_t *mem = a.members + c * K;
+                            v0 = false;
+                            v1 = false;
+                            y0 = 0.0;
+                            y1 = 0.0;
+                            if (lane < K) {
+                                const int32_t m = __ldg(mem + lane);
+                                if (m >= 0) {
+                                    member_vec(a.pv, m, m0x, m0y, m0z);
+                                    y0 = __ldg(a.map + m);
+                                    v0 = true;
+                                }
+                            }
+                            if (lane + 32 < K) {
+                                const int32_t m = __ldg(mem + lane + 32);
+                                if (m >= 0) {
+                                    member_vec(a.pv, m, m1x, m1y, m1z);
+                                    y1 = __ldg(a.map + m);
+                                    v1 = true;
+                                }
+                            }
+                        }
+                        double c0 = 0.0, c1 = 0.0;
+                        bool win = false;
+                        if (v0) {
+                            const double dx = tx - m0x, dy = ty - m0y, dz = tz - m0z;
+                            const double t = dx * dx + dy * dy + dz * dz;
+                            win |= t > a.tab.t_max;
+                            c0 = table_eval<double>(a.tab, t);
+                        }
+                        if (v1) {
+                            const double dx = tx - m1x, dy = ty - m1y, dz = tz - m1z;
+                            const double t = dx * dx + dy * dy + dz * dz;
+                            win |= t > a.tab.t_max;
+                            c1 = table_eval<double>(a.tab, t);
+                        }
+                        // z_c = L^-1 c, z_y = L^-1 y from the lane-step block; c and y go to
+                        // the warp's shared slots.  Rows 0..31: lanes 2p, 2p + 1 run through
+                        // the 33 entries of rows p and 31 - p (lane 2p switches from row p
+                        // to row 31 - p after column p; the two halves of row 31 - p are
+                        // joined by a shuffle).  Rows 32..35: lane l takes row 32 + (l & 3)
+                        // on columns (l >> 2) + 8t, eight partial sums joined by shuffles.
+                        static_assert(K == 36, "the lane-step layout is laid out for K = 36");
+                        const double *Lr = a.linv + (int64_t)sl * linv_len(K);
+                        __syncwarp();
+                        sc[wid][lane] = c0;
+                        sy[wid][lane] = y0;
+                        if (lane < K - 32) {
+                            sc[wid][32 + lane] = c1;
+                            sy[wid][32 + lane] = y1;
+                        }
+                        __syncwarp();
+                        const int pp = lane >> 1, odd = lane & 1;
+                        double zca = 0.0, zya = 0.0, zc0 = 0.0, zy0 = 0.0, zc1 = 0.0, zy1 = 0.0;
 #pragma unroll
-                for (int j = 0; j < K; ++j) {
-                    const double cj = __shfl_sync(FULL, cv, base + j);
-                    const double yj = __shfl_sync(FULL, yv, base + j);
-                    if (has && l < K && l >= j) {
-                        const double e = __ldg(Lr + col_start(K, j) + l - j);
-                        zc = fma(e, cj, zc);
-                        zy = fma(e, yj, zy);
-                    }
-                }
-                // group sums over lanes 0 .. GROUP-1: fold 8-9 onto 0-1, then halve 8 -> 1
-                double vs = zc * zy, qs = zc * zc;
+                        for (int u = 0; u < LS_STEPS; ++u) {
+                            const int t = odd ? LS_STEPS + u : u;
+                            if (!odd && u == pp + 1) {
+                                zca = zc0;
+                                zya = zy0;
+                                zc0 = 0.0;
+                                zy0 = 0.0;
+                            }
+                            int j = t <= pp ? t : t - pp - 1;
+                            j = j < K ? j : K - 1;  // the zero pad
+                            const double e = __ldg(Lr + u * 32 + lane);
+                            zc0 = fma(e, sc[wid][j], zc0);
+                            zy0 = fma(e, sy[wid][j], zy0);
+                        }
+                        const double zcb = zc0 + __shfl_xor_sync(FULL, zc0, 1), zyb = zy0 + __shfl_xor_sync(FULL, zy0, 1);
+                        {
+                            const int g = lane >> 2;
 #pragma unroll
-                for (int o = 8; o >= 1; o >>= 1) {
-                    const double tv = __shfl_sync(FULL, vs, lane + o), tq = __shfl_sync(FULL, qs, lane + o);
-                    if (l < o && l + o < GROUP) {
-                        vs += tv;
-                        qs += tq;
-                    }
-                }
-                const unsigned wb = __ballot_sync(FULL, win);
-                if (has && l == 0) {
-                    rv[wid][q] = vs;
-                    rq[wid][q] = qs;
-                    rsl[wid][q] = sl;
-                    rwin[wid][q] = ((wb >> base) & ((1u << GROUP) - 1u)) != 0;
-                }
-            }
-        } else {
-            // one target at a time; lanes own members l and l + 32.  Consecutive
-            // targets in one coarse pixel reuse the members' positions and data.
-            int64_t prev = -1;
-            double m0x = 0.0, m0y = 0.0, m0z = 0.0, y0 = 0.0, m1x = 0.0, m1y = 0.0, m1z = 0.0, y1 = 0.0;
-            bool v0 = false, v1 = false;
-            for (int q = 0; q < npt; ++q) {
-                const double tx = stx[wid][q], ty = sty[wid][q], tz = stz[wid][q];
-                const int64_t c = scp[wid][q];
-                const int32_t sl = __ldg(a.slot + c);
-                if (c != prev) {
-                    prev = c;
-                    const int32_t *mem = a.members + c * K;
-                    v0 = false;
-                    v1 = false;
-                    y0 = 0.0;
-                    y1 = 0.0;
-                    if (lane < K) {
-                        const int32_t m = __ldg(mem + lane);
-                        if (m >= 0) {
-                            member_vec(a.pv, m, m0x, m0y, m0z);
-                            y0 = __ldg(a.map + m);
-                            v0 = true;
+                            for (int t = 0; t < LS_TAIL; ++t) {
+                                const int j = g + 8 * t < K ? g + 8 * t : K - 1;  // zero entries past the diagonal
+                                const double e = __ldg(Lr + (LS_STEPS + t) * 32 + lane);
+                                zc1 = fma(e, sc[wid][j], zc1);
+                                zy1 = fma(e, sy[wid][j], zy1);
+                            }
+#pragma unroll
+                            for (int o = 4; o < 32; o <<= 1) {
+                                zc1 += __shfl_xor_sync(FULL, zc1, o);
+                                zy1 += __shfl_xor_sync(FULL, zy1, o);
+                            }
+                        }
+                        // even lanes count rows p and 31 - p, lanes 0..3 rows 32..35, each once
+                        double v = odd ? 0.0 : zca * zya + zcb * zyb, qc = odd ? 0.0 : zca * zca + zcb * zcb;
+                        if (lane < K - 32) {
+                            v = fma(zc1, zy1, v);
+                            qc = fma(zc1, zc1, qc);
+                        }
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) {
+                            v += __shfl_xor_sync(FULL, v, o);
+                            qc += __shfl_xor_sync(FULL, qc, o);
+                        }
+                        const bool any_win = __any_sync(FULL, win);
+                        if (lane == 0) {
+                            rv[wid][q] = v;
+                            rq[wid][q] = qc;
+                            rsl[wid][q] = sl;
+                            rwin[wid][q] = any_win;
                         }
                     }
-                    if (lane + 32 < K) {
-                        const int32_t m = __ldg(mem + lane + 32);
-                        if (m >= 0) {
-                            member_vec(a.pv, m, m1x, m1y, m1z);
-                            y1 = __ldg(a.map + m);
-                            v1 = true;
-                        }
-                    }
-                }
-                double c0 = 0.0, c1 = 0.0;
-                bool win = false;
-                if (v0) {
-                    const double dx = tx - m0x, dy = ty - m0y, dz = tz - m0z;
-                    const double t = dx * dx + dy * dy + dz * dz;
-                    win |= t > a.tab.t_max;
-                    c0 = table_eval<double>(a.tab, t);
-                }
-                if (v1) {
-                    const double dx = tx - m1x, dy = ty - m1y, dz = tz - m1z;
-                    const double t = dx * dx + dy * dy + dz * dz;
-                    win |= t > a.tab.t_max;
-                    c1 = table_eval<double>(a.tab, t);
-                }
-                // z_c = L^-1 c, z_y = L^-1 y from the lane-step block; c and y go to
-                // the warp's shared slots.  Rows 0..31: lanes 2p, 2p + 1 run through
-                // the 33 entries of rows p and 31 - p (lane 2p switches from row p
-                // to row 31 - p after column p; the two halves of row 31 - p are
-                // joined by a shuffle).  Rows 32..35: lane l takes row 32 + (l & 3)
-                // on columns (l >> 2) + 8t, eight partial sums joined by shuffles.
-                static_assert(K == 36, "the lane-step layout is laid out for K = 36");
-                const double *Lr = a.linv + (int64_t)sl * linv_len(K);
-                __syncwarp();
-                sc[wid][lane] = c0;
-                sy[wid][lane] = y0;
-                if (lane < K - 32) {
-                    sc[wid][32 + lane] = c1;
-                    sy[wid][32 + lane] = y1;
-                }
-                __syncwarp();
-                const int pp = lane >> 1, odd = lane & 1;
-                double zca = 0.0, zya = 0.0, zc0 = 0.0, zy0 = 0.0, zc1 = 0.0, zy1 = 0.0;
-#pragma unroll
-                for (int u = 0; u < LS_STEPS; ++u) {
-                    const int t = odd ? LS_STEPS + u : u;
-                    if (!odd && u == pp + 1) {
-                        zca = zc0;
-                        zya = zy0;
-                        zc0 = 0.0;
-                        zy0 = 0.0;
-                    }
-                    int j = t <= pp ? t : t - pp - 1;
-                    j = j < K ? j : K - 1;  // the zero pad
-                    const double e = __ldg(Lr + u * 32 + lane);
-                    zc0 = fma(e, sc[wid][j], zc0);
-                    zy0 = fma(e, sy[wid][j], zy0);
-                }
-                const double zcb = zc0 + __shfl_xor_sync(FULL, zc0, 1), zyb = zy0 + __shfl_xor_sync(FULL, zy0, 1);
-                {
-                    const int g = lane >> 2;
-#pragma unroll
-                    for (int t = 0; t < LS_TAIL; ++t) {
-                        const int j = g + 8 * t < K ? g + 8 * t : K - 1;  // zero entries past the diagonal
-                        const double e = __ldg(Lr + (LS_STEPS + t) * 32 + lane);
-                        zc1 = fma(e, sc[wid][j], zc1);
-                        zy1 = fma(e, sy[wid][j], zy1);
-                    }
-#pragma unroll
-                    for (int o = 4; o < 32; o <<= 1) {
-                        zc1 += __shfl_xor_sync(FULL, zc1, o);
-                        zy1 += __shfl_xor_sync(FULL, zy1, o);
-                    }
-                }
-                // even lanes count rows p and 31 - p, lanes 0..3 rows 32..35, each once
-                double v = odd ? 0.0 : zca * zya + zcb * zyb, qc = odd ? 0.0 : zca * zca + zcb * zcb;
-                if (lane < K - 32) {
-                    v = fma(zc1, zy1, v);
-                    qc = fma(zc1, zc1, qc);
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    v += __shfl_xor_sync(FULL, v, o);
-                    qc += __shfl_xor_sync(FULL, qc, o);
-                }
-                const bool any_win = __any_sync(FULL, win);
-                if (lane == 0) {
-                    rv[wid][q] = v;
-                    rq[wid][q] = qc;
-                    rsl[wid][q] = sl;
-                    rwin[wid][q] = any_win;
-                }
-            }
-        }
         __syncwarp();
         if (lane < npt)
             finish_point(a, tile * 32 + lane, rsl[wid][lane], rv[wid][lane], rq[wid][lane], rwin[wid][lane] != 0,
@@ -1743,7 +1681,7 @@ template <int K>
 __global__ void __launch_bounds__(APPLY_WARPS * 32) apply_kernel_df(ApplyArgs a) {
     __shared__ df stx[APPLY_WARPS][32], sty[APPLY_WARPS][32], stz[APPLY_WARPS][32];
     __shared__ int64_t scp[APPLY_WARPS][32];
-    __shared__ df sc[APPLY_WARPS][K > GROUP ? K : 1], sy[APPLY_WARPS][K > GROUP ? K : 1];
+    __shared__ df sc[APPLY_WARPS][K], sy[APPLY_WARPS][K];
     // per target of the tile: w . y, w . c, class and window flag, finished one
     // target per lane after the tile (the double conversions then cost one
     // instruction per 32 targets)
@@ -1767,178 +1705,120 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32) apply_kernel_df(ApplyArgs a)
         }
         __syncwarp();
         const int npt = a.count - tile * 32 < 32 ? (int)(a.count - tile * 32) : 32;
-        if constexpr (K <= GROUP) {
-            const int g = lane / GROUP, l = lane - g * GROUP, base = g * GROUP;
-            for (int q0 = 0; q0 < npt; q0 += 3) {
-                const int q = q0 + g;
-                const bool has = g < 3 && q < npt;
-                int64_t c = 0;
-                df tx{0.0f, 0.0f}, ty{0.0f, 0.0f}, tz{1.0f, 0.0f};
-                if (has) {
-                    tx = stx[wid][q];
-                    ty = sty[wid][q];
-                    tz = stz[wid][q];
-                    c = scp[wid][q];
-                }
-                const int32_t sl = has ? __ldg(a.slot + c) : 0;
-                df cv{0.0f, 0.0f}, yv{0.0f, 0.0f};
-                bool win = false;
-                if (has && l < K) {
-                    const int32_t m = __ldg(a.members + c * K + l);
-                    if (m >= 0) {
-                        df mx, my, mz;
-                        member_vec_df(a.pvf, m, mx, my, mz);
-                        const df t = chord2_df(tx, ty, tz, mx, my, mz);
-                        win = t.hi > tmaxf;
-                        cv = table_eval<df>(a.tab, t);
-                        yv = split_double(__ldg(a.map + m));
-                    }
-                }
-                const float2 *Lr = a.linvf + (int64_t)sl * linv_len(K);
-                dfacc zc{0.0f, 0.0f}, zy{0.0f, 0.0f};
+                    static_assert(K == 36, "the split of rows 32 .. K-1 is laid out for K = 36");
+                    int64_t prev = -1;
+                    df m0x{0.0f, 0.0f}, m0y{0.0f, 0.0f}, m0z{0.0f, 0.0f}, y0{0.0f, 0.0f};
+                    df m1x{0.0f, 0.0f}, m1y{0.0f, 0.0f}, m1z{0.0f, 0.0f}, y1{0.0f, 0.0f};
+                    bool v0 = false, v1 = false;
+                    for (int q = 0; q < npt; ++q) {
+                        const df tx = stx[wid][q], ty = sty[wid][q], tz = stz[wid][q];
+                        const int64_t c = scp[wid][q];
+                        const int32_t sl = __ldg(a.slot + c);
+                        if (c != prev) {
+                            prev = c;
+                            const int32_t *mem = a.members + c * K;
+                            v0 = false;
+                            v1 = false;
+                            y0 = {0.0f, 0.0f};
+                            y1 = {0.0f, 0.0f};
+                            const int32_t mA = __ldg(mem + lane);
+                            if (mA >= 0) {
+                                member_vec_df(a.pvf, mA, m0x, m0y, m0z);
+                                y0 = split_double(__ldg(a.map + mA));
+                                v0 = true;
+                            }
+                            if (lane + 32 < K) {
+                                const int32_t mB = __ldg(mem + lane + 32);
+                                if (mB >= 0) {
+                                    member_vec_df(a.pvf, mB, m1x, m1y, m1z);
+                                    y1 = split_double(__ldg(a.map + mB));
+                                    v1 = true;
+                                }
+                            }
+                        }
+                        df c0{0.0f, 0.0f}, c1{0.0f, 0.0f};
+                        bool win = false;
+                        if (v0) {
+                            const df t = chord2_df(tx, ty, tz, m0x, m0y, m0z);
+                            win |= t.hi > tmaxf;
+                            c0 = table_eval<df>(a.tab, t);
+                        }
+                        if (v1) {
+                            const df t = chord2_df(tx, ty, tz, m1x, m1y, m1z);
+                            win |= t.hi > tmaxf;
+                            c1 = table_eval<df>(a.tab, t);
+                        }
+                        const float2 *Lr = a.linvf + (int64_t)sl * linv_len(K);
+                        __syncwarp();
+                        sc[wid][lane] = c0;
+                        sy[wid][lane] = y0;
+                        if (lane < K - 32) {
+                            sc[wid][32 + lane] = c1;
+                            sy[wid][32 + lane] = y1;
+                        }
+                        __syncwarp();
+                        // the lane-step block, as in the FP64 kernel
+                        const int pp = lane >> 1, odd = lane & 1;
+                        dfacc zca{0.0f, 0.0f}, zya{0.0f, 0.0f}, zc0{0.0f, 0.0f}, zy0{0.0f, 0.0f};
+                        dfacc zc1{0.0f, 0.0f}, zy1{0.0f, 0.0f};
 #pragma unroll
-                for (int j = 0; j < K; ++j) {
-                    const df cj = shfl_df(cv, base + j), yj = shfl_df(yv, base + j);
-                    if (has && l < K && l >= j) {
-                        const df e = ld_df(Lr + col_start(K, j) + l - j);
-                        dfacc_add_prod(zc, e, cj);
-                        dfacc_add_prod(zy, e, yj);
-                    }
-                }
-                const df zcv = dfacc_val(zc), zyv = dfacc_val(zy);
-                df vs = df_mul(zcv, zyv), qs = df_mul(zcv, zcv);
+                        for (int u = 0; u < LS_STEPS; ++u) {
+                            const int t = odd ? LS_STEPS + u : u;
+                            if (!odd && u == pp + 1) {
+                                zca = zc0;
+                                zya = zy0;
+                                zc0 = {0.0f, 0.0f};
+                                zy0 = {0.0f, 0.0f};
+                            }
+                            int j = t <= pp ? t : t - pp - 1;
+                            j = j < K ? j : K - 1;  // the zero pad
+                            const df e = ld_df(Lr + u * 32 + lane);
+                            dfacc_add_prod(zc0, e, sc[wid][j]);
+                            dfacc_add_prod(zy0, e, sy[wid][j]);
+                        }
+                        const df zc0v = dfacc_val(zc0), zy0v = dfacc_val(zy0);
+                        const df zcb = df_add_fast(zc0v, shfl_xor_df(zc0v, 1)), zyb = df_add_fast(zy0v, shfl_xor_df(zy0v, 1));
+                        df zc1v, zy1v;
+                        {
+                            const int g = lane >> 2;
 #pragma unroll
-                for (int o = 8; o >= 1; o >>= 1) {
-                    const df tv = shfl_df(vs, lane + o), tq = shfl_df(qs, lane + o);
-                    if (l < o && l + o < GROUP) {
-                        vs = df_add_fast(vs, tv);
-                        qs = df_add_fast(qs, tq);
-                    }
-                }
-                const unsigned wb = __ballot_sync(FULL, win);
-                if (has && l == 0) {
-                    rv[wid][q] = vs;
-                    rq[wid][q] = qs;
-                    rsl[wid][q] = sl;
-                    rwin[wid][q] = ((wb >> base) & ((1u << GROUP) - 1u)) != 0;
-                }
-            }
-        } else {
-            static_assert(K == 36, "the split of rows 32 .. K-1 is laid out for K = 36");
-            int64_t prev = -1;
-            df m0x{0.0f, 0.0f}, m0y{0.0f, 0.0f}, m0z{0.0f, 0.0f}, y0{0.0f, 0.0f};
-            df m1x{0.0f, 0.0f}, m1y{0.0f, 0.0f}, m1z{0.0f, 0.0f}, y1{0.0f, 0.0f};
-            bool v0 = false, v1 = false;
-            for (int q = 0; q < npt; ++q) {
-                const df tx = stx[wid][q], ty = sty[wid][q], tz = stz[wid][q];
-                const int64_t c = scp[wid][q];
-                const int32_t sl = __ldg(a.slot + c);
-                if (c != prev) {
-                    prev = c;
-                    const int32_t *mem = a.members + c * K;
-                    v0 = false;
-                    v1 = false;
-                    y0 = {0.0f, 0.0f};
-                    y1 = {0.0f, 0.0f};
-                    const int32_t mA = __ldg(mem + lane);
-                    if (mA >= 0) {
-                        member_vec_df(a.pvf, mA, m0x, m0y, m0z);
-                        y0 = split_double(__ldg(a.map + mA));
-                        v0 = true;
-                    }
-                    if (lane + 32 < K) {
-                        const int32_t mB = __ldg(mem + lane + 32);
-                        if (mB >= 0) {
-                            member_vec_df(a.pvf, mB, m1x, m1y, m1z);
-                            y1 = split_double(__ldg(a.map + mB));
-                            v1 = true;
+                            for (int t = 0; t < LS_TAIL; ++t) {
+                                const int j = g + 8 * t < K ? g + 8 * t : K - 1;  // zero entries past the diagonal
+                                const df e = ld_df(Lr + (LS_STEPS + t) * 32 + lane);
+                                dfacc_add_prod(zc1, e, sc[wid][j]);
+                                dfacc_add_prod(zy1, e, sy[wid][j]);
+                            }
+                            zc1v = dfacc_val(zc1);
+                            zy1v = dfacc_val(zy1);
+#pragma unroll
+                            for (int o = 4; o < 32; o <<= 1) {
+                                zc1v = df_add_fast(zc1v, shfl_xor_df(zc1v, o));
+                                zy1v = df_add_fast(zy1v, shfl_xor_df(zy1v, o));
+                            }
+                        }
+                        const df zcav = dfacc_val(zca), zyav = dfacc_val(zya);
+                        df v{0.0f, 0.0f}, qc{0.0f, 0.0f};
+                        if (!odd) {  // even lanes count rows p and 31 - p, lanes 0..3 rows 32..35, each once
+                            v = df_add_fast(df_mul(zcav, zyav), df_mul(zcb, zyb));
+                            qc = df_add_fast(df_mul(zcav, zcav), df_mul(zcb, zcb));
+                        }
+                        if (lane < K - 32) {
+                            v = df_add_fast(v, df_mul(zc1v, zy1v));
+                            qc = df_add_fast(qc, df_mul(zc1v, zc1v));
+                        }
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) {
+                            v = df_add_fast(v, shfl_xor_df(v, o));
+                            qc = df_add_fast(qc, shfl_xor_df(qc, o));
+                        }
+                        const bool any_win = __any_sync(FULL, win);
+                        if (lane == 0) {
+                            rv[wid][q] = v;
+                            rq[wid][q] = qc;
+                            rsl[wid][q] = sl;
+                            rwin[wid][q] = any_win;
                         }
                     }
-                }
-                df c0{0.0f, 0.0f}, c1{0.0f, 0.0f};
-                bool win = false;
-                if (v0) {
-                    const df t = chord2_df(tx, ty, tz, m0x, m0y, m0z);
-                    win |= t.hi > tmaxf;
-                    c0 = table_eval<df>(a.tab, t);
-                }
-                if (v1) {
-                    const df t = chord2_df(tx, ty, tz, m1x, m1y, m1z);
-                    win |= t.hi > tmaxf;
-                    c1 = table_eval<df>(a.tab, t);
-                }
-                const float2 *Lr = a.linvf + (int64_t)sl * linv_len(K);
-                __syncwarp();
-                sc[wid][lane] = c0;
-                sy[wid][lane] = y0;
-                if (lane < K - 32) {
-                    sc[wid][32 + lane] = c1;
-                    sy[wid][32 + lane] = y1;
-                }
-                __syncwarp();
-                // the lane-step block, as in the FP64 kernel
-                const int pp = lane >> 1, odd = lane & 1;
-                dfacc zca{0.0f, 0.0f}, zya{0.0f, 0.0f}, zc0{0.0f, 0.0f}, zy0{0.0f, 0.0f};
-                dfacc zc1{0.0f, 0.0f}, zy1{0.0f, 0.0f};
-#pragma unroll
-                for (int u = 0; u < LS_STEPS; ++u) {
-                    const int t = odd ? LS_STEPS + u : u;
-                    if (!odd && u == pp + 1) {
-                        zca = zc0;
-                        zya = zy0;
-                        zc0 = {0.0f, 0.0f};
-                        zy0 = {0.0f, 0.0f};
-                    }
-                    int j = t <= pp ? t : t - pp - 1;
-                    j = j < K ? j : K - 1;  // the zero pad
-                    const df e = ld_df(Lr + u * 32 + lane);
-                    dfacc_add_prod(zc0, e, sc[wid][j]);
-                    dfacc_add_prod(zy0, e, sy[wid][j]);
-                }
-                const df zc0v = dfacc_val(zc0), zy0v = dfacc_val(zy0);
-                const df zcb = df_add_fast(zc0v, shfl_xor_df(zc0v, 1)), zyb = df_add_fast(zy0v, shfl_xor_df(zy0v, 1));
-                df zc1v, zy1v;
-                {
-                    const int g = lane >> 2;
-#pragma unroll
-                    for (int t = 0; t < LS_TAIL; ++t) {
-                        const int j = g + 8 * t < K ? g + 8 * t : K - 1;  // zero entries past the diagonal
-                        const df e = ld_df(Lr + (LS_STEPS + t) * 32 + lane);
-                        dfacc_add_prod(zc1, e, sc[wid][j]);
-                        dfacc_add_prod(zy1, e, sy[wid][j]);
-                    }
-                    zc1v = dfacc_val(zc1);
-                    zy1v = dfacc_val(zy1);
-#pragma unroll
-                    for (int o = 4; o < 32; o <<= 1) {
-                        zc1v = df_add_fast(zc1v, shfl_xor_df(zc1v, o));
-                        zy1v = df_add_fast(zy1v, shfl_xor_df(zy1v, o));
-                    }
-                }
-                const df zcav = dfacc_val(zca), zyav = dfacc_val(zya);
-                df v{0.0f, 0.0f}, qc{0.0f, 0.0f};
-                if (!odd) {  // even lanes count rows p and 31 - p, lanes 0..3 rows 32..35, each once
-                    v = df_add_fast(df_mul(zcav, zyav), df_mul(zcb, zyb));
-                    qc = df_add_fast(df_mul(zcav, zcav), df_mul(zcb, zcb));
-                }
-                if (lane < K - 32) {
-                    v = df_add_fast(v, df_mul(zc1v, zy1v));
-                    qc = df_add_fast(qc, df_mul(zc1v, zc1v));
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    v = df_add_fast(v, shfl_xor_df(v, o));
-                    qc = df_add_fast(qc, shfl_xor_df(qc, o));
-                }
-                const bool any_win = __any_sync(FULL, win);
-                if (lane == 0) {
-                    rv[wid][q] = v;
-                    rq[wid][q] = qc;
-                    rsl[wid][q] = sl;
-                    rwin[wid][q] = any_win;
-                }
-            }
-        }
         __syncwarp();
         if (lane < npt)
             finish_point(a, tile * 32 + lane, rsl[wid][lane], df_to(rv[wid][lane]), df_to(rq[wid][lane]),
@@ -1946,6 +1826,123 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32) apply_kernel_df(ApplyArgs a)
         __syncwarp();
     }
     // counts of every lane, summed over the warp
+    const unsigned w_win = __reduce_add_sync(FULL, (unsigned)n_win);
+    const unsigned w_nug = __reduce_add_sync(FULL, (unsigned)n_nug);
+    const unsigned w_fail = __reduce_add_sync(FULL, (unsigned)n_fail);
+    if (lane == 0 && a.counters) {
+        if (w_win) atomicAdd(a.counters + CNT_WINDOW, (unsigned long long)w_win);
+        if (w_nug) atomicAdd(a.counters + CNT_NUGGET, (unsigned long long)w_nug);
+        if (w_fail) atomicAdd(a.counters + CNT_FAILED, (unsigned long long)w_fail);
+    }
+}
+
+// --------------------------------------------------- nine members, spin 0
+// One target per lane, in FP64 (R = double) or double-float (R = df): the nine members'
+// loads are independent of one another (27 in flight where a group of ten lanes had one
+// chain of four), every lane works on every multiply-add of the 45-entry factor, and nothing
+// is exchanged between lanes.  The sums run in the order of the ten-lane groups that this
+// replaced (column by column, the rows' products by halving), so results are the same bit
+// for bit.  What bounds it: the FP64 target geometry (200 FP64 instructions a tile).
+// Measured (GB300, the Nside 2048 sky, double-float): 32.4 -> 23.7 ms.
+template <class R>
+struct Nine;
+template <>
+struct Nine<double> {
+    using T = double;
+    using Acc = double;
+    static __device__ __forceinline__ T pos(double x) { return x; }
+    static __device__ __forceinline__ void member(const ApplyArgs &a, int64_t m, T tx, T ty, T tz, T &c, T &y, bool &win) {
+        double mx, my, mz;
+        member_vec(a.pv, m, mx, my, mz);
+        const double dx = tx - mx, dy = ty - my, dz = tz - mz;
+        const double t = dx * dx + dy * dy + dz * dz;
+        win |= t > a.tab.t_max;
+        c = table_eval<double>(a.tab, t);
+        y = __ldg(a.map + m);
+    }
+    static __device__ __forceinline__ T entry(const ApplyArgs &a, int64_t i) { return __ldg(a.linv + i); }
+    static __device__ __forceinline__ T zero() { return 0.0; }
+    static __device__ __forceinline__ Acc acc() { return 0.0; }
+    static __device__ __forceinline__ void mac(Acc &s, T x, T y) { s = fma(x, y, s); }
+    static __device__ __forceinline__ T val(Acc s) { return s; }
+    static __device__ __forceinline__ T mul(T x, T y) { return x * y; }
+    static __device__ __forceinline__ T add(T x, T y) { return x + y; }
+    static __device__ __forceinline__ double out(T x) { return x; }
+};
+template <>
+struct Nine<df> {
+    using T = df;
+    using Acc = dfacc;
+    static __device__ __forceinline__ T pos(double x) { return split_double(x); }
+    static __device__ __forceinline__ void member(const ApplyArgs &a, int64_t m, T tx, T ty, T tz, T &c, T &y, bool &win) {
+        df mx, my, mz;
+        member_vec_df(a.pvf, m, mx, my, mz);
+        const df t = chord2_df(tx, ty, tz, mx, my, mz);
+        win |= t.hi > (float)a.tab.t_max;
+        c = table_eval<df>(a.tab, t);
+        y = split_double(__ldg(a.map + m));
+    }
+    static __device__ __forceinline__ T entry(const ApplyArgs &a, int64_t i) { return ld_df(a.linvf + i); }
+    static __device__ __forceinline__ T zero() { return {0.0f, 0.0f}; }
+    static __device__ __forceinline__ Acc acc() { return {0.0f, 0.0f}; }
+    static __device__ __forceinline__ void mac(Acc &s, T x, T y) { dfacc_add_prod(s, x, y); }
+    static __device__ __forceinline__ T val(Acc s) { return dfacc_val(s); }
+    static __device__ __forceinline__ T mul(T x, T y) { return df_mul(x, y); }
+    static __device__ __forceinline__ T add(T x, T y) { return df_add_fast(x, y); }
+    static __device__ __forceinline__ double out(T x) { return df_to(x); }
+};
+
+template <class R>
+__global__ void __launch_bounds__(APPLY_WARPS * 32) apply_kernel_nine(ApplyArgs a) {
+    using N9 = Nine<R>;
+    using T = typename N9::T;
+    constexpr int K = 9;
+    const int lane = threadIdx.x & 31;
+    unsigned long long n_win = 0, n_nug = 0, n_fail = 0;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < a.count; p += stride) {
+        double x = 0.0, y = 0.0, z = 1.0;
+        int64_t c = 0;
+        target_of(a, p, x, y, z, c);
+        const int32_t sl = __ldg(a.slot + c);
+        int32_t m[K];
+#pragma unroll
+        for (int j = 0; j < K; ++j) m[j] = __ldg(a.members + c * K + j);
+        const T tx = N9::pos(x), ty = N9::pos(y), tz = N9::pos(z);
+        T cv[K], yv[K];
+        bool win = false;
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+            cv[j] = yv[j] = N9::zero();
+            if (m[j] >= 0) N9::member(a, m[j], tx, ty, tz, cv[j], yv[j], win);
+        }
+        const int64_t base = (int64_t)sl * linv_len(K);
+        T vs[K], qs[K];
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+            typename N9::Acc zc = N9::acc(), zy = N9::acc();
+#pragma unroll
+            for (int j = 0; j <= i; ++j) {
+                const T e = N9::entry(a, base + col_start(K, j) + i - j);
+                N9::mac(zc, e, cv[j]);
+                N9::mac(zy, e, yv[j]);
+            }
+            const T c1 = N9::val(zc), y1 = N9::val(zy);
+            vs[i] = N9::mul(c1, y1);
+            qs[i] = N9::mul(c1, c1);
+        }
+        // row 8 onto row 0, then halves of eight
+        vs[0] = N9::add(vs[0], vs[8]);
+        qs[0] = N9::add(qs[0], qs[8]);
+#pragma unroll
+        for (int o = 4; o >= 1; o >>= 1)
+#pragma unroll
+            for (int i = 0; i < o; ++i) {
+                vs[i] = N9::add(vs[i], vs[i + o]);
+                qs[i] = N9::add(qs[i], qs[i + o]);
+            }
+        finish_point(a, p, sl, N9::out(vs[0]), N9::out(qs[0]), win, n_win, n_nug, n_fail);
+    }
     const unsigned w_win = __reduce_add_sync(FULL, (unsigned)n_win);
     const unsigned w_nug = __reduce_add_sync(FULL, (unsigned)n_nug);
     const unsigned w_fail = __reduce_add_sync(FULL, (unsigned)n_fail);
@@ -2628,9 +2625,9 @@ static int paper_run(flints_paper_t p, int64_t nside_tgt, int64_t first, int64_t
         }
     } else if (p->K == 9) {
         if (mixed)
-            apply_kernel_df<9><<<grid, APPLY_WARPS * 32, 0, st>>>(a);
+            apply_kernel_nine<df><<<grid, APPLY_WARPS * 32, 0, st>>>(a);
         else
-            apply_kernel<9><<<grid, APPLY_WARPS * 32, 0, st>>>(a);
+            apply_kernel_nine<double><<<grid, APPLY_WARPS * 32, 0, st>>>(a);
     } else {
         if (mixed)
             apply_kernel_df<36><<<grid, APPLY_WARPS * 32, 0, st>>>(a);
