@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(256, 2) batch_kernel(const BatchHeader *__rest
             if (J[mid].tile_begin <= (int64_t)t) lo = mid;
             else hi = mid - 1;
         }
-        const LensArgs a = J[lo].a;
+        const LensArgs &a = J[lo].a;
         process_tile<K, SPIN, MIXED>(a, J[lo].R_rings, (int64_t)t - J[lo].tile_begin, tile_pts, wbase, lane, ctr);
         flush_counters(ctr, a.counters, lane);
         __syncwarp();

@@ -5,9 +5,10 @@
 //   1. stencil search: the rings whose circle comes within the search radius r
 //      of n' (one ring per lane), the pixel range of each ring that can lie
 //      inside the disc, candidates enumerated in increasing RING index;
-//   2. exact K-nearest selection: FP32 keys of all candidates pre-select, FP64
-//      squared chords of the selected (or near-tied) ones decide, warp bitonic
-//      sorts on (chord^2, RING index); the K-th chord must lie inside the disc;
+//   2. exact K-nearest selection: a threshold with K of the candidates' FP32 keys
+//      below it pre-selects, FP64 squared chords of the selected (or near-tied)
+//      ones decide, warp bitonic sorts on (chord^2, RING index); the K-th chord
+//      must lie inside the disc;
 //   3. covariance assembly S_ij = xi(t_ij)/xi(0) (+ nugget on the diagonal)
 //      and c_i = xi(t_i)/xi(0), spin 2 with the parallel-transport phase
 //      exp(2i(a_ij - a_ji)); lower triangle spread over the lanes;
@@ -776,8 +777,8 @@ __device__ __forceinline__ bool factor_bordered(Elem *mat, int lane) {
 // products together).  The low words' product is dropped: at most 2^-56 a term and
 // without bias, 2^-58 rms, where FP64 rounds every term of these sums, which are near 1,
 // to 2^-54; where a word meets itself (pivots, the variance) its mean is put back.
-// Measured (GB300): 1,048,583 spin-0 targets (K = 32, Nside 2048) 52.4 -> 27.8 ms; 524,309
-// Q/U targets (K = 32, Nside 4096) 61.2 -> 26.9 ms.
+// Measured (GB300): 1,048,583 spin-0 targets (K = 32, Nside 2048) 52.4 -> 23.6 ms; 524,309
+// Q/U targets (K = 32, Nside 4096) 61.2 -> 24.0 ms.
 // Returns false when a pivot of S + nugget I is not positive.
 constexpr int FXB = 59;
 
@@ -1514,6 +1515,38 @@ __device__ __forceinline__ bool solve_any(SM &sm, const PointA &P, int lane, dou
         return solve_point<K, SPIN, R>(sm, P, lane, nugget, a.tab, keyd, yre, yim, vre, vim, vrel);
 }
 
+// FP64 solve of target q of the tile with the nugget rule of Sec. 2.4: points that the
+// kernel's own form declined.  Out of line: inlined, its registers and instructions weighed
+// on every point (FP64 kernels spilled 340 bytes and stalled on instruction fetch).
+template <int RPL>
+struct Rows {
+    double keyd[RPL], yre[RPL], yim[RPL];
+};
+struct Solved {
+    double re, im, var;
+    int flags;
+};
+template <int K, int SPIN, class SM>
+__device__ __attribute__((noinline)) Solved solve_fp64(SM &sm, int q, int lane, const LensArgs &a,
+                                                       Rows<Shape<K>::RPL> rows) {
+    Solved f;
+    f.re = f.im = f.var = __longlong_as_double(0x7ff8000000000000ll);
+    f.flags = 0;
+    double nug = NUGGET_EPS;
+    for (int step = 0; step <= MAX_NUGGET_STEPS; ++step) {
+        if (step > 0) {
+            nug *= 2.0;
+            f.flags |= FLINTS_ST_NUGGET;
+        }
+        const bool ok = solve_any<K, SPIN, double>(sm, sm.pts[q], lane, nug, a, rows.keyd, rows.yre, rows.yim, f.re, f.im, f.var);
+        __syncwarp();
+        if (ok) return f;
+    }
+    f.re = f.im = f.var = __longlong_as_double(0x7ff8000000000000ll);
+    f.flags |= FLINTS_ST_FAILED;
+    return f;
+}
+
 // ------------------------------------------------------------------ kernel
 struct Counters {
     unsigned long long nug = 0, fb = 0, win = 0, fail = 0;
@@ -1728,13 +1761,12 @@ __device__ __forceinline__ void process_tile(const LensArgs &a, int R_rings, int
         unsigned long long key[RPL];
         unsigned id[RPL];
         if (!fail) {
-            // 1. FP32 keys of all candidates, packed with the candidate id (ids follow
-            //    the RING index, so equal keys order by pixel), one sort
-            unsigned long long pk[SPL];
+            // 1. FP32 keys of all candidates (ids follow the RING index)
+            unsigned k32[SPL];
 #pragma unroll
             for (int s = 0; s < SPL; ++s) {
                 const int c = s * 32 + lane;
-                pk[s] = ~0ull;
+                k32[s] = ~0u;
                 if (c < C) {
                     int lo = 0, hi = 31;  // ring holding candidate c: first r with end > c
                     while (lo < hi) {
@@ -1750,17 +1782,53 @@ __device__ __forceinline__ void process_tile(const LensArgs &a, int R_rings, int
                     if (dj > rr.n_in / 2) dj -= rr.n_in;
                     if (dj < -(rr.n_in / 2)) dj += rr.n_in;
                     const float sn = sinpif(((float)dj + rr.frac) * rr.inv_n);
-                    const float k32 = fmaf(rr.b32, sn * sn, rr.a32);
                     sm.u.cand.cpix[c] = ((uint32_t)lo << 24) | (uint32_t)jj;
-                    pk[s] = ((unsigned long long)__float_as_uint(fmaxf(k32, 0.0f)) << 32) | (unsigned)c;
+                    k32[s] = __float_as_uint(fmaxf(fmaf(rr.b32, sn * sn, rr.a32), 0.0f));
                 }
             }
-            bitonic_sort_packed<SPL>(pk, lane);
-            // 2. exact set unless the K-th and (K+1)-th FP32 keys are within 2^-16
-            const unsigned long long ka = __shfl_sync(FULL, pk[(K - 1) >> 5], (K - 1) & 31);
-            const unsigned long long kb = __shfl_sync(FULL, pk[K >> 5], K & 31);
-            const float fa = __uint_as_float((unsigned)(ka >> 32)), fb = __uint_as_float((unsigned)(kb >> 32));
-            const bool exact = (C == K) || (fb - fa > fb * 1.52587890625e-05f);
+            // 2. the set is exact when some threshold has K FP32 keys below it and the keys on its
+            //    two sides are more than 2^-16 apart; only its members matter here (the FP64 keys
+            //    order them), so no sort.  Squared chords have K of the candidates below about
+            //    r^2 / 1.25^2 and are spaced evenly around there (equal-area pixels): steps of one
+            //    spacing per missing key, bisection where they leave the bracket.  Two or three
+            //    counts instead of the 28 stages (128 slots) of a sort; where eight do not do
+            //    (equal keys at the K-th place) the keys are sorted.  Measured (GB300, 2.1 M spin-0
+            //    targets, K = 32, mixed): 44.1 -> 40.1 ms, with the FP64 solve out of line.
+            unsigned sel = ~0u;  // keys up to here are selected
+            bool exact = C == K;
+            if (!exact) {
+                const float mid = 0.64f * (float)a.r2, gap = mid / (float)K;
+                float lo = 0.0f, hi = 4.0f * mid, x = mid;
+                int n = -1;
+#pragma unroll 1
+                for (int it = 0; it < 8; ++it) {
+                    sel = __float_as_uint(x);
+                    n = 0;
+#pragma unroll
+                    for (int s = 0; s < SPL; ++s) n += __popc(__ballot_sync(FULL, k32[s] <= sel));
+                    if (n == K) break;
+                    if (n < K) lo = x;
+                    else hi = x;
+                    const float step = x + (float)(K - n) * gap;
+                    x = step > lo && step < hi ? step : 0.5f * (lo + hi);
+                }
+                if (n == K) {
+                    unsigned below = 0, above = ~0u;
+#pragma unroll
+                    for (int s = 0; s < SPL; ++s) {
+                        if (k32[s] <= sel) below = k32[s] > below ? k32[s] : below;
+                        else above = k32[s] < above ? k32[s] : above;
+                    }
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) {
+                        const unsigned b2 = __shfl_xor_sync(FULL, below, o), a2 = __shfl_xor_sync(FULL, above, o);
+                        below = b2 > below ? b2 : below;
+                        above = a2 < above ? a2 : above;
+                    }
+                    const float fa = __uint_as_float(below), fb = __uint_as_float(above);
+                    exact = fb - fa > fb * 1.52587890625e-05f;
+                }
+            }
             __syncwarp();
             // 3. FP64 positions and keys: of the K selected (fast) or of all candidates
             auto place = [&](int c) -> unsigned long long {
@@ -1779,12 +1847,24 @@ __device__ __forceinline__ void process_tile(const LensArgs &a, int R_rings, int
                 return (unsigned long long)__double_as_longlong(ex * ex + ey * ey + ez * ez);
             };
             if (exact) {
+                // the selected ids, packed over the lanes (ktf is free until the neighbours are known)
+                int *ids = reinterpret_cast<int *>(sm.ktf);
+                int base = 0;
+#pragma unroll
+                for (int s = 0; s < SPL; ++s) {
+                    const int c = s * 32 + lane;
+                    const bool in = c < C && k32[s] <= sel;
+                    const unsigned b = __ballot_sync(FULL, in);
+                    if (in) ids[base + __popc(b & ((1u << lane) - 1u))] = c;
+                    base += __popc(b);
+                }
+                __syncwarp();
 #pragma unroll
                 for (int r = 0; r < RPL; ++r) {
                     key[r] = 0x7ff0000000000000ull;
                     id[r] = 0xffffffffu;
                     if (lane + 32 * r < K) {
-                        const unsigned c = (unsigned)(pk[r] & 0xffffffffu);
+                        const unsigned c = (unsigned)ids[lane + 32 * r];
                         key[r] = place((int)c);
                         id[r] = c;
                     }
@@ -1792,6 +1872,12 @@ __device__ __forceinline__ void process_tile(const LensArgs &a, int R_rings, int
                 __syncwarp();
                 bitonic_sort<RPL>(key, id, lane);
             } else {
+                unsigned long long pk[SPL];
+#pragma unroll
+                for (int s = 0; s < SPL; ++s)
+                    pk[s] = k32[s] == ~0u ? ~0ull : ((unsigned long long)k32[s] << 32) | (unsigned)(s * 32 + lane);
+                bitonic_sort_packed<SPL>(pk, lane);
+                const float fa = __uint_as_float((unsigned)(__shfl_sync(FULL, pk[(K - 1) >> 5], (K - 1) & 31) >> 32));
                 // Near-tie at the K-th place.  A candidate whose FP32 key exceeds the
                 // K-th one by more than the margin is farther than the true K-th
                 // neighbour (FP32 keys are within 2^-17 relative), so FP64 keys are
@@ -1962,18 +2048,19 @@ __device__ __forceinline__ void process_tile(const LensArgs &a, int R_rings, int
                     if (!solved) fx_restore<K>(sm, lane, a.two_r);
                 }
             }
-            double nug = NUGGET_EPS;
-            for (int step = 0; !solved && step <= MAX_NUGGET_STEPS; ++step) {
-                if (step > 0) {
-                    nug *= 2.0;
-                    flags |= FLINTS_ST_NUGGET;
-                }
-                solved = solve_any<K, SPIN, double>(sm, P, lane, nug, a, keyd, yre, yim, vre, vim, vrel);
-                __syncwarp();
-            }
             if (!solved) {
-                flags |= FLINTS_ST_FAILED;
-                vre = vim = vrel = __longlong_as_double(0x7ff8000000000000ll);
+                Rows<RPL> rows;
+#pragma unroll
+                for (int r = 0; r < RPL; ++r) {
+                    rows.keyd[r] = keyd[r];
+                    rows.yre[r] = yre[r];
+                    rows.yim[r] = yim[r];
+                }
+                const Solved f = solve_fp64<K, SPIN>(sm, q, lane, a, rows);
+                flags |= f.flags;
+                vre = f.re;
+                vim = f.im;
+                vrel = f.var;
             }
         }
         if (lane == 0) {
