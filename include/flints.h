@@ -193,7 +193,7 @@ int flints_stencil(flints_plan_t plan, int64_t first, int64_t count,
  *   warps_per_block 1..8 (0: 8 for spin-0 and spin-2 plans, 4 for spin-1 and
  *   augmented ones; lowered to what fits in shared memory),
  *   blocks_per_sm cap (0: as many as fit),
- *   tile_points targets per warp tile 1..16 (0: 16).  cfg NULL restores the
+ *   tile_points targets per warp tile 1..16 (0: from the target count).  cfg NULL restores the
  *   defaults.  Results do not depend on the launch shape. */
 typedef struct {
     int warps_per_block, blocks_per_sm, tile_points;
@@ -220,9 +220,11 @@ int flints_lens_batch(const flints_job *jobs, int n, void *stream);
  *     max_jobs jobs, plus pinned host staging (allocates; not capturable).
  *   flints_batch_stage: host-only: validate the jobs, order them by precision
  *     class and decreasing estimated cost, cut them into tiles of tile_points
- *     targets (1..16; 0: 16), write the table into the pinned staging buffer.
+ *     targets (1..16; 0: chosen from the batch's target count), write the table
+ *     into the pinned staging buffer.
  *   flints_batch_launch: upload the staged table, reset the work queues and
- *     launch the two persistent kernels (FP64 and mixed jobs) on `stream`:
+ *     launch the persistent class kernels on `stream` and on streams of the
+ *     batch that are forked from it and joined to it by events:
  *     stream operations only, so it can be captured in a CUDA graph; a replay
  *     runs whatever table was staged last.  The warps_per_block of cfg must
  *     have been used by an earlier launch before capture (changing it
@@ -263,13 +265,14 @@ const char *flints_last_error(void);
  *   flints_synth_plan: ring geometry, work arrays (about (4 Nside - 1)(2 lmax + 1)
  *     + 2 Npix complex doubles) and the cuFFT plans for Nside (1..8192), lmax
  *     (spin..16384) and spin (0, 1, 2).  precision FLINTS_FP64: the l-recurrence
- *     in FP64; FLINTS_MIXED: in double-float on the FP32 pipe (relative error
- *     about 1e-13 at lmax 4096).  Allocates; not capturable.
+ *     in FP64; FLINTS_MIXED: in 64-bit fixed point on the integer pipe (error
+ *     about 2e-13 of the map at lmax 2048; 40 (spin 0) or 56 bytes more per
+ *     (l, m) for its tables).  Allocates; not capturable.
  *   flints_synthesize: alm (and blm for spin 1, 2; NULL = 0) DEVICE complex
  *     double [lmax+1][lmax+1] (index [l][m], m <= l read), 16-byte aligned;
  *     map DEVICE double [Npix] (spin 0) or [Npix][2] (spin 1, 2), RING order.
- *     Asynchronous on `stream`: an l-recurrence kernel, a folding kernel and
- *     one inverse FFT per ring size.
+ *     Asynchronous on `stream`: a weight kernel (FLINTS_MIXED), an l-recurrence
+ *     kernel, a folding kernel and one inverse FFT per ring size.
  * Errors: FLINTS_EINVAL (arguments), FLINTS_ENOMEM, FLINTS_ECUDA; the message
  * is returned by flints_synth_last_error. */
 typedef struct flints_synth_s *flints_synth_t;

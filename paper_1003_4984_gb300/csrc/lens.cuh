@@ -1762,11 +1762,11 @@ __device__ __forceinline__ void process_tile(const LensArgs &a, int R_rings, int
         unsigned id[RPL];
         if (!fail) {
             // 1. FP32 keys of all candidates (ids follow the RING index)
-            unsigned k32[SPL];
+            unsigned keys[SPL];
 #pragma unroll
             for (int s = 0; s < SPL; ++s) {
                 const int c = s * 32 + lane;
-                k32[s] = ~0u;
+                keys[s] = ~0u;
                 if (c < C) {
                     int lo = 0, hi = 31;  // ring holding candidate c: first r with end > c
                     while (lo < hi) {
@@ -1782,8 +1782,9 @@ __device__ __forceinline__ void process_tile(const LensArgs &a, int R_rings, int
                     if (dj > rr.n_in / 2) dj -= rr.n_in;
                     if (dj < -(rr.n_in / 2)) dj += rr.n_in;
                     const float sn = sinpif(((float)dj + rr.frac) * rr.inv_n);
+                    const float k32 = fmaf(rr.b32, sn * sn, rr.a32);
                     sm.u.cand.cpix[c] = ((uint32_t)lo << 24) | (uint32_t)jj;
-                    k32[s] = __float_as_uint(fmaxf(fmaf(rr.b32, sn * sn, rr.a32), 0.0f));
+                    keys[s] = __float_as_uint(fmaxf(k32, 0.0f));
                 }
             }
             // 2. the set is exact when some threshold has K FP32 keys below it and the keys on its
@@ -1805,7 +1806,7 @@ __device__ __forceinline__ void process_tile(const LensArgs &a, int R_rings, int
                     sel = __float_as_uint(x);
                     n = 0;
 #pragma unroll
-                    for (int s = 0; s < SPL; ++s) n += __popc(__ballot_sync(FULL, k32[s] <= sel));
+                    for (int s = 0; s < SPL; ++s) n += __popc(__ballot_sync(FULL, keys[s] <= sel));
                     if (n == K) break;
                     if (n < K) lo = x;
                     else hi = x;
@@ -1816,8 +1817,8 @@ __device__ __forceinline__ void process_tile(const LensArgs &a, int R_rings, int
                     unsigned below = 0, above = ~0u;
 #pragma unroll
                     for (int s = 0; s < SPL; ++s) {
-                        if (k32[s] <= sel) below = k32[s] > below ? k32[s] : below;
-                        else above = k32[s] < above ? k32[s] : above;
+                        if (keys[s] <= sel) below = keys[s] > below ? keys[s] : below;
+                        else above = keys[s] < above ? keys[s] : above;
                     }
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) {
@@ -1853,7 +1854,7 @@ __device__ __forceinline__ void process_tile(const LensArgs &a, int R_rings, int
 #pragma unroll
                 for (int s = 0; s < SPL; ++s) {
                     const int c = s * 32 + lane;
-                    const bool in = c < C && k32[s] <= sel;
+                    const bool in = c < C && keys[s] <= sel;
                     const unsigned b = __ballot_sync(FULL, in);
                     if (in) ids[base + __popc(b & ((1u << lane) - 1u))] = c;
                     base += __popc(b);
@@ -1875,7 +1876,7 @@ __device__ __forceinline__ void process_tile(const LensArgs &a, int R_rings, int
                 unsigned long long pk[SPL];
 #pragma unroll
                 for (int s = 0; s < SPL; ++s)
-                    pk[s] = k32[s] == ~0u ? ~0ull : ((unsigned long long)k32[s] << 32) | (unsigned)(s * 32 + lane);
+                    pk[s] = keys[s] == ~0u ? ~0ull : ((unsigned long long)keys[s] << 32) | (unsigned)(s * 32 + lane);
                 bitonic_sort_packed<SPL>(pk, lane);
                 const float fa = __uint_as_float((unsigned)(__shfl_sync(FULL, pk[(K - 1) >> 5], (K - 1) & 31) >> 32));
                 // Near-tie at the K-th place.  A candidate whose FP32 key exceeds the

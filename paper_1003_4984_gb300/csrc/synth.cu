@@ -51,8 +51,6 @@
 
 namespace {
 
-
-
 constexpr double PI_D = 3.14159265358979323846;
 
 struct SynthRing {
