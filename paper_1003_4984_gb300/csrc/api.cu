@@ -473,8 +473,10 @@ int flints_stencil(flints_plan_t p, int64_t first, int64_t count, const double *
 // stream each begins only when the slowest tile of the one before it has ended, and
 // that tail leaves most of the GPU idle once per class.  On several streams the next
 // kernel's blocks start as the blocks of the earlier ones leave.  Measured (GB300, 8
-// jobs of 15 to 105 thousand targets, 7 classes): 27.4 ms in one stream, 23.5 ms with the side streams and the tile rule of auto_tile_points.  Four streams in all: one
-// class's blocks already fill the GPU, so more of them would only queue.
+// jobs of 15 to 105 thousand targets, 7 classes): 27.4 ms in one stream, 23.5 ms
+// with the side streams and the tile rule of auto_tile_points (21.5 ms with the
+// FP64 classes in fixed point and the threshold selection).  Four streams in all:
+// one class's blocks already fill the GPU, so more of them would only queue.
 constexpr int BATCH_SIDE = 3;
 
 struct ClassStreams {

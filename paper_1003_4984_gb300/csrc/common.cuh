@@ -417,7 +417,7 @@ struct LaunchCfg {
 // tile holds.  The size with the shortest such launch is taken, the largest one on
 // ties; past 8 rounds of full tiles the tail is within a few percent and the size
 // stays at its maximum, which displaces the most targets per pass.  Measured
-// (GB300, full tiles -> this rule): 1,009 targets (spin 0, K = 16) 389 -> 49 us,
+// (GB300, full tiles -> this rule): 1,009 targets (spin 0, K = 16) 389 -> 51 us,
 // 20,011 targets (spin 2, K = 32) 1222 -> 721 us.
 inline int auto_tile_points(int64_t count, int64_t warps) {
     if (warps < 1 || count >= 8 * MAX_TILE_POINTS * warps) return MAX_TILE_POINTS;

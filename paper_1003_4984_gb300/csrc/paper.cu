@@ -20,8 +20,9 @@
 //      columns (column j, rows j .. K-1, contiguous: coalesced lane loads).
 // Per call (apply_kernel): one warp per tile of 32 targets.  Lane l displaces
 // target l and locates its coarse pixel (RING ang2pix at Nc); then per target
-// (three at a time in groups of 10 lanes for K = 9, one at a time for K = 36)
-// the lanes own stencil members l (and l + 32): c_l = xi(|n' - x_l|^2)/xi(0),
+// (three at a time in groups of 10 lanes for K = 9 at spin 2, one at a time for
+// K = 36; K = 9 at spin 0 keeps one target per lane, apply_kernel_nine, and FP64
+// plans at K = 36 use apply_kernel_fx where the grid allows) the lanes own stencil members l (and l + 32): c_l = xi(|n' - x_l|^2)/xi(0),
 // y_l = map[x_l]; lane i accumulates row i of z_c = L^-1 c and z_y = L^-1 y
 // (c_j, y_j broadcast by shuffles); value = z_c . z_y and variance
 // xi(0) (1 - z_c . z_c), the kriging estimate and its error (Eqs.
@@ -1208,7 +1209,7 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32) apply_kernel_aug(ApplyArgs a
 // the largest row of the target needs.
 // Member terms are formed for FX_G = 8 targets at a time, flattened over the lanes (288
 // terms, nine full passes; member by member a target needs two, the second with four
-// lanes).  Measured (GB300, 2,097,169 Q/U targets, Nside 1024): 40.5 -> 15.2 ms.
+// lanes).  Measured (GB300, 2,097,169 Q/U targets, Nside 1024): 40.5 -> 14.3 ms.
 constexpr int FX_G = 8, FX_K = 36, FXA = 58;  // FXA: units of c, y and their products, 2^-58
 
 constexpr int FX_FP64 = 1 << 20;

@@ -4,7 +4,8 @@ Counting convention (used for every roofline fraction reported by the bench):
 
 * a fused multiply-add counts 2 flops, any other add, subtract or multiply 1;
   square roots, reciprocals and the table index count 2 each;
-* FP64 path: the arithmetic of the method itself, per target point, with K
+* FP64 path (whatever executes it: FP64 plans solve in 64-bit fixed point, and
+  fall back to FP64 instructions): the arithmetic of the method itself, per target point, with K
   stencil members and P = K(K-1)/2 pairs:
     - left-looking Cholesky: (K^3 - K)/6 multiply-adds plus K pivots and P
       scalings; complex Hermitian (spin 2) multiply-adds are 4 real ones;
@@ -66,6 +67,9 @@ def mixed_fp32_flops(K: int, spin: int) -> float:
 # 152 SMs x 128 FP32 lanes x 2 flops x 2.07 GHz; FP64 at the 1.25 TFLOP/s nominal rate.
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12
 FP64_PEAK_TFLOPS = 1.25
+# method flops a 64-bit fixed-point solve could reach: a multiply-add (2 flops) is three
+# 32 x 32 -> 64 bit products, half-rate instructions (64 lanes per SM and cycle; 58 measured)
+FIXED_PEAK_TFLOPS = 152 * 64 / 3 * 2 * 2.070e9 / 1e12
 
 
 def augmented_flops(K: int, mixed: bool) -> float:
