@@ -470,6 +470,13 @@ __device__ __forceinline__ fx fx_split(int64_t v) {
     const uint32_t l = (uint32_t)v | 1u;
     return {(int)((uint32_t)((uint64_t)v >> 32) + (l >> 31)), (int)l};
 }
+// The pair of v with every bit kept, but for low words of -2^31 (one more unit there), which
+// could not be negated.
+__device__ __forceinline__ fx fx_split_all(int64_t v) {
+    uint32_t l = (uint32_t)v;
+    l += l == 0x80000000u;
+    return {(int)((uint32_t)((uint64_t)v >> 32) + (l >> 31)), (int)l};
+}
 __device__ __forceinline__ fx fx_neg(fx a) { return {(int)(0u - (unsigned)a.hi), (int)(0u - (unsigned)a.lo)}; }
 __device__ __forceinline__ uint64_t mul_wide(int a, int b) { return (uint64_t)((int64_t)a * (int64_t)b); }
 // s + a b in one instruction
