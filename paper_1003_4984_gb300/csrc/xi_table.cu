@@ -133,13 +133,12 @@ __global__ void normalise_kernel(double *f, double *g, int n, double xi0) {
     g[k] /= xi0;
 }
 
-// The interval coefficients in units of 2^-59 (all of them below 2 in size, see fixed_table_ok).
+// The interval coefficients rounded to units of 2^-59 (all of them below 2 in size, see fixed_table_ok).
 __global__ void fixed_table_kernel(const Coef64 *__restrict__ c64, int n, CoefFx *__restrict__ cfx) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
-    const double u = 576460752303423488.0;  // 2^59
     const Coef64 c = c64[k];
-    cfx[k] = CoefFx{(int64_t)(c.f * u), (int64_t)(c.m * u), (int64_t)(c.c2 * u), (int64_t)(c.c3 * u)};
+    cfx[k] = CoefFx{fx_of(c.f, 59), fx_of(c.m, 59), fx_of(c.c2, 59), fx_of(c.c3, 59)};
 }
 
 cudaError_t launch_xi_table(int spin, int lmax, const double *cl_dev, const double *clbb_dev, double t_max,
