@@ -523,6 +523,15 @@ __device__ __forceinline__ int64_t fx_of(double x, int sh) {
     const uint64_t v = p >= 0 ? m << (p & 15) : (p < -54 ? 0 : (m + ((uint64_t)1 << (-p - 1))) >> -p);
     return (b >> 63) ? -(int64_t)v : (int64_t)v;
 }
+// biased exponent of a data value, 0 for zeros only (subnormals, which fx_of drops, count as
+// the smallest normal): where the largest of a stencil is below DATA_EXPO_MIN they may weigh
+// more than 2^-55 of it, and the stencil takes an FP64 form
+constexpr int DATA_EXPO_MIN = 64;
+__device__ __forceinline__ int data_expo(double x) {
+    const uint64_t b = (uint64_t)__double_as_longlong(x) << 1;
+    const int e = (int)(b >> 53);
+    return e == 0 && b != 0 ? 1 : e;
+}
 __device__ __forceinline__ double fx_scale2(double x, int e) {  // x 2^e, |e| <= 2000, in two exact steps
     const int a = e / 2, c = e - a;
     return x * __longlong_as_double((long long)(1023 + a) << 52) * __longlong_as_double((long long)(1023 + c) << 52);

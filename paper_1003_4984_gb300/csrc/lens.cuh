@@ -1049,8 +1049,8 @@ __device__ __forceinline__ void phase_fx(fxc a, fxc b, int64_t q, int64_t tt, fx
 // offsets become integers in units of the disc's diameter (in place: gx, gy, gz, the
 // phases and tangent coordinates; fx_restore gives gx, gy, gz back), chords, table
 // lookups, pair phases, factor and final sums stay integers; FP64 serves the one phase
-// per neighbour.  False (nothing solved): a data value that is not finite, or a matrix
-// that is not safely positive.
+// per neighbour.  False (nothing solved): a data value that is not finite, data so small that
+// subnormal values count, or a matrix that is not safely positive.
 template <int K, int SPIN, class SM>
 __device__ bool solve_point_fixed(SM &sm, const PointA &P, int lane, const LensArgs &a,
                                   const double (&keyd)[Shape<K>::RPL], const double (&yre)[Shape<K>::RPL],
@@ -1080,8 +1080,7 @@ __device__ bool solve_point_fixed(SM &sm, const PointA &P, int lane, const LensA
         const int i = lane + 32 * r;
         tau[r] = 0;
         if (i < K) {
-            const int e0 = (int)((uint64_t)__double_as_longlong(yre[r]) >> 52 & 0x7ff);
-            const int e1 = SPIN == 0 ? 0 : (int)((uint64_t)__double_as_longlong(yim[r]) >> 52 & 0x7ff);
+            const int e0 = data_expo(yre[r]), e1 = SPIN == 0 ? 0 : data_expo(yim[r]);
             ymax = e0 > ymax ? e0 : ymax;
             ymax = e1 > ymax ? e1 : ymax;
             tau[r] = fx_of(keyd[r] * (a.inv_2r * a.inv_2r), 62);
@@ -1106,7 +1105,7 @@ __device__ bool solve_point_fixed(SM &sm, const PointA &P, int lane, const LensA
         ymax = v > ymax ? v : ymax;
     }
     __syncwarp();
-    if (ymax == 0x7ff) return false;
+    if (ymax == 0x7ff || (ymax > 0 && ymax < DATA_EXPO_MIN)) return false;
     int ey = ymax - 1022 + 4;  // |y| < 2^(ey - 4)
 
     const fx hr = fx_split(fx_of(0.5 * a.r2, 64)), r2 = fx_split(fx_of(a.r2, 62));
@@ -1202,8 +1201,8 @@ __device__ bool solve_point_fixed(SM &sm, const PointA &P, int lane, const LensA
         if constexpr (SPIN != 0) w += __shfl_xor_sync(FULL, w, o);
         n += __shfl_xor_sync(FULL, n, o);
     }
-    val_re = fx_scale2((double)v, ey - FXB);
-    val_im = SPIN == 0 ? 0.0 : fx_scale2((double)w, ey - FXB);
+    val_re = ymax == 0 ? 0.0 : fx_scale2((double)v, ey - FXB);  // no data but zeros: exactly 0
+    val_im = SPIN == 0 || ymax == 0 ? 0.0 : fx_scale2((double)w, ey - FXB);
     var_rel = (double)(((int64_t)1 << FXB) - n) * 1.734723475976807e-18;  // 2^-59
     return true;
 }
