@@ -835,8 +835,14 @@ __device__ __forceinline__ bool fx_beyond(int64_t v, int lim) {
 // data, scaled by its caller below 2^-4; its solve has no bound, and where an entry
 // passes 1/8 the row is shifted down by 3 bits (counted in ey) and the panel's slot redone:
 // the largest entry of the row keeps at least 53 bits.
-// With rows of at most unit length (|L_r| <= 1) a cross sum of n terms stays below
-// 2 sqrt(n) 2^58, with the data row below 2.3 sqrt(n) 2^58: no overflow up to n = 96 terms.
+// The sums here are taken modulo 32, and on a matrix that is not positive a row can be longer
+// than that before its own pivot says so.  A row's squared length is therefore also read from
+// the high words' sum, which holds 512 (n = 96 terms of at most 1.9^2 each are 347): beyond
+// FX_LEN the form declines.  (The three columns of its own panel add at most 21.7, which no
+// wrap turns into an accepted pivot.)  The caller does the same for the row of c, which has no
+// pivot.  With rows of at most that length a cross sum of n terms stays below 2.5 sqrt(n) 2^58,
+// with the data row too: no overflow up to n = 96.
+constexpr float FX_LEN = 1.5f;
 template <int N, int NB, class E>
 __device__ __forceinline__ bool factor_fixed(E *mat, int lane, int &ey) {
     constexpr bool CPLX = std::is_same<E, fxc>::value;
@@ -857,6 +863,7 @@ __device__ __forceinline__ bool factor_fixed(E *mat, int lane, int &ey) {
             const E *Lr = mat + tri<N>(act ? r : j0, 0);
             for (;;) {
                 int64_t vr[PW], vi[PW];
+                int len = 0;  // a pivot row's squared length so far, units of 2^-14
                 {
                     fxacc ar[PW], ai[PW];
 #pragma unroll
@@ -884,9 +891,11 @@ __device__ __forceinline__ bool factor_fixed(E *mat, int lane, int &ey) {
                     for (int c = 0; c < PW; ++c) {
                         vr[c] = fx_down<FXB>(ar[c]);
                         vi[c] = CPLX ? fx_down<FXB>(ai[c]) : 0;
+                        if (first && grp == c) len = (int)((int64_t)ar[c].hh >> (2 * FXB - 64 - 14));
                     }
                 }
                 for (int o = 1; o < s; o <<= 1) {
+                    if (first) len += __shfl_xor_sync(FULL, len, o);
 #pragma unroll
                     for (int c = 0; c < PW; ++c) {
                         vr[c] = fx_add(vr[c], __shfl_xor_sync(FULL, vr[c], o));
@@ -904,7 +913,7 @@ __device__ __forceinline__ bool factor_fixed(E *mat, int lane, int &ey) {
                     }
                 }
                 E l[PW];
-                bool bad = false, high = false;
+                bool bad = len > (int)(FX_LEN * 16384.0f), high = false;
 #pragma unroll
                 for (int c = 0; c < PW; ++c) {
                     if (first) {
@@ -1195,12 +1204,15 @@ __device__ bool solve_point_fixed(SM &sm, const PointA &P, int lane, const LensA
         }
     }
     int64_t v = fx_down<FXB>(sr), w = fx_down<FXB>(si), n = fx_down<FXB>(sn);
+    int len = (int)((int64_t)sn.hh >> (2 * FXB - 64 - 14));  // |L^-1 c|^2 as a row's length in factor_fixed
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        v += __shfl_xor_sync(FULL, v, o);
-        if constexpr (SPIN != 0) w += __shfl_xor_sync(FULL, w, o);
-        n += __shfl_xor_sync(FULL, n, o);
+        v = fx_add(v, __shfl_xor_sync(FULL, v, o));
+        if constexpr (SPIN != 0) w = fx_add(w, __shfl_xor_sync(FULL, w, o));
+        n = fx_add(n, __shfl_xor_sync(FULL, n, o));
+        len += __shfl_xor_sync(FULL, len, o);
     }
+    if (len > (int)(FX_LEN * 16384.0f)) return false;
     val_re = ymax == 0 ? 0.0 : fx_scale2((double)v, ey - FXB);  // no data but zeros: exactly 0
     val_im = SPIN == 0 || ymax == 0 ? 0.0 : fx_scale2((double)w, ey - FXB);
     var_rel = (double)(((int64_t)1 << FXB) - n) * 1.734723475976807e-18;  // 2^-59
