@@ -40,7 +40,7 @@ namespace flints {
 namespace paper {
 
 constexpr int SINV_THREADS = 64;
-constexpr int ROW_EXP_MIN = -6, ROW_EXP_MAX = 24;  // what the fixed-point kernel takes: 2^24 is above 1/sqrt(n)
+constexpr int ROW_EXP_MIN = -6, ROW_EXP_MAX = 16;  // what the fixed-point kernel takes: 2^16 is above 1/sqrt(n)
 
 // offset of column j of a K x K lower-triangular matrix packed by columns
 __host__ __device__ constexpr int col_start(int K, int j) { return j * K - j * (j - 1) / 2; }
@@ -162,10 +162,12 @@ __device__ __forceinline__ int expo_of(double x) {
 }
 
 // the exponent stored for a row whose largest biased exponent is ex: |entry| < 2^(ex - 1022)
-// (rows of L^-1 lie between 1/sqrt(1 + n) and 1/sqrt(n) in size; 0 for absent rows)
+// (rows of L^-1 lie between 1/sqrt(1 + n) and 1/sqrt(n) in size; 0 for absent rows).  Larger
+// rows, which a covariance that is not positive can have, and rows that are not finite read
+// ROW_EXP_MAX + 1: the class's targets take the FP64 form.
 __device__ __forceinline__ int8_t row_exponent(int ex) {
     const int e = ex == 0 ? 0 : ex - 1022;
-    return (int8_t)(e < ROW_EXP_MIN ? ROW_EXP_MIN : e);
+    return (int8_t)(e < ROW_EXP_MIN ? ROW_EXP_MIN : (e > ROW_EXP_MAX ? ROW_EXP_MAX + 1 : e));
 }
 
 struct LinvArgs {
@@ -1265,6 +1267,7 @@ __device__ __forceinline__ void fx_mac3(fxacc3 &a, fx x, int xl, fx y, int yl) {
 __device__ __forceinline__ fxacc fx_fold(fxacc3 a) { return {a.hh, a.cr + (uint64_t)((int64_t)a.ll * 64)}; }
 
 // FP64 form of one target (rows per lane): data that is not finite, classes with a raised nugget
+// or rows above 2^ROW_EXP_MAX
 template <int S>
 __device__ __attribute__((noinline)) void target_fp64(const double *linv, bool mir, const FxApplyWarp<S> &sm, int g, int lane,
                                          double &vr, double &vi, double &qc) {
@@ -1437,9 +1440,10 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32, 4) apply_kernel_fx(ApplyArgs
                 } else {
                     ymax = max(max(expo(y0.x), expo(y0.y)), max(expo(y1.x), expo(y1.y)));
                 }
+                if (max(ep, max(eq, et)) > ROW_EXP_MAX) ymax = 0x7ff;
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) ymax = max(ymax, __shfl_xor_sync(FULL, ymax, o));
-                if (ymax == 0x7ff || __ldg(a.slot_steps + sl) != 0) {  // warp-uniform
+                auto fp64_form = [&]() {
                     double vr, vi, qc;
                     target_fp64<S>(a.linv + (int64_t)sl * linv_len(FX_K) * (S ? 2 : 1), mir, sm, g, lane, vr, vi, qc);
                     if (lane == 0) {
@@ -1448,6 +1452,9 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32, 4) apply_kernel_fx(ApplyArgs
                         sm.q[q] = __double_as_longlong(qc);
                         sm.ve[q] = FX_FP64;
                     }
+                };
+                if (ymax == 0x7ff || __ldg(a.slot_steps + sl) != 0) {  // warp-uniform
+                    fp64_form();
                     continue;
                 }
                 const int ey = ymax - 1022 + 2;  // |y| < 2^(ey - 2)
