@@ -1267,7 +1267,7 @@ __device__ __forceinline__ void fx_mac3(fxacc3 &a, fx x, int xl, fx y, int yl) {
 __device__ __forceinline__ fxacc fx_fold(fxacc3 a) { return {a.hh, a.cr + (uint64_t)((int64_t)a.ll * 64)}; }
 
 // FP64 form of one target (rows per lane): data that is not finite, classes with a raised nugget
-// or rows above 2^ROW_EXP_MAX
+// or rows above 2^ROW_EXP_MAX, targets whose |L^-1 c|^2 no positive covariance has
 template <int S>
 __device__ __attribute__((noinline)) void target_fp64(const double *linv, bool mir, const FxApplyWarp<S> &sm, int g, int lane,
                                          double &vr, double &vi, double &qc) {
@@ -1525,6 +1525,23 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32, 4) apply_kernel_fx(ApplyArgs
                     f1[i].hh -= f0[i].hh;  // (zero on odd lanes)
                     f1[i].cr -= f0[i].cr;
                 }
+                // z_c has at most unit length where the covariance is positive; its entries are taken
+                // modulo 32 and their squares' sum too, so beyond that the length must be known.  The
+                // rows' sums are formed once more from the upper halves of the high words, units of
+                // 2^(e - 19), which cannot wrap (16 units off at most, 2 at e = ROW_EXP_MAX): entries
+                // above 8 would stand out, and below that the sum of squares is exact (beyond)
+                bool beyond = false;
+#pragma unroll
+                for (int i = 0; i < NC / 2; ++i) {
+                    auto top = [](fxacc s) { return (int)((int64_t)s.hh >> 32); };
+                    auto over = [](int t, int e) { return (t < 0 ? -t : t) > 8 << (19 - e); };
+                    const int t0 = top(f0[i]);
+                    int t1 = top(f1[i]), t2 = top(f2[i]);
+                    t1 += __shfl_xor_sync(FULL, t1, 1);
+#pragma unroll
+                    for (int o = 4; o < 32; o <<= 1) t2 += __shfl_xor_sync(FULL, t2, o);
+                    beyond |= over(t0, ep) || over(t1, eq) || over(t2, et);
+                }
                 // shift of z_y: by the bits its largest partial sum takes, rows on their own units
                 int top = 0;
 #pragma unroll
@@ -1574,6 +1591,20 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32, 4) apply_kernel_fx(ApplyArgs
                     dots(w1);
                 }
                 if (lane < FX_K - 32) dots(w2);
+                // |z_c|^2 in units of 2^-14, from the high words (600 a lane at most while entries are below 10)
+                const unsigned len = beyond ? 1u << 26 : (unsigned)(sq.hh >> (2 * FXA - 64 - 14));
+                if (__reduce_add_sync(FULL, len) > (unsigned)(FX_LEN * 16384.0f)) {  // warp-uniform
+                    __syncwarp();
+                    for (int i = lane; i < FX_K; i += 32) {  // the data in FP64 again
+                        const int32_t m = __ldg(a.members + sm.cp[q] * FX_K + i);
+                        typename W::Y v{};
+                        if (m >= 0) v = __ldg(reinterpret_cast<const typename W::Y *>(a.map) + m);
+                        sm.y[g * FX_K + i] = v;
+                    }
+                    __syncwarp();
+                    fp64_form();
+                    continue;
+                }
                 int64_t vr = fx_down<FXA>(sr), vi = fx_down<FXA>(si), vq = fx_down<FXA>(sq);
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) {
