@@ -1266,7 +1266,8 @@ __device__ __forceinline__ void fx_mac3(fxacc3 &a, fx x, int xl, fx y, int yl) {
 }
 __device__ __forceinline__ fxacc fx_fold(fxacc3 a) { return {a.hh, a.cr + (uint64_t)((int64_t)a.ll * 64)}; }
 
-// FP64 form of one target (rows per lane): data that is not finite, classes with a raised nugget
+// FP64 form of one target (rows per lane): data that is not finite or so small that
+// subnormal values count, classes with a raised nugget
 // or rows above 2^ROW_EXP_MAX, targets whose |L^-1 c|^2 no positive covariance has
 template <int S>
 __device__ __attribute__((noinline)) void target_fp64(const double *linv, bool mir, const FxApplyWarp<S> &sm, int g, int lane,
@@ -1433,12 +1434,11 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32, 4) apply_kernel_fx(ApplyArgs
                 // data to integers: the largest of the target into [2^-3, 2^-2)
                 typename W::Y y0 = sm.y[g * FX_K + lane], y1{};
                 if (lane < FX_K - 32) y1 = sm.y[g * FX_K + 32 + lane];
-                auto expo = [](double v) { return (int)((uint64_t)__double_as_longlong(v) >> 52 & 0x7ff); };
                 int ymax;
                 if constexpr (S == 0) {
-                    ymax = max(expo(y0), expo(y1));
+                    ymax = max(data_expo(y0), data_expo(y1));
                 } else {
-                    ymax = max(max(expo(y0.x), expo(y0.y)), max(expo(y1.x), expo(y1.y)));
+                    ymax = max(max(data_expo(y0.x), data_expo(y0.y)), max(data_expo(y1.x), data_expo(y1.y)));
                 }
                 if (max(ep, max(eq, et)) > ROW_EXP_MAX) ymax = 0x7ff;
 #pragma unroll
@@ -1453,7 +1453,7 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32, 4) apply_kernel_fx(ApplyArgs
                         sm.ve[q] = FX_FP64;
                     }
                 };
-                if (ymax == 0x7ff || __ldg(a.slot_steps + sl) != 0) {  // warp-uniform
+                if (ymax == 0x7ff || (ymax > 0 && ymax < DATA_EXPO_MIN) || __ldg(a.slot_steps + sl) != 0) {  // warp-uniform
                     fp64_form();
                     continue;
                 }
@@ -1461,14 +1461,14 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32, 4) apply_kernel_fx(ApplyArgs
                 fx *yf = reinterpret_cast<fx *>(sm.y);
                 __syncwarp();
                 if constexpr (S == 0) {
-                    yf[g * FX_K + lane] = fx_split(fx_of(y0, FXA - ey));
-                    if (lane < FX_K - 32) yf[g * FX_K + 32 + lane] = fx_split(fx_of(y1, FXA - ey));
+                    yf[g * FX_K + lane] = fx_split_all(fx_of(y0, FXA - ey));
+                    if (lane < FX_K - 32) yf[g * FX_K + 32 + lane] = fx_split_all(fx_of(y1, FXA - ey));
                 } else {
                     reinterpret_cast<fxc *>(yf)[g * FX_K + lane] =
-                        fxc{fx_split(fx_of(y0.x, FXA - ey)), fx_split(fx_of(y0.y, FXA - ey))};
+                        fxc{fx_split_all(fx_of(y0.x, FXA - ey)), fx_split_all(fx_of(y0.y, FXA - ey))};
                     if (lane < FX_K - 32)
                         reinterpret_cast<fxc *>(yf)[g * FX_K + 32 + lane] =
-                            fxc{fx_split(fx_of(y1.x, FXA - ey)), fx_split(fx_of(y1.y, FXA - ey))};
+                            fxc{fx_split_all(fx_of(y1.x, FXA - ey)), fx_split_all(fx_of(y1.y, FXA - ey))};
                 }
                 __syncwarp();
                 const E *X = sm.x + g * FX_K, *Y = reinterpret_cast<const E *>(yf) + g * FX_K;
@@ -1613,8 +1613,8 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32, 4) apply_kernel_fx(ApplyArgs
                     vq = shfl_add(vq, o);
                 }
                 if (lane == 0) {
-                    sm.vr[q] = vr;
-                    sm.vi[q] = vi;
+                    sm.vr[q] = ymax == 0 ? 0 : vr;  // no data but zeros: exactly 0
+                    sm.vi[q] = ymax == 0 ? 0 : vi;
                     sm.q[q] = vq;
                     sm.ve[q] = D - 115 + ey;  // z_y counts 2^(D - e - (57 - e) - (58 - ey))
                 }

@@ -110,3 +110,19 @@ def test_target_covariances_of_any_length(row, k, call):
     """|L^-1 c|^2 beyond 1, through 32 (where the kernel's sums wrap), up to 2^22."""
     cl, m, defl = _inputs(0, 16, 40)
     _agree(*call(16, 0, cl, m, 700, defl, row, k), 1e-9)
+
+
+def test_zero_maps_give_zeros(call):
+    cl, m, defl = _inputs(0, 16, 40)
+    (_, v, q), (_, v0, q0) = call(16, 0, cl, 0.0 * m, 700, defl)[1], call(16, 0, cl, m, 700, defl)[1]
+    assert np.all(v == 0) and np.array_equal(q, q0)
+
+
+@pytest.mark.parametrize("size", [2.0 ** -1022, 2.0 ** -960])
+def test_tiny_values_are_kept(size, call):
+    """Maps whose values are subnormal in part or whole, to 1e-9 of the largest and, below
+    that, the rounding of the 36 x 36 products to 2^-1074 carried through L^-1 (2^13)."""
+    cl, m, defl = _inputs(0, 16, 40)
+    (s0, v0, _), (s1, v1, _) = call(16, 0, cl, m * (size / np.max(np.abs(m))), 700, defl)
+    assert np.array_equal(s0, s1)
+    assert np.max(np.abs(v1 - v0)) <= 1e-9 * np.max(np.abs(v0)) + 36 * 2 ** 13 * 5e-324
