@@ -1239,15 +1239,16 @@ __device__ __forceinline__ int lanestep_index(int row, int col) {
 }
 
 // a double below 2^e in size in units of 2^(e - 57), truncated with the lowest bit set (which
-// leaves no bias); flip: the sign bit is inverted
+// leaves no bias), 0 for zeros (pads, entries past the diagonal); flip: the sign bit is inverted
 __device__ __forceinline__ fx fx_entry(double v, int e, unsigned flip) {
     const uint64_t b = (uint64_t)__double_as_longlong(v);
     const uint32_t h = (uint32_t)(b >> 32);
-    const int r = e + 1022 - (int)((h >> 20) & 0x7ffu);  // >= 0
+    const int ex = (int)((h >> 20) & 0x7ffu), r = e + 1022 - ex;  // >= 0
     const uint64_t m = (((uint64_t)((h & 0xfffffu) | 0x100000u) << 32) | (uint32_t)b) << 4;
     const uint64_t a = (m >> (r < 63 ? r : 63)) | 1;
     const int64_t neg = (int64_t)(int)(h ^ flip) >> 63;
-    return fx_split((int64_t)((a ^ (uint64_t)neg) - (uint64_t)neg));
+    const fx p = fx_split((int64_t)((a ^ (uint64_t)neg) - (uint64_t)neg));
+    return ex == 0 ? fx{0, 0} : p;
 }
 
 // Sum of products of L^-1 entries with the low words' products kept: entries grow to
