@@ -1208,7 +1208,7 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32) apply_kernel_aug(ApplyArgs a
 // (row_exp): 2^-3 of the rounding of that entry's products in FP64, and the cross sums of a
 // row's 72 products stay below 2^63.
 // z_y = L^-1 y has no bound of its own: its two 64-bit sums are kept and shifted by what
-// the largest row of the target needs.
+// the largest row sum of the target needs.
 // Member terms are formed for FX_G = 8 targets at a time, flattened over the lanes (288
 // terms, nine full passes; member by member a target needs two, the second with four
 // lanes).  Measured (GB300, 2,097,169 Q/U targets, Nside 1024): 40.5 -> 14.3 ms.
@@ -1526,32 +1526,35 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32, 4) apply_kernel_fx(ApplyArgs
                     f1[i].hh -= f0[i].hh;  // (zero on odd lanes)
                     f1[i].cr -= f0[i].cr;
                 }
-                // z_c has at most unit length where the covariance is positive; its entries are taken
-                // modulo 32 and their squares' sum too, so beyond that the length must be known.  The
-                // rows' sums are formed once more from the upper halves of the high words, units of
-                // 2^(e - 19), which cannot wrap (16 units off at most, 2 at e = ROW_EXP_MAX): entries
-                // above 8 would stand out, and below that the sum of squares is exact (beyond)
+                // Row sums from the upper halves of the high words, in units of 2^(e - 19): nothing
+                // wraps, and they are at most 16 units off (2 at e = ROW_EXP_MAX).  They bound the
+                // sums below, which are taken modulo 2^64.
+                // z_c has at most unit length where the covariance is positive, and its entries and
+                // their squares' sum are held modulo 32: entries above 8 stand out here, and with
+                // none the sum of squares is exact (beyond).
+                // z_y is shifted by the bits of its largest row, not of the lanes' partial sums:
+                // on a map with an offset those are up to 2^13 times larger and cancel, and the
+                // first rows, where z_c is of order 1, would lose these bits (rms error on a map
+                // with an offset of a hundred times its size, Nside 64, spin 2, against long
+                // double: 2.0e-13 of the map from the partial sums' bits, 1.7e-14 now, FP64
+                // kernel 3.1e-14).
                 bool beyond = false;
-#pragma unroll
-                for (int i = 0; i < NC / 2; ++i) {
-                    auto top = [](fxacc s) { return (int)((int64_t)s.hh >> 32); };
-                    auto over = [](int t, int e) { return (t < 0 ? -t : t) > 8 << (19 - e); };
-                    const int t0 = top(f0[i]);
-                    int t1 = top(f1[i]), t2 = top(f2[i]);
-                    t1 += __shfl_xor_sync(FULL, t1, 1);
-#pragma unroll
-                    for (int o = 4; o < 32; o <<= 1) t2 += __shfl_xor_sync(FULL, t2, o);
-                    beyond |= over(t0, ep) || over(t1, eq) || over(t2, et);
-                }
-                // shift of z_y: by the bits its largest partial sum takes, rows on their own units
                 int top = 0;
 #pragma unroll
-                for (int i = NC / 2; i < NC; ++i) {
-                    auto bits = [](fxacc s) {
-                        const int64_t h = (int64_t)(s.hh + (uint64_t)((int64_t)s.cr >> 32));
-                        return 64 - fx_clz((uint64_t)(h ^ (h >> 63)) | 1);
-                    };
-                    top = max(max(top, bits(f0[i]) + ep), max(bits(f1[i]) + eq, bits(f2[i]) + et));
+                for (int i = 0; i < NC; ++i) {
+                    auto high = [](fxacc s) { return (int)((int64_t)s.hh >> 32); };
+                    const int t0 = abs(high(f0[i]));
+                    int t1 = high(f1[i]), t2 = high(f2[i]);
+                    t1 = abs(t1 + __shfl_xor_sync(FULL, t1, 1));
+#pragma unroll
+                    for (int o = 4; o < 32; o <<= 1) t2 += __shfl_xor_sync(FULL, t2, o);
+                    t2 = abs(t2);
+                    if (i < NC / 2) {
+                        beyond |= t0 > 8 << (19 - ep) || t1 > 8 << (19 - eq) || t2 > 8 << (19 - et);
+                    } else {
+                        auto bits = [](int t) { return 64 - __clz((unsigned)t + 16); };
+                        top = max(max(top, bits(t0) + ep), max(bits(t1) + eq, bits(t2) + et));
+                    }
                 }
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(FULL, top, o));
