@@ -224,12 +224,13 @@ int flints_lens_batch(const flints_job *jobs, int n, void *stream);
  *     into the pinned staging buffer.
  *   flints_batch_launch: upload the staged table, reset the work queues and
  *     launch the persistent class kernels on `stream` and on streams of the
- *     batch that are forked from it and joined to it by events:
- *     stream operations only, so it can be captured in a CUDA graph; a replay
- *     runs whatever table was staged last.  The warps_per_block of cfg must
- *     have been used by an earlier launch before capture (changing it
- *     reconfigures the kernel).  Jobs of one batch must not write overlapping
- *     outputs.
+ *     batch that are forked from it, with its priority, and joined to it by
+ *     events: stream operations only, so it can be captured in a CUDA graph; a
+ *     replay runs whatever table was staged last.  The warps_per_block of cfg
+ *     must have been used by an earlier launch before capture (changing it
+ *     reconfigures the kernel); on a stream of a priority that no earlier launch
+ *     used (the default's is always there) a capture holds the class kernels one
+ *     after another.  Jobs of one batch must not write overlapping outputs.
  *   flints_batch_run: stage + launch (tile size from cfg).
  * Errors: FLINTS_EINVAL for bad jobs (message names the job index). */
 typedef struct flints_batch_s *flints_batch_t;

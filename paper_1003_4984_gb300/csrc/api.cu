@@ -482,20 +482,32 @@ constexpr int BATCH_SIDE = 3;
 struct ClassStreams {
     int n;  // side streams of the launch in hand
 #ifdef __CUDACC__
-    cudaStream_t side[BATCH_SIDE];
+    // Side streams have the priority of the stream that they are forked from (the class kernels
+    // of a batch on a high-priority stream would otherwise wait behind other work): one set per
+    // priority, made at the first launch that needs it, the default priority's with the batch.
+    static constexpr int LEVELS = 8;  // priorities least .. least - 7 (the device has six)
+    cudaStream_t sets[LEVELS][BATCH_SIDE], *side;
     cudaEvent_t forked, joined[BATCH_SIDE];
-    cudaError_t create() {
-        cudaError_t e = cudaEventCreateWithFlags(&forked, cudaEventDisableTiming);
-        for (int i = 0; i < BATCH_SIDE && e == cudaSuccess; ++i) {
-            e = cudaStreamCreateWithFlags(&side[i], cudaStreamNonBlocking);
-            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&joined[i], cudaEventDisableTiming);
-        }
+    int least;
+    cudaError_t make(int level) {
+        cudaError_t e = cudaSuccess;
+        for (int i = 0; i < BATCH_SIDE && e == cudaSuccess; ++i)
+            if (!sets[level][i]) e = cudaStreamCreateWithPriority(&sets[level][i], cudaStreamNonBlocking, least - level);
         return e;
+    }
+    cudaError_t create() {
+        int greatest = 0;
+        cudaError_t e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&forked, cudaEventDisableTiming);
+        for (int i = 0; i < BATCH_SIDE && e == cudaSuccess; ++i)
+            e = cudaEventCreateWithFlags(&joined[i], cudaEventDisableTiming);
+        return e == cudaSuccess ? make(0) : e;
     }
     void release() {
         for (int i = 0; i < BATCH_SIDE; ++i) {
             if (joined[i]) cudaEventDestroy(joined[i]);
-            if (side[i]) cudaStreamDestroy(side[i]);
+            for (int l = 0; l < LEVELS; ++l)
+                if (sets[l][i]) cudaStreamDestroy(sets[l][i]);
         }
         if (forked) cudaEventDestroy(forked);
     }
@@ -505,10 +517,20 @@ struct ClassStreams {
         yes = c != cudaStreamCaptureStatusNone;
         return e;
     }
-    // side streams for `kernels` independent launches, ordered after what st holds
-    cudaError_t fork(cudaStream_t st, int kernels) {
-        n = kernels - 1 < BATCH_SIDE ? (kernels > 1 ? kernels - 1 : 0) : BATCH_SIDE;
-        cudaError_t e = n ? cudaEventRecord(forked, st) : cudaSuccess;
+    // side streams for `kernels` independent launches, ordered after what st holds; none (all
+    // kernels in st) in a capture on a priority that no earlier launch has made streams for
+    cudaError_t fork(cudaStream_t st, int kernels, bool capture) {
+        n = 0;
+        if (kernels < 2) return cudaSuccess;
+        int priority = 0;
+        cudaError_t e = cudaStreamGetPriority(st, &priority);
+        const int level = least - priority;
+        if (e != cudaSuccess || level < 0 || level >= LEVELS) return e;
+        if (capture && !sets[level][BATCH_SIDE - 1]) return cudaSuccess;
+        if ((e = make(level)) != cudaSuccess) return e;
+        side = sets[level];
+        n = kernels - 1 < BATCH_SIDE ? kernels - 1 : BATCH_SIDE;
+        e = cudaEventRecord(forked, st);
         for (int i = 0; i < n && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(side[i], forked, 0);
         return e;
     }
@@ -530,7 +552,7 @@ struct ClassStreams {
         yes = false;
         return cudaSuccess;
     }
-    cudaError_t fork(cudaStream_t, int) { return cudaSuccess; }
+    cudaError_t fork(cudaStream_t, int, bool) { return cudaSuccess; }
     cudaStream_t of(cudaStream_t st, int) const { return st; }
     cudaError_t join(cudaStream_t) { return cudaSuccess; }
 #endif
@@ -728,7 +750,7 @@ int flints_batch_launch(flints_batch_t b, const flints_launch_cfg *cfg, void *st
     }
     // costliest class first, dealt over the streams in turn
     std::stable_sort(order, order + nk, [&](int x, int y) { return cost[x] > cost[y]; });
-    cudaError_t err = b->streams.fork(st, nk);
+    cudaError_t err = b->streams.fork(st, nk, all);
     for (int q = 0; q < nk && err == cudaSuccess; ++q) {
         const int cls = order[q];
         cudaStream_t sq = b->streams.of(st, q);
