@@ -629,11 +629,15 @@ int flints_batch_stage(flints_batch_t b, const flints_job *jobs, int n, int tile
         return fail(FLINTS_EINVAL, "flints_batch_stage: %d jobs for a batch of capacity %d", n, b->max_jobs);
     if (tile_points < 0 || tile_points > MAX_TILE_POINTS)
         return fail(FLINTS_EINVAL, "flints_batch_stage: tile_points 0..%d", MAX_TILE_POINTS);
-    // the library's choice: the size that balances all the batch's targets over the 16
-    // warps per SM of the class kernels
+    // the library's choice: the size that balances all the batch's targets over the warps
+    // that the class's kernel keeps resident
     int64_t targets = 0;
     for (int i = 0; i < n; ++i) targets += jobs[i].count > 0 ? jobs[i].count : 0;
-    const int tp = tile_points > 0 ? tile_points : auto_tile_points(targets, (int64_t)b->num_sms * 16);
+    int tp[BATCH_CLASSES];
+    for (int cls = 0; cls < BATCH_CLASSES; ++cls)
+        tp[cls] = tile_points > 0 ? tile_points
+                                  : auto_tile_points(targets, (int64_t)b->num_sms * b->max_bps[cls] * b->wpb[cls]);
+    auto cls_of = [](const BatchJob &x) { return 8 * x.precision + (x.spin == 2 ? 4 : 0) + batch_k_index(x.K); };
     std::vector<BatchJob> v;
     v.reserve(n);
     std::vector<double> cost;
@@ -683,14 +687,14 @@ int flints_batch_stage(flints_batch_t b, const flints_job *jobs, int n, int tile
         bj.K = p->K;
         bj.spin = p->spin;
         bj.precision = p->precision;
-        bj.ntiles = (j.count + tp - 1) / tp;
+        const int tpj = tp[cls_of(bj)];
+        bj.ntiles = (j.count + tpj - 1) / tpj;
         v.push_back(bj);
     }
     // every job is valid: count its points (a refused stage counts none)
     for (int i = 0; i < n; ++i) jobs[i].plan->points += jobs[i].count;
     // classes (precision, spin, K), each in decreasing estimated cost
     // (longest jobs start first)
-    auto cls_of = [](const BatchJob &x) { return 8 * x.precision + (x.spin == 2 ? 4 : 0) + batch_k_index(x.K); };
     auto est = [](const BatchJob &x) {
         return (double)x.a.count * x.K * x.K * x.K * (x.spin == 2 ? 4.0 : 1.0);
     };
@@ -701,7 +705,7 @@ int flints_batch_stage(flints_batch_t b, const flints_job *jobs, int n, int tile
     BatchHeader h{};
     int k = 0;
     for (int cls = 0; cls < BATCH_CLASSES; ++cls) {
-        h.tile_pts[cls] = tp;
+        h.tile_pts[cls] = tp[cls];
         h.job_offset[cls] = k;
         int64_t tiles = 0;
         while (k < (int)v.size() && cls_of(v[k]) == cls) {
