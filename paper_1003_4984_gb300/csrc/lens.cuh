@@ -782,6 +782,26 @@ __device__ __forceinline__ bool factor_bordered(Elem *mat, int lane) {
 // Returns false when a pivot of S + nugget I is not positive.
 constexpr int FXB = 59;
 
+// maximum and sum over the warp: one instruction each on the device
+__device__ __forceinline__ int warp_max(int v) {
+#ifdef __CUDA_ARCH__
+    return __reduce_max_sync(FULL, v);
+#else
+    for (int o = 16; o > 0; o >>= 1) {
+        const int w = __shfl_xor_sync(FULL, v, o);
+        v = w > v ? w : v;
+    }
+    return v;
+#endif
+}
+__device__ __forceinline__ int warp_add(int v) {
+#ifdef __CUDA_ARCH__
+    return __reduce_add_sync(FULL, v);
+#else
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+    return v;
+#endif
+}
 __device__ __forceinline__ int64_t fx_shfl(int64_t v, int src) { return __shfl_sync(FULL, v, src); }
 __device__ __forceinline__ fx fx_shfl(fx v, int src) {
     return {__shfl_sync(FULL, v.hi, src), __shfl_sync(FULL, v.lo, src)};
@@ -832,17 +852,28 @@ __device__ __forceinline__ bool fx_beyond(int64_t v, int lim) {
 // pivot rows passed by shuffles.  Only entries below the diagonal are written (the
 // diagonal is not read again).  Matrix rows beyond 1.9 (not a factor of a positive
 // matrix) end it: false, the caller's FP64 path decides.  The last bordered row holds the
-// data, scaled by its caller below 2^-4; its solve has no bound, and where an entry
-// passes 1/8 the row is shifted down by 3 bits (counted in ey) and the panel's slot redone:
-// the largest entry of the row keeps at least 53 bits.
+// data, scaled by its caller below 2^-FxData::expo; its solve has no bound, and where an entry
+// passes 1.9 / 2^room the row is shifted down by 3 bits (counted in ey) and the panel's slot
+// redone: the largest entry of the row keeps at least 53 bits.
 // The sums here are taken modulo 32, and on a matrix that is not positive a row can be longer
 // than that before its own pivot says so.  A row's squared length is therefore also read from
-// the high words' sum, which holds 512 (n = 96 terms of at most 1.9^2 each are 347): beyond
-// FX_LEN the form declines.  (The three columns of its own panel add at most 21.7, which no
-// wrap turns into an accepted pivot.)  The caller does the same for the row of c, which has no
-// pivot.  With rows of at most that length a cross sum of n terms stays below 2.5 sqrt(n) 2^58,
-// with the data row too: no overflow up to n = 96.
+// the high words' sums, which hold 512 (n = 96 terms of at most 1.9^2 each are 347): where a
+// lane's part of it (s <= 4 lanes share a row) is above 2 the form declines.  What passes is at
+// most 8, the three columns of the row's own panel add 21.7 at most, and a wrap into an accepted
+// pivot needs 31; so an accepted row is as long as its pivot says, at most sqrt(1 + n).  The
+// caller looks at the row of c, which has no pivot, against FX_LEN.  With rows of at most
+// sqrt(1.5) a cross sum of n terms stays below 2.5 sqrt(n) 2^58; with the data row, of entries
+// up to Y, below (sqrt(n) + n Y) 2^58: no overflow (32 2^58) up to n = 96 with the Y of FxData.
+// A redone slot costs, room does not: with Y = 1/8 for all sizes up to one target in four redid
+// one on realisations of the field; with Y by n one in sixty (GB300, the Nside 64
+// temperature sky 796 -> 744 us, 524 k Q/U targets, K = 32, 24.4 -> 23.4 ms).
 constexpr float FX_LEN = 1.5f;
+template <int N, class E>
+struct FxData {
+    static constexpr int terms = std::is_same<E, fxc>::value ? 2 * N : N;
+    static constexpr int room = terms <= 24 ? 1 : (terms <= 48 ? 2 : (terms <= 64 ? 3 : 4));  // Y = 1.9 / 2^room
+    static constexpr int expo = terms <= 64 ? 4 : 5;                                          // data below 2^-expo
+};
 template <int N, int NB, class E>
 __device__ __forceinline__ bool factor_fixed(E *mat, int lane, int &ey) {
     constexpr bool CPLX = std::is_same<E, fxc>::value;
@@ -863,7 +894,7 @@ __device__ __forceinline__ bool factor_fixed(E *mat, int lane, int &ey) {
             const E *Lr = mat + tri<N>(act ? r : j0, 0);
             for (;;) {
                 int64_t vr[PW], vi[PW];
-                int len = 0;  // a pivot row's squared length so far, units of 2^-14
+                bool bad = false, high = false;
                 {
                     fxacc ar[PW], ai[PW];
 #pragma unroll
@@ -891,11 +922,13 @@ __device__ __forceinline__ bool factor_fixed(E *mat, int lane, int &ey) {
                     for (int c = 0; c < PW; ++c) {
                         vr[c] = fx_down<FXB>(ar[c]);
                         vi[c] = CPLX ? fx_down<FXB>(ai[c]) : 0;
-                        if (first && grp == c) len = (int)((int64_t)ar[c].hh >> (2 * FXB - 64 - 14));
+                    }
+                    if (first) {
+#pragma unroll
+                        for (int c = 0; c < PW; ++c) bad |= grp == c && (int)(ar[c].hh >> 32) > 2 << (2 * FXB - 96);
                     }
                 }
                 for (int o = 1; o < s; o <<= 1) {
-                    if (first) len += __shfl_xor_sync(FULL, len, o);
 #pragma unroll
                     for (int c = 0; c < PW; ++c) {
                         vr[c] = fx_add(vr[c], __shfl_xor_sync(FULL, vr[c], o));
@@ -913,7 +946,6 @@ __device__ __forceinline__ bool factor_fixed(E *mat, int lane, int &ey) {
                     }
                 }
                 E l[PW];
-                bool bad = len > (int)(FX_LEN * 16384.0f), high = false;
 #pragma unroll
                 for (int c = 0; c < PW; ++c) {
                     if (first) {
@@ -923,7 +955,7 @@ __device__ __forceinline__ bool factor_fixed(E *mat, int lane, int &ey) {
                         piv[c] = fx_pivot(d);
                     }
                     if (act && r > j0 + c) {
-                        const int lim = data ? piv[c].lim >> 4 : piv[c].lim;
+                        const int lim = data ? piv[c].lim >> FxData<N, E>::room : piv[c].lim;
                         const bool big = fx_beyond(vr[c], lim) || (CPLX && fx_beyond(vi[c], lim));
                         bad |= big && !data;
                         high |= big && data;
@@ -1079,9 +1111,10 @@ __device__ bool solve_point_fixed(SM &sm, const PointA &P, int lane, const LensA
         return fx{(int)(b >> 32), (int)(uint32_t)b};
     };
     // data exponent: the largest |y| of the stencil is scaled into [2^-5, 2^-4), where units of
-    // 2^-59 hold more than its 53 bits (rms error against a long double solve of the same
-    // inputs, 48 targets, spin 0, K = 16, Nside 64, a map with an offset: 5.7e-16 of the map,
-    // the FP64 form 8.3e-16, [2^-9, 2^-8) with forced lowest bits 1.1e-14)
+    // 2^-59 hold more than its 53 bits ([2^-6, 2^-5) and just these at K = 48, spin 1 and 2).
+    // Rms error against a long double solve of the same inputs (48 targets, spin 0, K = 16,
+    // Nside 64, a map with an offset): 5.7e-16 of the map, the FP64 form 8.3e-16,
+    // [2^-9, 2^-8) with forced lowest bits 1.1e-14.
     int ymax = 0;
     int64_t tau[RPL];
 #pragma unroll
@@ -1108,14 +1141,11 @@ __device__ bool solve_point_fixed(SM &sm, const PointA &P, int lane, const LensA
             put(sm.gz[i], fx_of(sm.gz[i] * a.inv_2r, 60));
         }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const int v = __shfl_xor_sync(FULL, ymax, o);
-        ymax = v > ymax ? v : ymax;
-    }
+    ymax = warp_max(ymax);
     __syncwarp();
     if (ymax == 0x7ff || (ymax > 0 && ymax < DATA_EXPO_MIN)) return false;
-    int ey = ymax - 1022 + 4;  // |y| < 2^(ey - 4)
+    constexpr int DE = FxData<K, E>::expo;
+    int ey = ymax - 1022 + DE;  // |y| < 2^(ey - DE)
 
     const fx hr = fx_split(fx_of(0.5 * a.r2, 64)), r2 = fx_split(fx_of(a.r2, 62));
     constexpr int64_t DIAG = (int64_t)((1.0 + NUGGET_EPS) * 576460752303423488.0);  // 2^59
@@ -1204,13 +1234,13 @@ __device__ bool solve_point_fixed(SM &sm, const PointA &P, int lane, const LensA
         }
     }
     int64_t v = fx_down<FXB>(sr), w = fx_down<FXB>(si), n = fx_down<FXB>(sn);
-    int len = (int)((int64_t)sn.hh >> (2 * FXB - 64 - 14));  // |L^-1 c|^2 as a row's length in factor_fixed
+    // |L^-1 c|^2 from the high words, units of 2^-14
+    const int len = warp_add((int)((int64_t)sn.hh >> (2 * FXB - 64 - 14)));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         v = fx_add(v, __shfl_xor_sync(FULL, v, o));
         if constexpr (SPIN != 0) w = fx_add(w, __shfl_xor_sync(FULL, w, o));
         n = fx_add(n, __shfl_xor_sync(FULL, n, o));
-        len += __shfl_xor_sync(FULL, len, o);
     }
     if (len > (int)(FX_LEN * 16384.0f)) return false;
     val_re = ymax == 0 ? 0.0 : fx_scale2((double)v, ey - FXB);  // no data but zeros: exactly 0

@@ -1442,8 +1442,7 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32, 4) apply_kernel_fx(ApplyArgs
                     ymax = max(max(data_expo(y0.x), data_expo(y0.y)), max(data_expo(y1.x), data_expo(y1.y)));
                 }
                 if (max(ep, max(eq, et)) > ROW_EXP_MAX) ymax = 0x7ff;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) ymax = max(ymax, __shfl_xor_sync(FULL, ymax, o));
+                ymax = warp_max(ymax);
                 auto fp64_form = [&]() {
                     double vr, vi, qc;
                     target_fp64<S>(a.linv + (int64_t)sl * linv_len(FX_K) * (S ? 2 : 1), mir, sm, g, lane, vr, vi, qc);
@@ -1556,8 +1555,7 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32, 4) apply_kernel_fx(ApplyArgs
                         top = max(max(top, bits(t0) + ep), max(bits(t1) + eq, bits(t2) + et));
                     }
                 }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) top = max(top, __shfl_xor_sync(FULL, top, o));
+                top = warp_max(top);
                 const int D = top + 6 > 33 + ROW_EXP_MAX ? top + 6 : 33 + ROW_EXP_MAX;  // |z_y| < 2^58 units
                 auto down = [](fxacc s, int d) {
                     if (d > 64) return (int64_t)(s.hh + (uint64_t)((int64_t)s.cr >> 32)) >> (d - 64);
@@ -1596,8 +1594,8 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32, 4) apply_kernel_fx(ApplyArgs
                 }
                 if (lane < FX_K - 32) dots(w2);
                 // |z_c|^2 in units of 2^-14, from the high words (600 a lane at most while entries are below 10)
-                const unsigned len = beyond ? 1u << 26 : (unsigned)(sq.hh >> (2 * FXA - 64 - 14));
-                if (__reduce_add_sync(FULL, len) > (unsigned)(FX_LEN * 16384.0f)) {  // warp-uniform
+                const unsigned len = beyond ? 1u << 25 : (unsigned)(sq.hh >> (2 * FXA - 64 - 14));
+                if (warp_add((int)len) > (int)(FX_LEN * 16384.0f)) {  // warp-uniform
                     __syncwarp();
                     for (int i = lane; i < FX_K; i += 32) {  // the data in FP64 again
                         const int32_t m = __ldg(a.members + sm.cp[q] * FX_K + i);
