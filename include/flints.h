@@ -267,8 +267,10 @@ const char *flints_last_error(void);
  *     + 2 Npix complex doubles) and the cuFFT plans for Nside (1..8192), lmax
  *     (spin..16384) and spin (0, 1, 2).  precision FLINTS_FP64: the l-recurrence
  *     in FP64; FLINTS_MIXED: in 64-bit fixed point on the integer pipe (error
- *     about 2e-13 of the map at lmax 2048; 40 (spin 0) or 56 bytes more per
- *     (l, m) for its tables).  Allocates; not capturable.
+ *     about 2e-13 of the map at lmax 2048; 24 bytes more per (l, m) for its
+ *     tables, and room for 16 (spin 0) or 32 bytes per (l, m) of weights in the
+ *     work arrays where they hold less).  Set-up takes as long as in FP64 within
+ *     a few percent.  Allocates; not capturable.
  *   flints_synthesize: alm (and blm for spin 1, 2; NULL = 0) DEVICE complex
  *     double [lmax+1][lmax+1] (index [l][m], m <= l read), 16-byte aligned;
  *     map DEVICE double [Npix] (spin 0) or [Npix][2] (spin 1, 2), RING order.

@@ -282,56 +282,109 @@ __host__ __device__ __forceinline__ long long tri_row(int lmax, int m) {
     return (long long)m * (lmax + 1) - (long long)m * (m - 1) / 2 - m;
 }
 
-// C_l = q_l / q_{l+1} with q_l = sqrt((l^2 - m^2)(l^2 - s^2)) / l, so alpha_l alpha_{l-1} q_l is
-// the same for all l.  Three kernels: q_l for every (l, m); alpha downwards in l, one thread
-// per m (the only serial part: one division a step); coefficients, weights' factors and starts.
-__global__ void synth_q_kernel(int lmax, int s, double *__restrict__ na) {
-    const int m = blockIdx.y, l = (m > s ? m : s) + blockIdx.x * blockDim.x + threadIdx.x;
+// What depends on l alone: with q_l = sqrt((l^2 - m^2)(l^2 - s^2)) / l, q_l = g sqrt(l^2 - m^2).
+struct alignas(16) SynthOrder {
+    double g, ig, igl;  // sqrt(1 - s^2 / l^2) and its reciprocal, a pair of doubles (0 for l <= s)
+    double n, b;        // N_l = sqrt((2l + 1) / 4 pi), s / (l (l + 1))
+    double pad;
+};
+// what 1 / sqrt(x) adds to r, its value in FP64
+__device__ __forceinline__ double rsqrt_rest(double x, double r) {
+    const double p = x * r, pl = fma(x, r, -p);
+    return 0.5 * r * (fma(-p, r, 1.0) - pl * r);
+}
+__global__ void synth_order_kernel(int lmax, int s, SynthOrder *__restrict__ ord, double *__restrict__ start) {
+    const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l > lmax) return;
-    const double ld = l, md = m, sd = s;
-    na[tri_row(lmax, m) + l] = l > 0 ? sqrt((ld * ld - md * md) * (ld * ld - sd * sd)) / ld : 0.0;
-}
-
-// na: q_l in, alpha_l out
-__global__ void synth_alpha_kernel(int lmax, int s, double *__restrict__ na) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m > lmax) return;
-    const int l0 = m > s ? m : s;
-    double *n = na + tri_row(lmax, m);
-    double q = n[lmax], alpha = 1.0;
-    const double same = q;  // alpha = 1 at lmax and lmax - 1
-    n[lmax] = 1.0;
-    for (int l = lmax - 1; l >= l0; --l) {
-        const double below = n[l];
-        alpha = l == lmax - 1 ? 1.0 : same / (alpha * q);
-        n[l] = alpha;
-        q = below;
+    const double ld = l, sd = s;
+    SynthOrder o{0.0, 0.0, 0.0, sqrt((2.0 * ld + 1.0) / (4.0 * PI_D)), s > 0 && l > 0 ? sd / (ld * (ld + 1.0)) : 0.0, 0.0};
+    if (l > s) {
+        const double x = (ld - sd) * (ld + sd), r = rsqrt(x);
+        o.g = sqrt(x) / ld;
+        o.ig = ld * r;
+        o.igl = fma(ld, r, -o.ig) + ld * rsqrt_rest(x, r);
     }
+    ord[l] = o;
+    start[l] = start_factor(l, s);  // m = l
 }
 
-// na: alpha_l in, alpha_l N_l out (per block of one m, whose threads take l in turn from the top)
-__global__ void synth_coef_kernel(int lmax, int s, SynthStep *__restrict__ steps, double *__restrict__ na,
-                                  double *__restrict__ start) {
-    const int m = blockIdx.x, l0 = m > s ? m : s;
+// C_l = q_l / q_{l+1}, so alpha_l alpha_{l-1} q_l is the same for all l, and
+// alpha_l = alpha_{l+2} q_{l+2} / q_{l+1}: two chains of products downwards in l.  One block per
+// m; a thread multiplies along its stretch of both chains, and by what lies above it.  The coefficients are a_l = (2l + 1) / q_{l+1} alpha_l / alpha_{l+1}
+// and b_l = a_l m s / (l (l + 1)), with the quotient of the alphas as they are stored; a_l is
+// formed as a pair of doubles, because its error moves the recurrence's phase (FP64 alone
+// leaves two to four units of 2^-54).
+// What bounds it: the FP64 pipe, one reciprocal square root and one division per (l, m).
+// Measured (GB300, lmax 4096, spin 2): 0.77 ms; with a chain per thread, a division a step and
+// the roots in FP64 divisions 5.1 ms, of which the host's FFT planning hid none: the plan's
+// set-up took 16.2 ms, 11.4 now, an FP64 plan's 11.0.
+constexpr int COEF_THREADS = 256;
+__global__ void __launch_bounds__(COEF_THREADS) synth_coef_kernel(int lmax, int s, const SynthOrder *__restrict__ ord,
+                                                                  SynthStep *steps, double *na, double *start) {
+    __shared__ double prod[2][COEF_THREADS];
+    const int m = blockIdx.x, l0 = m > s ? m : s, tid = threadIdx.x;
     SynthStep *st = steps + tri_row(lmax, m);
     double *n = na + tri_row(lmax, m);
-    const double md = m, sd = s, inv4pi = 1.0 / (4.0 * PI_D);
-    if (threadIdx.x == 0) start[m] = start_factor(m, s) - log2(n[l0]);
-    for (int base = l0; base <= lmax; base += blockDim.x) {  // upwards: alpha_{l+1} is read before its block overwrites it
-        const int l = base + threadIdx.x;
-        const double cur = l <= lmax ? n[l] : 1.0, up = l < lmax ? n[l + 1] : 1.0;
+    // 1 / sqrt(l^2 - m^2), kept in the steps' places until these are formed
+    auto root = [&](int l) { return __longlong_as_double(st[l].b); };
+    for (int l = l0 + tid; l <= lmax; l += COEF_THREADS) {
+        const int x = (l - m) * (l + m);
+        st[l].b = __double_as_longlong(x > 0 ? rsqrt((double)x) : 0.0);
+    }
+    __syncthreads();
+    auto ratio = [&](int l) {  // q_{l+2} / q_{l+1}
+        const double above = (double)((l + 2 - m) * (l + 2 + m)) * root(l + 2) * ord[l + 2].g;
+        return above * (root(l + 1) * ord[l + 1].ig);
+    };
+    const int pairs = (lmax - l0 + 2) / 2, per = (pairs + COEF_THREADS - 1) / COEF_THREADS;
+    const int p0 = tid * per < pairs ? tid * per : pairs, p1 = p0 + per < pairs ? p0 + per : pairs;
+    double c0 = 1.0, c1 = 1.0;  // alpha = 1 at lmax and lmax - 1
+    for (int p = p0; p < p1; ++p) {
+        const int l = lmax - 2 * p;
+        if (p > 0) c0 *= ratio(l);
+        n[l] = c0;
+        if (l > l0) {
+            if (p > 0) c1 *= ratio(l - 1);
+            n[l - 1] = c1;
+        }
+    }
+    prod[0][tid] = c0;
+    prod[1][tid] = c1;
+    __syncthreads();
+    if (tid < 2) {  // in order: the last alpha of a stretch is then exactly what the next one is multiplied by
+        double v = 1.0;
+        for (int t = 0; t < COEF_THREADS; ++t) {
+            const double c = prod[tid][t];
+            prod[tid][t] = v;
+            v *= c;
+        }
+    }
+    __syncthreads();
+    c0 = prod[0][tid];
+    c1 = prod[1][tid];
+    for (int p = p0; p < p1; ++p) {
+        const int l = lmax - 2 * p;
+        n[l] *= c0;
+        if (l > l0) n[l - 1] *= c1;
+    }
+    __syncthreads();
+    for (int base = l0; base <= lmax; base += COEF_THREADS) {  // upwards: what lies above l is read before its block overwrites it
+        const int l = base + tid;
+        const double cur = l <= lmax ? n[l] : 1.0, up = l < lmax ? n[l + 1] : 1.0, r = l < lmax ? root(l + 1) : 0.0;
+        if (l == l0) start[m] -= log2(cur);
         __syncthreads();
         if (l > lmax) continue;
-        const double ld = l, lp = ld + 1.0;
-        n[l] = sqrt((2.0 * ld + 1.0) * inv4pi) * cur;
-        const double den = ld * sqrt((lp * lp - md * md) * (lp * lp - sd * sd));
-        double a = 1.0, b = 0.0;  // l = m = s = 0: d^1 = x d^0
-        if (l > 0 && den > 0.0) {
-            a = (2.0 * ld + 1.0) * ld * lp / den;
-            b = (2.0 * ld + 1.0) * md * sd / den;
+        n[l] = ord[l].n * cur;
+        double a = 0.0, al = 0.0;  // (lmax: no step)
+        if (l < lmax) {
+            const double k = 2.0 * l + 1.0, iu = 1.0 / up, v = cur * iu, vl = fma(-v, up, cur) * iu;
+            const double ig = ord[l + 1].ig, t = k * r, tl = fma(k, r, -t) + k * rsqrt_rest((double)((l + 1 - m) * (l + 1 + m)), r);
+            const double u = t * ig, ul = fma(t, ig, -u) + tl * ig + t * ord[l + 1].igl;
+            a = u * v;
+            al = fma(u, v, -a) + ul * v + u * vl;
         }
-        const double r = cur / up;
-        st[l] = SynthStep{halves(flints::fx_of(a * r, AS) + OFF), (long long)flints::fx_of(b * r, GS)};
+        const double b = a * ((double)m * ord[l].b);
+        st[l] = SynthStep{halves(flints::fx_of(a, AS) + flints::fx_of(al, AS) + OFF), (long long)flints::fx_of(b, GS)};
     }
 }
 
@@ -729,11 +782,13 @@ struct flints_synth_s {
     SynthRing *d_rings;
     int *d_polar;      // indices of the polar rings
     double2 *d_F, *d_H, *d_A, *d_FB;
-    SynthStep *d_steps;    // recurrence coefficients per (m, l)
+    SynthStep *d_steps;    // recurrence coefficients per (m, l); these and the next three lie behind F
     double *d_na;          // alpha_l N_l per (m, l)
     double *d_start;       // log2 of the columns' start factor per m
-    flints::fxc *d_W;      // weights of the call in hand per (m, l)
-    int *d_we;             // their exponents per m
+    int *d_we;             // exponents of the weights per m, of the call in hand
+    // the weights themselves, per (m, l), lie in d_H: the l-sums have read them before the fold
+    // writes there
+    flints::fxc *weights() const { return reinterpret_cast<flints::fxc *>(d_H); }
     void *d_work;
     std::vector<SynthRing> rings;
     int npolar;
@@ -752,11 +807,6 @@ static void synth_release(flints_synth_s *s) {
     cudaFree(s->d_H);
     cudaFree(s->d_A);
     cudaFree(s->d_FB);
-    cudaFree(s->d_steps);
-    cudaFree(s->d_na);
-    cudaFree(s->d_start);
-    cudaFree(s->d_W);
-    cudaFree(s->d_we);
     cudaFree(s->d_work);
 }
 
@@ -773,8 +823,8 @@ static void launch_sums(flints_synth_s *s, const double2 *alm, const double2 *bl
     const int N = (int)s->nside, lmax = s->lmax, nr = 4 * N - 1;
     const dim3 grid((2 * N + 127) / 128, lmax + 1);
     if (s->precision == FLINTS_MIXED) {
-        synth_weight_kernel<S><<<lmax + 1, 256, 0, st>>>(lmax, s->d_na, alm, blm, s->d_W, s->d_we);
-        legendre_fx_kernel<S><<<grid, 128, 0, st>>>(lmax, N, s->d_rings, s->d_steps, s->d_W, s->d_we, s->d_start, s->d_F);
+        synth_weight_kernel<S><<<lmax + 1, 256, 0, st>>>(lmax, s->d_na, alm, blm, s->weights(), s->d_we);
+        legendre_fx_kernel<S><<<grid, 128, 0, st>>>(lmax, N, s->d_rings, s->d_steps, s->weights(), s->d_we, s->d_start, s->d_F);
     } else {
         legendre_kernel<S><<<grid, 128, 0, st>>>(lmax, N, s->d_rings, alm, blm, s->d_F);
     }
@@ -806,7 +856,6 @@ int flints_synth_plan(flints_synth_t *out, int64_t nside, int lmax, int spin, in
     s->d_F = s->d_H = s->d_A = s->d_FB = nullptr;
     s->d_steps = nullptr;
     s->d_na = s->d_start = nullptr;
-    s->d_W = nullptr;
     s->d_we = nullptr;
     s->d_work = nullptr;
     s->belt_made = false;
@@ -879,18 +928,24 @@ int flints_synth_plan(flints_synth_t *out, int64_t nside, int lmax, int spin, in
     s->npolar = (int)polar.size();
     const size_t NM = spin == 0 ? (size_t)lmax + 1 : 2 * (size_t)lmax + 1;
     const size_t npair = (size_t)(lmax + 1) * (lmax + 2) / 2;
+    // tables of a mixed plan, behind F: steps, alpha_l N_l, starts, exponents
+    const size_t tbytes = precision == FLINTS_MIXED
+                              ? (sizeof(SynthStep) + sizeof(double)) * npair + (sizeof(double) + sizeof(int)) * (lmax + 1)
+                              : 0;
+    // the belt's FFT inputs and, before them in a call, the weights (mixed)
+    const size_t wbytes = precision == FLINTS_MIXED ? sizeof(flints::fxc) * npair * (spin == 0 ? 1 : 2) : 0;
+    const size_t hbytes = sizeof(double2) * (size_t)hsize > wbytes ? sizeof(double2) * (size_t)hsize : wbytes;
     cudaError_t e;
     if ((e = cudaMalloc(&s->d_rings, sizeof(SynthRing) * nr)) != cudaSuccess ||
-        (e = cudaMalloc(&s->d_F, sizeof(double2) * NM * nr)) != cudaSuccess ||
-        (e = cudaMalloc(&s->d_H, sizeof(double2) * (size_t)hsize)) != cudaSuccess)
+        (e = cudaMalloc(&s->d_F, sizeof(double2) * NM * nr + tbytes)) != cudaSuccess ||
+        (e = cudaMalloc(&s->d_H, hbytes)) != cudaSuccess)
         return synth_bail(s, e == cudaErrorMemoryAllocation ? FLINTS_ENOMEM : FLINTS_ECUDA, "allocation", e);
-    if (precision == FLINTS_MIXED &&
-        ((e = cudaMalloc(&s->d_steps, sizeof(SynthStep) * npair)) != cudaSuccess ||
-         (e = cudaMalloc(&s->d_na, sizeof(double) * npair)) != cudaSuccess ||
-         (e = cudaMalloc(&s->d_start, sizeof(double) * (size_t)(lmax + 1))) != cudaSuccess ||
-         (e = cudaMalloc(&s->d_W, sizeof(flints::fxc) * npair * (spin == 0 ? 1 : 2))) != cudaSuccess ||
-         (e = cudaMalloc(&s->d_we, sizeof(int) * (size_t)(lmax + 1))) != cudaSuccess))
-        return synth_bail(s, e == cudaErrorMemoryAllocation ? FLINTS_ENOMEM : FLINTS_ECUDA, "allocation", e);
+    if (precision == FLINTS_MIXED) {
+        s->d_steps = reinterpret_cast<SynthStep *>(s->d_F + NM * nr);
+        s->d_na = reinterpret_cast<double *>(s->d_steps + npair);
+        s->d_start = s->d_na + npair;
+        s->d_we = reinterpret_cast<int *>(s->d_start + lmax + 1);
+    }
     if (s->npolar > 0 &&
         ((e = cudaMalloc(&s->d_polar, sizeof(int) * polar.size())) != cudaSuccess ||
          (e = cudaMalloc(&s->d_A, sizeof(double2) * (size_t)aoff)) != cudaSuccess ||
@@ -904,9 +959,11 @@ int flints_synth_plan(flints_synth_t *out, int64_t nside, int lmax, int spin, in
                                               cudaMemcpyHostToDevice, st)) != cudaSuccess)
         return synth_bail(s, FLINTS_ECUDA, "copy", e);
     if (precision == FLINTS_MIXED) {
-        synth_q_kernel<<<dim3((lmax + 256) / 256, lmax + 1), 256, 0, st>>>(lmax, spin, s->d_na);
-        synth_alpha_kernel<<<(lmax + 32) / 32, 32, 0, st>>>(lmax, spin, s->d_na);
-        synth_coef_kernel<<<lmax + 1, 128, 0, st>>>(lmax, spin, s->d_steps, s->d_na, s->d_start);
+        // (the orders' table lies in d_F, which no call has written yet)
+        SynthOrder *ord = reinterpret_cast<SynthOrder *>(s->d_F);
+        static_assert(sizeof(SynthOrder) <= 3 * sizeof(double2), "F holds at least 3 (lmax + 1) complex numbers");
+        synth_order_kernel<<<(lmax + 256) / 256, 256, 0, st>>>(lmax, spin, ord, s->d_start);
+        synth_coef_kernel<<<lmax + 1, COEF_THREADS, 0, st>>>(lmax, spin, ord, s->d_steps, s->d_na, s->d_start);
         if ((e = cudaGetLastError()) != cudaSuccess) return synth_bail(s, FLINTS_ECUDA, "coefficients", e);
     }
     // cuFFT plans sharing one work area
