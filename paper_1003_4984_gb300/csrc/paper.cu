@@ -1311,13 +1311,13 @@ struct FxChord {
 };
 
 template <int S>
-__global__ void __launch_bounds__(APPLY_WARPS * 32, 4) apply_kernel_fx(ApplyArgs a, FxChord ch) {
+__global__ void __launch_bounds__(APPLY_WARPS * 32, 4) apply_kernel_fx(ApplyArgs a, FxChord ch, int tile_pts) {
     extern __shared__ __align__(16) unsigned char fx_smem[];
     using W = FxApplyWarp<S>;
     using E = typename W::E;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     W &sm = reinterpret_cast<W *>(fx_smem)[wid];
-    const int64_t ntiles = (a.count + 31) / 32;
+    const int64_t ntiles = (a.count + tile_pts - 1) / tile_pts;
     const int64_t mirror_from = 6 * a.Nc * a.Nc + 2 * a.Nc;  // first pixel of coarse ring 2 Nc + 1
     unsigned long long n_win = 0, n_nug = 0, n_fail = 0;
     for (int64_t tile = (int64_t)blockIdx.x * APPLY_WARPS + wid; tile < ntiles;
@@ -1325,7 +1325,7 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32, 4) apply_kernel_fx(ApplyArgs
         {
             double x = 0.0, y = 0.0, z = 1.0;
             int64_t c = 0;
-            target_of(a, tile * 32 + lane, x, y, z, c);
+            target_of(a, lane < tile_pts ? tile * tile_pts + lane : a.count, x, y, z, c);
             if (!(z == z)) {  // not finite: NaN outputs whatever is computed (finish_point)
                 x = y = 0.0;
                 z = 1.0;
@@ -1345,16 +1345,16 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32, 4) apply_kernel_fx(ApplyArgs
             sm.win[lane] = 0;
         }
         __syncwarp();
-        const int npt = a.count - tile * 32 < 32 ? (int)(a.count - tile * 32) : 32;
+        const int npt = a.count - tile * tile_pts < tile_pts ? (int)(a.count - tile * tile_pts) : tile_pts;
         for (int q0 = 0; q0 < npt; q0 += FX_G) {
             // ---- member terms of targets q0 .. q0 + 7
 #pragma unroll 1
-            for (int it = lane; it < FX_G * FX_K; it += 32) {
+            for (int it = lane; it < (npt - q0 < FX_G ? npt - q0 : FX_G) * FX_K; it += 32) {
                 const int g = it / FX_K, q = q0 + g;
                 E xc{};
                 typename W::Y yv{};
                 const int64_t c = sm.cp[q];
-                const int32_t m = q < npt ? __ldg(a.members + c * FX_K + (it - g * FX_K)) : -1;
+                const int32_t m = __ldg(a.members + c * FX_K + (it - g * FX_K));
                 if (m >= 0) {
                     const double2 p0 = __ldg(a.pv + 2 * (int64_t)m), p1 = __ldg(a.pv + 2 * (int64_t)m + 1);
                     double dx, dy;  // as the FP64 kernels form them (spin 1, 2: the product is not rounded)
@@ -1629,7 +1629,7 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32, 4) apply_kernel_fx(ApplyArgs
             const double vr = f64 ? __longlong_as_double(sm.vr[lane]) : fx_scale2((double)sm.vr[lane], ve);
             const double vi = f64 ? __longlong_as_double(sm.vi[lane]) : fx_scale2((double)sm.vi[lane], ve);
             const double qc = f64 ? __longlong_as_double(sm.q[lane]) : (double)sm.q[lane] * 3.469446951953614e-18;
-            const int64_t p = tile * 32 + lane;
+            const int64_t p = tile * tile_pts + lane;
             if constexpr (S == 0) finish_point(a, p, sm.sl[lane], vr, qc, sm.win[lane] != 0, n_win, n_nug, n_fail);
             else finish_point_s2(a, p, sm.sl[lane], vr, vi, qc, sm.win[lane] != 0, n_win, n_nug, n_fail);
         }
@@ -2339,8 +2339,18 @@ static int table_intervals(const double *cl, const double *cl_bb, int lmax, doub
     return want > 16 ? 65536 : (want < 6 ? 64 : (1 << (int)want));
 }
 
+// Targets per tile of the fixed-point kernel: a warp works through its tile one target after
+// another, so a call with fewer targets than full tiles for all resident warps (four blocks of
+// four per SM) takes smaller ones, whole groups of FX_G where a tile has more than one.
+// Measured (GB300, Nside 512, spin 0, us; the FP64 kernel, tiles of 32, this rule): 333 targets 175,
+// 218, 20; 5,000 181, 223, 49; 20,000 233, 240, 147.
+static int fx_tile_points(int64_t count) {
+    const int64_t warps = (int64_t)device_sm_count() * 4 * APPLY_WARPS, t = (count + warps - 1) / warps;
+    return t <= FX_G ? (int)t : (t >= 32 ? 32 : (int)((t + FX_G - 1) / FX_G * FX_G));
+}
+
 template <int S>
-static cudaError_t launch_fx(const ApplyArgs &a, double t_max, unsigned grid, cudaStream_t st) {
+static cudaError_t launch_fx(const ApplyArgs &a, double t_max, cudaStream_t st) {
     FxChord ch;
     ch.k = (int)std::floor(-0.5 * std::log2(t_max));  // t_max 4^k in (1/4, 1]
     ch.k = ch.k < 0 ? 0 : ch.k;
@@ -2350,7 +2360,9 @@ static cudaError_t launch_fx(const ApplyArgs &a, double t_max, unsigned grid, cu
     const size_t smem = APPLY_WARPS * sizeof(FxApplyWarp<S>);
     const cudaError_t e = cudaFuncSetAttribute(apply_kernel_fx<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    apply_kernel_fx<S><<<grid, APPLY_WARPS * 32, smem, st>>>(a, ch);
+    const int tile = fx_tile_points(a.count);
+    const int64_t blocks = ((a.count + tile - 1) / tile + APPLY_WARPS - 1) / APPLY_WARPS, cap = (int64_t)device_sm_count() * 16;
+    apply_kernel_fx<S><<<(unsigned)(blocks < cap ? blocks : cap), APPLY_WARPS * 32, smem, st>>>(a, ch, tile);
     return cudaGetLastError();
 }
 
@@ -2636,9 +2648,9 @@ static int paper_run(flints_paper_t p, int64_t nside_tgt, int64_t first, int64_t
     const bool mixed = p->precision == FLINTS_MIXED;
     if (p->fixed) {
         a.tab.cfx = p->d_cfx;
-        const cudaError_t ef = p->spin == 0 ? launch_fx<0>(a, p->t_max, grid, st)
-                               : p->spin == 1 ? launch_fx<1>(a, p->t_max, grid, st)
-                                              : launch_fx<2>(a, p->t_max, grid, st);
+        const cudaError_t ef = p->spin == 0 ? launch_fx<0>(a, p->t_max, st)
+                               : p->spin == 1 ? launch_fx<1>(a, p->t_max, st)
+                                              : launch_fx<2>(a, p->t_max, st);
         if (ef != cudaSuccess) return pcuda(ef, "paper apply kernel launch");
     } else if (p->flags & FLINTS_SPIN2_AUGMENTED) {
         if (p->K == 9)
