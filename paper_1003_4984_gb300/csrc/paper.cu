@@ -1882,9 +1882,8 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32) apply_kernel_df(ApplyArgs a)
 // loads are independent of one another (27 in flight where a group of ten lanes had one
 // chain of four), every lane works on every multiply-add of the 45-entry factor, and nothing
 // is exchanged between lanes.  The sums run in the order of the ten-lane groups that this
-// replaced (column by column, the rows' products by halving), so results are the same bit
-// for bit.  What bounds it: the FP64 target geometry (200 FP64 instructions a tile).
-// Measured (GB300, the Nside 2048 sky, double-float): 32.4 -> 23.7 ms.
+// replaced (column by column, the rows' products by halving).  What bounds it: the FP64 target geometry (200 FP64 instructions a tile).
+// Measured (GB300, the Nside 2048 sky, double-float): 32.4 -> 22.7 ms.
 template <class R>
 struct Nine;
 template <>
@@ -1906,9 +1905,13 @@ struct Nine<double> {
     static __device__ __forceinline__ Acc acc() { return 0.0; }
     static __device__ __forceinline__ void mac(Acc &s, T x, T y) { s = fma(x, y, s); }
     static __device__ __forceinline__ T val(Acc s) { return s; }
-    static __device__ __forceinline__ T mul(T x, T y) { return x * y; }
+    // a product of its own, and a product and a sum in one rounding: written out, because what the
+    // compiler contracts would depend on the kernel that holds it
+    static __device__ __forceinline__ T mul(T x, T y) { return fma(x, y, 0.0); }
+    static __device__ __forceinline__ T fold(T x, T y, T s) { return fma(x, y, s); }
     static __device__ __forceinline__ T add(T x, T y) { return x + y; }
     static __device__ __forceinline__ double out(T x) { return x; }
+    static __device__ __forceinline__ T shfl(T x, int src) { return __shfl_sync(FULL, x, src); }
 };
 template <>
 struct Nine<df> {
@@ -1929,8 +1932,10 @@ struct Nine<df> {
     static __device__ __forceinline__ void mac(Acc &s, T x, T y) { dfacc_add_prod(s, x, y); }
     static __device__ __forceinline__ T val(Acc s) { return dfacc_val(s); }
     static __device__ __forceinline__ T mul(T x, T y) { return df_mul(x, y); }
+    static __device__ __forceinline__ T fold(T x, T y, T s) { return df_add_fast(df_mul(x, y), s); }
     static __device__ __forceinline__ T add(T x, T y) { return df_add_fast(x, y); }
     static __device__ __forceinline__ double out(T x) { return df_to(x); }
+    static __device__ __forceinline__ T shfl(T x, int src) { return shfl_df(x, src); }
 };
 
 template <class R>
@@ -1958,7 +1963,8 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32) apply_kernel_nine(ApplyArgs 
             if (m[j] >= 0) N9::member(a, m[j], tx, ty, tz, cv[j], yv[j], win);
         }
         const int64_t base = (int64_t)sl * linv_len(K);
-        T vs[K], qs[K];
+        // row 8 onto row 0, then halves of eight
+        T c1[4], y1[4], vs[4], qs[4], v4 = N9::zero(), q4 = N9::zero();
 #pragma unroll
         for (int i = 0; i < K; ++i) {
             typename N9::Acc zc = N9::acc(), zy = N9::acc();
@@ -1968,15 +1974,23 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32) apply_kernel_nine(ApplyArgs 
                 N9::mac(zc, e, cv[j]);
                 N9::mac(zy, e, yv[j]);
             }
-            const T c1 = N9::val(zc), y1 = N9::val(zy);
-            vs[i] = N9::mul(c1, y1);
-            qs[i] = N9::mul(c1, c1);
+            const T c = N9::val(zc), y = N9::val(zy);
+            if (i < 4) {
+                c1[i] = c;
+                y1[i] = y;
+            } else if (i == 4) {
+                v4 = N9::mul(c, y);
+                q4 = N9::mul(c, c);
+            } else if (i < 8) {
+                vs[i - 4] = N9::fold(c1[i - 4], y1[i - 4], N9::mul(c, y));
+                qs[i - 4] = N9::fold(c1[i - 4], c1[i - 4], N9::mul(c, c));
+            } else {
+                vs[0] = N9::add(N9::fold(c1[0], y1[0], N9::mul(c, y)), v4);
+                qs[0] = N9::add(N9::fold(c1[0], c1[0], N9::mul(c, c)), q4);
+            }
         }
-        // row 8 onto row 0, then halves of eight
-        vs[0] = N9::add(vs[0], vs[8]);
-        qs[0] = N9::add(qs[0], qs[8]);
 #pragma unroll
-        for (int o = 4; o >= 1; o >>= 1)
+        for (int o = 2; o >= 1; o >>= 1)
 #pragma unroll
             for (int i = 0; i < o; ++i) {
                 vs[i] = N9::add(vs[i], vs[i + o]);
@@ -1984,6 +1998,69 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32) apply_kernel_nine(ApplyArgs 
             }
         finish_point(a, p, sl, N9::out(vs[0]), N9::out(qs[0]), win, n_win, n_nug, n_fail);
     }
+    const unsigned w_win = __reduce_add_sync(FULL, (unsigned)n_win);
+    const unsigned w_nug = __reduce_add_sync(FULL, (unsigned)n_nug);
+    const unsigned w_fail = __reduce_add_sync(FULL, (unsigned)n_fail);
+    if (lane == 0 && a.counters) {
+        if (w_win) atomicAdd(a.counters + CNT_WINDOW, (unsigned long long)w_win);
+        if (w_nug) atomicAdd(a.counters + CNT_NUGGET, (unsigned long long)w_nug);
+        if (w_fail) atomicAdd(a.counters + CNT_FAILED, (unsigned long long)w_fail);
+    }
+}
+
+// The same for calls too small to fill the GPU, where one lane's instructions are the time:
+// sixteen lanes a target, two targets a warp, each lane one member and one row.  Every sum has
+// apply_kernel_nine's order.  Taken up to NINE_SPREAD targets per SM, a block's worth: beyond,
+// the geometry that the sixteen lanes repeat fills the FP64 pipe.  Measured (GB300, Nside 512,
+// us; one target per lane, this form): 1 target 20.5, 12.3; 600 22.6, 14.3; 1,800 22.6, 20.5;
+// 3,600 22.6, 28.7 in FP64, double-float within 2 us of that.
+constexpr int NINE_SPREAD = 8;
+template <class R>
+__global__ void __launch_bounds__(APPLY_WARPS * 32) apply_kernel_nine_spread(ApplyArgs a) {
+    using N9 = Nine<R>;
+    using T = typename N9::T;
+    constexpr int K = 9, W = 16;
+    const int lane = threadIdx.x & 31, l = lane & (W - 1), base = lane & W;
+    unsigned long long n_win = 0, n_nug = 0, n_fail = 0;
+    const int64_t p = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / W;
+    const bool has = p < a.count;
+    double x = 0.0, y = 0.0, z = 1.0;
+    int64_t c = 0;
+    target_of(a, p, x, y, z, c);
+    const int32_t sl = __ldg(a.slot + c);
+    T cv = N9::zero(), yv = N9::zero();
+    bool win = false;
+    if (has && l < K) {
+        const int32_t m = __ldg(a.members + c * K + l);
+        if (m >= 0) N9::member(a, m, N9::pos(x), N9::pos(y), N9::pos(z), cv, yv, win);
+    }
+    const int64_t blk = (int64_t)sl * linv_len(K);
+    typename N9::Acc zc = N9::acc(), zy = N9::acc();
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+        const T cj = N9::shfl(cv, base + j), yj = N9::shfl(yv, base + j);
+        if (l >= j && l < K) {
+            const T e = N9::entry(a, blk + col_start(K, j) + l - j);
+            N9::mac(zc, e, cj);
+            N9::mac(zy, e, yj);
+        }
+    }
+    const T c1 = N9::val(zc), y1 = N9::val(zy);
+    T vs = N9::mul(c1, y1), qs = N9::mul(c1, c1);
+    // row 8 onto row 0, then halves of eight
+#pragma unroll
+    for (int o = 8; o >= 1; o >>= 1) {
+        const T tv = N9::shfl(vs, base + ((l + o) & (W - 1))), tq = N9::shfl(qs, base + ((l + o) & (W - 1)));
+        if (o == 8 ? l == 0 : (o == 4 && l > 0 && l < 4)) {  // this lane's own product is still one
+            vs = N9::fold(c1, y1, tv);
+            qs = N9::fold(c1, c1, tq);
+        } else if (o < 8 && l < o) {
+            vs = N9::add(vs, tv);
+            qs = N9::add(qs, tq);
+        }
+    }
+    const bool any_win = ((__ballot_sync(FULL, win) >> base) & 0xffffu) != 0;
+    if (has && l == 0) finish_point(a, p, sl, N9::out(vs), N9::out(qs), any_win, n_win, n_nug, n_fail);
     const unsigned w_win = __reduce_add_sync(FULL, (unsigned)n_win);
     const unsigned w_nug = __reduce_add_sync(FULL, (unsigned)n_nug);
     const unsigned w_fail = __reduce_add_sync(FULL, (unsigned)n_fail);
@@ -2676,6 +2753,12 @@ static int paper_run(flints_paper_t p, int64_t nside_tgt, int64_t first, int64_t
                 else apply_kernel_s2<36, 1><<<grid, APPLY_WARPS * 32, 0, st>>>(a);
             }
         }
+    } else if (p->K == 9 && count <= (int64_t)device_sm_count() * NINE_SPREAD) {
+        const unsigned spread = (unsigned)((count * 16 + APPLY_WARPS * 32 - 1) / (APPLY_WARPS * 32));
+        if (mixed)
+            apply_kernel_nine_spread<df><<<spread, APPLY_WARPS * 32, 0, st>>>(a);
+        else
+            apply_kernel_nine_spread<double><<<spread, APPLY_WARPS * 32, 0, st>>>(a);
     } else if (p->K == 9) {
         if (mixed)
             apply_kernel_nine<df><<<grid, APPLY_WARPS * 32, 0, st>>>(a);

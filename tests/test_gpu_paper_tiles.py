@@ -1,6 +1,7 @@
 """Launch shapes of the tabulated route chosen from the number of targets: ranges of every
-tile size of the fixed-point kernel (y = 2, FP64; one target to full tiles) have the values
-of the same range inside the whole-sky call, bit for bit."""
+tile size of the fixed-point kernel (y = 2, FP64; one target to full tiles), and ranges on
+both sides of the line between the two forms for nine members at spin 0, have the values of
+the same range inside the whole-sky call, bit for bit."""
 import pytest
 
 import workloads as wl
@@ -39,3 +40,11 @@ def test_fixed_point_tiles(fl, spin):
 
     warps = torch.cuda.get_device_properties(0).multi_processor_count * 16  # 1, 2, 8, 9 -> 16, 24, 32 targets a tile
     _ranges_equal_the_whole_sky(fl, spin, 2, "fp64", [1, 2, 31, warps, warps + 1, 8 * warps - 3, 8 * warps + 1, 17 * warps, 24 * warps + 5])
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_nine_members(fl, precision):
+    import torch
+
+    line = torch.cuda.get_device_properties(0).multi_processor_count * 8
+    _ranges_equal_the_whole_sky(fl, 0, 1, precision, [1, 2, 3, 7, 8, 9, 101, line - 1, line, line + 1, 3 * line])
