@@ -767,6 +767,9 @@ __device__ __forceinline__ bool factor_bordered(Elem *mat, int lane) {
         return bordered_cholesky<N, NB, R>(mat, lane);
 }
 
+// Both solves of a point, solve_point_fixed and solve_point below, keep one contract:
+// Returns false when a pivot of S + nugget I is not positive.
+
 // ------------------------------------------------------- fixed-point solve
 // The FP64 solve in 64-bit fixed point.  This part's FP64 pipe takes 16 cycles of an
 // SM per warp instruction, its integer multiply-add IMAD.WIDE (32 x 32 + 64 bits) half
@@ -777,9 +780,8 @@ __device__ __forceinline__ bool factor_bordered(Elem *mat, int lane) {
 // products together).  The low words' product is dropped: at most 2^-56 a term and
 // without bias, 2^-58 rms, where FP64 rounds every term of these sums, which are near 1,
 // to 2^-54; where a word meets itself (pivots, the variance) its mean is put back.
-// Measured (GB300): 1,048,583 spin-0 targets (K = 32, Nside 2048) 52.4 -> 23.6 ms; 524,309
-// Q/U targets (K = 32, Nside 4096) 61.2 -> 24.0 ms.
-// Returns false when a pivot of S + nugget I is not positive.
+// Measured (GB300): 1,048,583 spin-0 targets (K = 32, Nside 2048) 52.4 -> 22.7 ms; 524,309
+// Q/U targets (K = 32, Nside 4096) 61.2 -> 23.4 ms.
 constexpr int FXB = 59;
 
 // maximum and sum over the warp: one instruction each on the device

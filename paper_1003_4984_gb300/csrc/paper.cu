@@ -21,9 +21,10 @@
 // Per call (apply_kernel): one warp per tile of 32 targets.  Lane l displaces
 // target l and locates its coarse pixel (RING ang2pix at Nc); then per target
 // (three at a time in groups of 10 lanes for K = 9 at spin 2, one at a time for
-// K = 36; K = 9 at spin 0 keeps one target per lane, apply_kernel_nine, and FP64
-// plans at K = 36 use apply_kernel_fx where the grid allows) the lanes own stencil members l (and l + 32): c_l = xi(|n' - x_l|^2)/xi(0),
-// y_l = map[x_l]; lane i accumulates row i of z_c = L^-1 c and z_y = L^-1 y
+// K = 36; K = 9 at spin 0 keeps one target per lane, apply_kernel_nine, or
+// sixteen lanes in small calls, and FP64 plans at K = 36 use apply_kernel_fx
+// where the grid allows) the lanes own stencil members l (and l + 32):
+// c_l = xi(|n' - x_l|^2)/xi(0), y_l = map[x_l]; lane i accumulates row i of z_c = L^-1 c and z_y = L^-1 y
 // (c_j, y_j broadcast by shuffles); value = z_c . z_y and variance
 // xi(0) (1 - z_c . z_c), the kriging estimate and its error (Eqs.
 // best_temperature_field, gaussvar).
@@ -575,121 +576,121 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32) apply_kernel(ApplyArgs a) {
         }
         __syncwarp();
         const int npt = a.count - tile * 32 < 32 ? (int)(a.count - tile * 32) : 32;
-                    // one target at a time; lanes own members l and l + 32.  Consecutive
-                    // targets in one coarse pixel reuse the members' positions and data.
-                    int64_t prev = -1;
-                    double m0x = 0.0, m0y = 0.0, m0z = 0.0, y0 = 0.0, m1x = 0.0, m1y = 0.0, m1z = 0.0, y1 = 0.0;
-                    bool v0 = false, v1 = false;
-                    for (int q = 0; q < npt; ++q) {
-                        const double tx = stx[wid][q], ty = sty[wid][q], tz = stz[wid][q];
-                        const int64_t c = scp[wid][q];
-                        const int32_t sl = __ldg(a.slot + c);
-                        if (c != prev) {
-                            prev = c;
-                            const int32_t *mem = a.members + c * K;
-                            v0 = false;
-                            v1 = false;
-                            y0 = 0.0;
-                            y1 = 0.0;
-                            if (lane < K) {
-                                const int32_t m = __ldg(mem + lane);
-                                if (m >= 0) {
-                                    member_vec(a.pv, m, m0x, m0y, m0z);
-                                    y0 = __ldg(a.map + m);
-                                    v0 = true;
-                                }
-                            }
-                            if (lane + 32 < K) {
-                                const int32_t m = __ldg(mem + lane + 32);
-                                if (m >= 0) {
-                                    member_vec(a.pv, m, m1x, m1y, m1z);
-                                    y1 = __ldg(a.map + m);
-                                    v1 = true;
-                                }
-                            }
-                        }
-                        double c0 = 0.0, c1 = 0.0;
-                        bool win = false;
-                        if (v0) {
-                            const double dx = tx - m0x, dy = ty - m0y, dz = tz - m0z;
-                            const double t = dx * dx + dy * dy + dz * dz;
-                            win |= t > a.tab.t_max;
-                            c0 = table_eval<double>(a.tab, t);
-                        }
-                        if (v1) {
-                            const double dx = tx - m1x, dy = ty - m1y, dz = tz - m1z;
-                            const double t = dx * dx + dy * dy + dz * dz;
-                            win |= t > a.tab.t_max;
-                            c1 = table_eval<double>(a.tab, t);
-                        }
-                        // z_c = L^-1 c, z_y = L^-1 y from the lane-step block; c and y go to
-                        // the warp's shared slots.  Rows 0..31: lanes 2p, 2p + 1 run through
-                        // the 33 entries of rows p and 31 - p (lane 2p switches from row p
-                        // to row 31 - p after column p; the two halves of row 31 - p are
-                        // joined by a shuffle).  Rows 32..35: lane l takes row 32 + (l & 3)
-                        // on columns (l >> 2) + 8t, eight partial sums joined by shuffles.
-                        static_assert(K == 36, "the lane-step layout is laid out for K = 36");
-                        const double *Lr = a.linv + (int64_t)sl * linv_len(K);
-                        __syncwarp();
-                        sc[wid][lane] = c0;
-                        sy[wid][lane] = y0;
-                        if (lane < K - 32) {
-                            sc[wid][32 + lane] = c1;
-                            sy[wid][32 + lane] = y1;
-                        }
-                        __syncwarp();
-                        const int pp = lane >> 1, odd = lane & 1;
-                        double zca = 0.0, zya = 0.0, zc0 = 0.0, zy0 = 0.0, zc1 = 0.0, zy1 = 0.0;
-#pragma unroll
-                        for (int u = 0; u < LS_STEPS; ++u) {
-                            const int t = odd ? LS_STEPS + u : u;
-                            if (!odd && u == pp + 1) {
-                                zca = zc0;
-                                zya = zy0;
-                                zc0 = 0.0;
-                                zy0 = 0.0;
-                            }
-                            int j = t <= pp ? t : t - pp - 1;
-                            j = j < K ? j : K - 1;  // the zero pad
-                            const double e = __ldg(Lr + u * 32 + lane);
-                            zc0 = fma(e, sc[wid][j], zc0);
-                            zy0 = fma(e, sy[wid][j], zy0);
-                        }
-                        const double zcb = zc0 + __shfl_xor_sync(FULL, zc0, 1), zyb = zy0 + __shfl_xor_sync(FULL, zy0, 1);
-                        {
-                            const int g = lane >> 2;
-#pragma unroll
-                            for (int t = 0; t < LS_TAIL; ++t) {
-                                const int j = g + 8 * t < K ? g + 8 * t : K - 1;  // zero entries past the diagonal
-                                const double e = __ldg(Lr + (LS_STEPS + t) * 32 + lane);
-                                zc1 = fma(e, sc[wid][j], zc1);
-                                zy1 = fma(e, sy[wid][j], zy1);
-                            }
-#pragma unroll
-                            for (int o = 4; o < 32; o <<= 1) {
-                                zc1 += __shfl_xor_sync(FULL, zc1, o);
-                                zy1 += __shfl_xor_sync(FULL, zy1, o);
-                            }
-                        }
-                        // even lanes count rows p and 31 - p, lanes 0..3 rows 32..35, each once
-                        double v = odd ? 0.0 : zca * zya + zcb * zyb, qc = odd ? 0.0 : zca * zca + zcb * zcb;
-                        if (lane < K - 32) {
-                            v = fma(zc1, zy1, v);
-                            qc = fma(zc1, zc1, qc);
-                        }
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) {
-                            v += __shfl_xor_sync(FULL, v, o);
-                            qc += __shfl_xor_sync(FULL, qc, o);
-                        }
-                        const bool any_win = __any_sync(FULL, win);
-                        if (lane == 0) {
-                            rv[wid][q] = v;
-                            rq[wid][q] = qc;
-                            rsl[wid][q] = sl;
-                            rwin[wid][q] = any_win;
-                        }
+        // one target at a time; lanes own members l and l + 32.  Consecutive
+        // targets in one coarse pixel reuse the members' positions and data.
+        int64_t prev = -1;
+        double m0x = 0.0, m0y = 0.0, m0z = 0.0, y0 = 0.0, m1x = 0.0, m1y = 0.0, m1z = 0.0, y1 = 0.0;
+        bool v0 = false, v1 = false;
+        for (int q = 0; q < npt; ++q) {
+            const double tx = stx[wid][q], ty = sty[wid][q], tz = stz[wid][q];
+            const int64_t c = scp[wid][q];
+            const int32_t sl = __ldg(a.slot + c);
+            if (c != prev) {
+                prev = c;
+                const int32_t *mem = a.members + c * K;
+                v0 = false;
+                v1 = false;
+                y0 = 0.0;
+                y1 = 0.0;
+                if (lane < K) {
+                    const int32_t m = __ldg(mem + lane);
+                    if (m >= 0) {
+                        member_vec(a.pv, m, m0x, m0y, m0z);
+                        y0 = __ldg(a.map + m);
+                        v0 = true;
                     }
+                }
+                if (lane + 32 < K) {
+                    const int32_t m = __ldg(mem + lane + 32);
+                    if (m >= 0) {
+                        member_vec(a.pv, m, m1x, m1y, m1z);
+                        y1 = __ldg(a.map + m);
+                        v1 = true;
+                    }
+                }
+            }
+            double c0 = 0.0, c1 = 0.0;
+            bool win = false;
+            if (v0) {
+                const double dx = tx - m0x, dy = ty - m0y, dz = tz - m0z;
+                const double t = dx * dx + dy * dy + dz * dz;
+                win |= t > a.tab.t_max;
+                c0 = table_eval<double>(a.tab, t);
+            }
+            if (v1) {
+                const double dx = tx - m1x, dy = ty - m1y, dz = tz - m1z;
+                const double t = dx * dx + dy * dy + dz * dz;
+                win |= t > a.tab.t_max;
+                c1 = table_eval<double>(a.tab, t);
+            }
+            // z_c = L^-1 c, z_y = L^-1 y from the lane-step block; c and y go to
+            // the warp's shared slots.  Rows 0..31: lanes 2p, 2p + 1 run through
+            // the 33 entries of rows p and 31 - p (lane 2p switches from row p
+            // to row 31 - p after column p; the two halves of row 31 - p are
+            // joined by a shuffle).  Rows 32..35: lane l takes row 32 + (l & 3)
+            // on columns (l >> 2) + 8t, eight partial sums joined by shuffles.
+            static_assert(K == 36, "the lane-step layout is laid out for K = 36");
+            const double *Lr = a.linv + (int64_t)sl * linv_len(K);
+            __syncwarp();
+            sc[wid][lane] = c0;
+            sy[wid][lane] = y0;
+            if (lane < K - 32) {
+                sc[wid][32 + lane] = c1;
+                sy[wid][32 + lane] = y1;
+            }
+            __syncwarp();
+            const int pp = lane >> 1, odd = lane & 1;
+            double zca = 0.0, zya = 0.0, zc0 = 0.0, zy0 = 0.0, zc1 = 0.0, zy1 = 0.0;
+#pragma unroll
+            for (int u = 0; u < LS_STEPS; ++u) {
+                const int t = odd ? LS_STEPS + u : u;
+                if (!odd && u == pp + 1) {
+                    zca = zc0;
+                    zya = zy0;
+                    zc0 = 0.0;
+                    zy0 = 0.0;
+                }
+                int j = t <= pp ? t : t - pp - 1;
+                j = j < K ? j : K - 1;  // the zero pad
+                const double e = __ldg(Lr + u * 32 + lane);
+                zc0 = fma(e, sc[wid][j], zc0);
+                zy0 = fma(e, sy[wid][j], zy0);
+            }
+            const double zcb = zc0 + __shfl_xor_sync(FULL, zc0, 1), zyb = zy0 + __shfl_xor_sync(FULL, zy0, 1);
+            {
+                const int g = lane >> 2;
+#pragma unroll
+                for (int t = 0; t < LS_TAIL; ++t) {
+                    const int j = g + 8 * t < K ? g + 8 * t : K - 1;  // zero entries past the diagonal
+                    const double e = __ldg(Lr + (LS_STEPS + t) * 32 + lane);
+                    zc1 = fma(e, sc[wid][j], zc1);
+                    zy1 = fma(e, sy[wid][j], zy1);
+                }
+#pragma unroll
+                for (int o = 4; o < 32; o <<= 1) {
+                    zc1 += __shfl_xor_sync(FULL, zc1, o);
+                    zy1 += __shfl_xor_sync(FULL, zy1, o);
+                }
+            }
+            // even lanes count rows p and 31 - p, lanes 0..3 rows 32..35, each once
+            double v = odd ? 0.0 : zca * zya + zcb * zyb, qc = odd ? 0.0 : zca * zca + zcb * zcb;
+            if (lane < K - 32) {
+                v = fma(zc1, zy1, v);
+                qc = fma(zc1, zc1, qc);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                v += __shfl_xor_sync(FULL, v, o);
+                qc += __shfl_xor_sync(FULL, qc, o);
+            }
+            const bool any_win = __any_sync(FULL, win);
+            if (lane == 0) {
+                rv[wid][q] = v;
+                rq[wid][q] = qc;
+                rsl[wid][q] = sl;
+                rwin[wid][q] = any_win;
+            }
+        }
         __syncwarp();
         if (lane < npt)
             finish_point(a, tile * 32 + lane, rsl[wid][lane], rv[wid][lane], rq[wid][lane], rwin[wid][lane] != 0,
@@ -1211,7 +1212,7 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32) apply_kernel_aug(ApplyArgs a
 // the largest row sum of the target needs.
 // Member terms are formed for FX_G = 8 targets at a time, flattened over the lanes (288
 // terms, nine full passes; member by member a target needs two, the second with four
-// lanes).  Measured (GB300, 2,097,169 Q/U targets, Nside 1024): 40.5 -> 14.3 ms.
+// lanes).  Measured (GB300, 2,097,169 Q/U targets, Nside 1024): 40.5 -> 14.4 ms.
 constexpr int FX_G = 8, FX_K = 36, FXA = 58;  // FXA: units of c, y and their products, 2^-58
 
 constexpr int FX_FP64 = 1 << 20;
@@ -1746,120 +1747,120 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32) apply_kernel_df(ApplyArgs a)
         }
         __syncwarp();
         const int npt = a.count - tile * 32 < 32 ? (int)(a.count - tile * 32) : 32;
-                    static_assert(K == 36, "the split of rows 32 .. K-1 is laid out for K = 36");
-                    int64_t prev = -1;
-                    df m0x{0.0f, 0.0f}, m0y{0.0f, 0.0f}, m0z{0.0f, 0.0f}, y0{0.0f, 0.0f};
-                    df m1x{0.0f, 0.0f}, m1y{0.0f, 0.0f}, m1z{0.0f, 0.0f}, y1{0.0f, 0.0f};
-                    bool v0 = false, v1 = false;
-                    for (int q = 0; q < npt; ++q) {
-                        const df tx = stx[wid][q], ty = sty[wid][q], tz = stz[wid][q];
-                        const int64_t c = scp[wid][q];
-                        const int32_t sl = __ldg(a.slot + c);
-                        if (c != prev) {
-                            prev = c;
-                            const int32_t *mem = a.members + c * K;
-                            v0 = false;
-                            v1 = false;
-                            y0 = {0.0f, 0.0f};
-                            y1 = {0.0f, 0.0f};
-                            const int32_t mA = __ldg(mem + lane);
-                            if (mA >= 0) {
-                                member_vec_df(a.pvf, mA, m0x, m0y, m0z);
-                                y0 = split_double(__ldg(a.map + mA));
-                                v0 = true;
-                            }
-                            if (lane + 32 < K) {
-                                const int32_t mB = __ldg(mem + lane + 32);
-                                if (mB >= 0) {
-                                    member_vec_df(a.pvf, mB, m1x, m1y, m1z);
-                                    y1 = split_double(__ldg(a.map + mB));
-                                    v1 = true;
-                                }
-                            }
-                        }
-                        df c0{0.0f, 0.0f}, c1{0.0f, 0.0f};
-                        bool win = false;
-                        if (v0) {
-                            const df t = chord2_df(tx, ty, tz, m0x, m0y, m0z);
-                            win |= t.hi > tmaxf;
-                            c0 = table_eval<df>(a.tab, t);
-                        }
-                        if (v1) {
-                            const df t = chord2_df(tx, ty, tz, m1x, m1y, m1z);
-                            win |= t.hi > tmaxf;
-                            c1 = table_eval<df>(a.tab, t);
-                        }
-                        const float2 *Lr = a.linvf + (int64_t)sl * linv_len(K);
-                        __syncwarp();
-                        sc[wid][lane] = c0;
-                        sy[wid][lane] = y0;
-                        if (lane < K - 32) {
-                            sc[wid][32 + lane] = c1;
-                            sy[wid][32 + lane] = y1;
-                        }
-                        __syncwarp();
-                        // the lane-step block, as in the FP64 kernel
-                        const int pp = lane >> 1, odd = lane & 1;
-                        dfacc zca{0.0f, 0.0f}, zya{0.0f, 0.0f}, zc0{0.0f, 0.0f}, zy0{0.0f, 0.0f};
-                        dfacc zc1{0.0f, 0.0f}, zy1{0.0f, 0.0f};
-#pragma unroll
-                        for (int u = 0; u < LS_STEPS; ++u) {
-                            const int t = odd ? LS_STEPS + u : u;
-                            if (!odd && u == pp + 1) {
-                                zca = zc0;
-                                zya = zy0;
-                                zc0 = {0.0f, 0.0f};
-                                zy0 = {0.0f, 0.0f};
-                            }
-                            int j = t <= pp ? t : t - pp - 1;
-                            j = j < K ? j : K - 1;  // the zero pad
-                            const df e = ld_df(Lr + u * 32 + lane);
-                            dfacc_add_prod(zc0, e, sc[wid][j]);
-                            dfacc_add_prod(zy0, e, sy[wid][j]);
-                        }
-                        const df zc0v = dfacc_val(zc0), zy0v = dfacc_val(zy0);
-                        const df zcb = df_add_fast(zc0v, shfl_xor_df(zc0v, 1)), zyb = df_add_fast(zy0v, shfl_xor_df(zy0v, 1));
-                        df zc1v, zy1v;
-                        {
-                            const int g = lane >> 2;
-#pragma unroll
-                            for (int t = 0; t < LS_TAIL; ++t) {
-                                const int j = g + 8 * t < K ? g + 8 * t : K - 1;  // zero entries past the diagonal
-                                const df e = ld_df(Lr + (LS_STEPS + t) * 32 + lane);
-                                dfacc_add_prod(zc1, e, sc[wid][j]);
-                                dfacc_add_prod(zy1, e, sy[wid][j]);
-                            }
-                            zc1v = dfacc_val(zc1);
-                            zy1v = dfacc_val(zy1);
-#pragma unroll
-                            for (int o = 4; o < 32; o <<= 1) {
-                                zc1v = df_add_fast(zc1v, shfl_xor_df(zc1v, o));
-                                zy1v = df_add_fast(zy1v, shfl_xor_df(zy1v, o));
-                            }
-                        }
-                        const df zcav = dfacc_val(zca), zyav = dfacc_val(zya);
-                        df v{0.0f, 0.0f}, qc{0.0f, 0.0f};
-                        if (!odd) {  // even lanes count rows p and 31 - p, lanes 0..3 rows 32..35, each once
-                            v = df_add_fast(df_mul(zcav, zyav), df_mul(zcb, zyb));
-                            qc = df_add_fast(df_mul(zcav, zcav), df_mul(zcb, zcb));
-                        }
-                        if (lane < K - 32) {
-                            v = df_add_fast(v, df_mul(zc1v, zy1v));
-                            qc = df_add_fast(qc, df_mul(zc1v, zc1v));
-                        }
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) {
-                            v = df_add_fast(v, shfl_xor_df(v, o));
-                            qc = df_add_fast(qc, shfl_xor_df(qc, o));
-                        }
-                        const bool any_win = __any_sync(FULL, win);
-                        if (lane == 0) {
-                            rv[wid][q] = v;
-                            rq[wid][q] = qc;
-                            rsl[wid][q] = sl;
-                            rwin[wid][q] = any_win;
-                        }
+        static_assert(K == 36, "the split of rows 32 .. K-1 is laid out for K = 36");
+        int64_t prev = -1;
+        df m0x{0.0f, 0.0f}, m0y{0.0f, 0.0f}, m0z{0.0f, 0.0f}, y0{0.0f, 0.0f};
+        df m1x{0.0f, 0.0f}, m1y{0.0f, 0.0f}, m1z{0.0f, 0.0f}, y1{0.0f, 0.0f};
+        bool v0 = false, v1 = false;
+        for (int q = 0; q < npt; ++q) {
+            const df tx = stx[wid][q], ty = sty[wid][q], tz = stz[wid][q];
+            const int64_t c = scp[wid][q];
+            const int32_t sl = __ldg(a.slot + c);
+            if (c != prev) {
+                prev = c;
+                const int32_t *mem = a.members + c * K;
+                v0 = false;
+                v1 = false;
+                y0 = {0.0f, 0.0f};
+                y1 = {0.0f, 0.0f};
+                const int32_t mA = __ldg(mem + lane);
+                if (mA >= 0) {
+                    member_vec_df(a.pvf, mA, m0x, m0y, m0z);
+                    y0 = split_double(__ldg(a.map + mA));
+                    v0 = true;
+                }
+                if (lane + 32 < K) {
+                    const int32_t mB = __ldg(mem + lane + 32);
+                    if (mB >= 0) {
+                        member_vec_df(a.pvf, mB, m1x, m1y, m1z);
+                        y1 = split_double(__ldg(a.map + mB));
+                        v1 = true;
                     }
+                }
+            }
+            df c0{0.0f, 0.0f}, c1{0.0f, 0.0f};
+            bool win = false;
+            if (v0) {
+                const df t = chord2_df(tx, ty, tz, m0x, m0y, m0z);
+                win |= t.hi > tmaxf;
+                c0 = table_eval<df>(a.tab, t);
+            }
+            if (v1) {
+                const df t = chord2_df(tx, ty, tz, m1x, m1y, m1z);
+                win |= t.hi > tmaxf;
+                c1 = table_eval<df>(a.tab, t);
+            }
+            const float2 *Lr = a.linvf + (int64_t)sl * linv_len(K);
+            __syncwarp();
+            sc[wid][lane] = c0;
+            sy[wid][lane] = y0;
+            if (lane < K - 32) {
+                sc[wid][32 + lane] = c1;
+                sy[wid][32 + lane] = y1;
+            }
+            __syncwarp();
+            // the lane-step block, as in the FP64 kernel
+            const int pp = lane >> 1, odd = lane & 1;
+            dfacc zca{0.0f, 0.0f}, zya{0.0f, 0.0f}, zc0{0.0f, 0.0f}, zy0{0.0f, 0.0f};
+            dfacc zc1{0.0f, 0.0f}, zy1{0.0f, 0.0f};
+#pragma unroll
+            for (int u = 0; u < LS_STEPS; ++u) {
+                const int t = odd ? LS_STEPS + u : u;
+                if (!odd && u == pp + 1) {
+                    zca = zc0;
+                    zya = zy0;
+                    zc0 = {0.0f, 0.0f};
+                    zy0 = {0.0f, 0.0f};
+                }
+                int j = t <= pp ? t : t - pp - 1;
+                j = j < K ? j : K - 1;  // the zero pad
+                const df e = ld_df(Lr + u * 32 + lane);
+                dfacc_add_prod(zc0, e, sc[wid][j]);
+                dfacc_add_prod(zy0, e, sy[wid][j]);
+            }
+            const df zc0v = dfacc_val(zc0), zy0v = dfacc_val(zy0);
+            const df zcb = df_add_fast(zc0v, shfl_xor_df(zc0v, 1)), zyb = df_add_fast(zy0v, shfl_xor_df(zy0v, 1));
+            df zc1v, zy1v;
+            {
+                const int g = lane >> 2;
+#pragma unroll
+                for (int t = 0; t < LS_TAIL; ++t) {
+                    const int j = g + 8 * t < K ? g + 8 * t : K - 1;  // zero entries past the diagonal
+                    const df e = ld_df(Lr + (LS_STEPS + t) * 32 + lane);
+                    dfacc_add_prod(zc1, e, sc[wid][j]);
+                    dfacc_add_prod(zy1, e, sy[wid][j]);
+                }
+                zc1v = dfacc_val(zc1);
+                zy1v = dfacc_val(zy1);
+#pragma unroll
+                for (int o = 4; o < 32; o <<= 1) {
+                    zc1v = df_add_fast(zc1v, shfl_xor_df(zc1v, o));
+                    zy1v = df_add_fast(zy1v, shfl_xor_df(zy1v, o));
+                }
+            }
+            const df zcav = dfacc_val(zca), zyav = dfacc_val(zya);
+            df v{0.0f, 0.0f}, qc{0.0f, 0.0f};
+            if (!odd) {  // even lanes count rows p and 31 - p, lanes 0..3 rows 32..35, each once
+                v = df_add_fast(df_mul(zcav, zyav), df_mul(zcb, zyb));
+                qc = df_add_fast(df_mul(zcav, zcav), df_mul(zcb, zcb));
+            }
+            if (lane < K - 32) {
+                v = df_add_fast(v, df_mul(zc1v, zy1v));
+                qc = df_add_fast(qc, df_mul(zc1v, zc1v));
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                v = df_add_fast(v, shfl_xor_df(v, o));
+                qc = df_add_fast(qc, shfl_xor_df(qc, o));
+            }
+            const bool any_win = __any_sync(FULL, win);
+            if (lane == 0) {
+                rv[wid][q] = v;
+                rq[wid][q] = qc;
+                rsl[wid][q] = sl;
+                rwin[wid][q] = any_win;
+            }
+        }
         __syncwarp();
         if (lane < npt)
             finish_point(a, tile * 32 + lane, rsl[wid][lane], df_to(rv[wid][lane]), df_to(rq[wid][lane]),
@@ -1882,7 +1883,8 @@ __global__ void __launch_bounds__(APPLY_WARPS * 32) apply_kernel_df(ApplyArgs a)
 // loads are independent of one another (27 in flight where a group of ten lanes had one
 // chain of four), every lane works on every multiply-add of the 45-entry factor, and nothing
 // is exchanged between lanes.  The sums run in the order of the ten-lane groups that this
-// replaced (column by column, the rows' products by halving).  What bounds it: the FP64 target geometry (200 FP64 instructions a tile).
+// replaced (column by column, the rows' products by halving).  What bounds it: the FP64
+// target geometry (200 FP64 instructions a tile).
 // Measured (GB300, the Nside 2048 sky, double-float): 32.4 -> 22.7 ms.
 template <class R>
 struct Nine;
