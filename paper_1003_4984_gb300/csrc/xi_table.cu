@@ -138,7 +138,8 @@ __global__ void fixed_table_kernel(const Coef64 *__restrict__ c64, int n, CoefFx
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     const Coef64 c = c64[k];
-    cfx[k] = CoefFx{fx_of(c.f, 59), fx_of(c.m, 59), fx_of(c.c2, 59), fx_of(c.c3, 59)};
+    const double u = 576460752303423488.0;  // 2^59
+    cfx[k] = CoefFx{(int64_t)rint(c.f * u), (int64_t)rint(c.m * u), (int64_t)rint(c.c2 * u), (int64_t)rint(c.c3 * u)};
 }
 
 cudaError_t launch_xi_table(int spin, int lmax, const double *cl_dev, const double *clbb_dev, double t_max,
