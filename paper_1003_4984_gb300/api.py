@@ -535,8 +535,9 @@ class PaperPlan:
     """The paper's stencil with tabulated inverses (flints_paper_*): level-y
     pixel-centred stencil of 9 * 4^(y-1) pixels, L^-1 (the factor of S^-1)
     tabulated per symmetry class of central pixels, two triangular
-    matrix-vector products per target (spin 0; precision "fp64" or "mixed",
-    the per-target arithmetic in double-float on the FP32 pipe)."""
+    matrix-vector products per target (spin 0, 1, 2; precision "fp64" or
+    "mixed", the per-target arithmetic in double-float on the FP32 pipe: the
+    faster one but for y = 2 at spin 1 and 2, where "fp64" is faster)."""
 
     def __init__(self, nside: int, cl, y: int = 1, precision: str = "fp64", spin: int = 0, cl_bb=None,
                  augmented: bool = False, stream=None):

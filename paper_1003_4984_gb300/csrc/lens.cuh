@@ -855,8 +855,9 @@ __device__ __forceinline__ bool fx_beyond(int64_t v, int lim) {
 // diagonal is not read again).  Matrix rows beyond 1.9 (not a factor of a positive
 // matrix) end it: false, the caller's FP64 path decides.  The last bordered row holds the
 // data, scaled by its caller below 2^-FxData::expo; its solve has no bound, and where an entry
-// passes 1.9 / 2^room the row is shifted down by 3 bits (counted in ey) and the panel's slot
-// redone: the largest entry of the row keeps at least 53 bits.
+// passes 1.9 / 2^room the row is shifted down (counted in ey) and the panel's slot redone: by
+// 5 bits, which leaves the rounding of the largest entry at 2^-53 of it, as in FP64, and by 8
+// once data that is no realisation of the field has passed that too.
 // The sums here are taken modulo 32, and on a matrix that is not positive a row can be longer
 // than that before its own pivot says so.  A row's squared length is therefore also read from
 // the high words' sums, which hold 512 (n = 96 terms of at most 1.9^2 each are 347): where a
@@ -991,14 +992,15 @@ __device__ __forceinline__ bool factor_fixed(E *mat, int lane, int &ey) {
                 }
                 if (__ballot_sync(FULL, bad)) return false;
                 if (__ballot_sync(FULL, high)) {
-                    if (++grown > 20) return false;
-                    ey += 3;
+                    const int down = grown++ ? 8 : 5;
+                    if (grown > 8) return false;
+                    ey += down;
                     for (int k = lane; k < N; k += 32) {
                         E *y = mat + tri<N>(NROW - 1, k);
                         if constexpr (CPLX) {
-                            *y = E{fx_split_all((fx_val(y->re) + 4) >> 3), fx_split_all((fx_val(y->im) + 4) >> 3)};
+                            *y = E{fx_split_all((fx_val(y->re) + (1 << (down - 1))) >> down), fx_split_all((fx_val(y->im) + (1 << (down - 1))) >> down)};
                         } else {
-                            *y = fx_split_all((fx_val(*y) + 4) >> 3);
+                            *y = fx_split_all((fx_val(*y) + (1 << (down - 1))) >> down);
                         }
                     }
                     __syncwarp();
