@@ -1,5 +1,5 @@
 """Tile sizes that a batch chooses (csrc/api.cu, flints_batch_stage) on the host: per class
-the size that balances the batch's targets over the warps which that class's kernel keeps
+the size that balances that class's targets over the warps which its kernel keeps
 resident (the stand-in's occupancy: two blocks per SM of the warps that fit), as plan
 calls choose it; a tile size of the caller's is taken as it is."""
 import numpy as np
@@ -25,6 +25,7 @@ int main() {
     flints_batch_t b = nullptr;
     if (flints_batch_create(&b, 64)) return 4;
     while (scanf("%lld %d", &count, &tile) == 2) {
+        int64_t own[BATCH_CLASSES] = {0};
         std::vector<flints_job> jobs;  // `count` targets in jobs of at most a sky, plans in turn
         for (long long left = count; left > 0; left -= jobs.back().count) {
             flints_job j{};
@@ -33,11 +34,13 @@ int main() {
             j.out = buf;
             j.count = left < 3072 ? left : 3072;
             jobs.push_back(j);
+            const int *k = kinds[(jobs.size() - 1) % 3];
+            own[8 * k[2] + (k[0] == 2 ? 4 : 0) + batch_k_index(k[1])] += j.count;
         }
         if (flints_batch_stage(b, jobs.data(), (int)jobs.size(), tile)) return 5;
         for (int cls = 0; cls < BATCH_CLASSES; ++cls)
             printf("%d %d\n", hdr_of(b->h_buf)->tile_pts[cls],
-                   tile ? tile : auto_tile_points(count, (int64_t)152 * 2 * b->wpb[cls]));
+                   tile ? tile : auto_tile_points(own[cls], (int64_t)152 * 2 * b->wpb[cls]));
     }
     flints_batch_free(b);
     for (flints_plan_t q : p) flints_free(q);
