@@ -220,7 +220,7 @@ int flints_lens_batch(const flints_job *jobs, int n, void *stream);
  *     max_jobs jobs, plus pinned host staging (allocates; not capturable).
  *   flints_batch_stage: host-only: validate the jobs, order them by precision
  *     class and decreasing estimated cost, cut them into tiles of tile_points
- *     targets (1..16; 0: chosen from the batch's target count), write the table
+ *     targets (1..16; 0: chosen per class from its target count), write the table
  *     into the pinned staging buffer.
  *   flints_batch_launch: upload the staged table, reset the work queues and
  *     launch the persistent class kernels on `stream` and on streams of the
@@ -368,7 +368,9 @@ void flints_free(flints_plan_t plan);
  *   precision FLINTS_FP64, or FLINTS_MIXED: the per-target chords,
  *   correlation lookups and triangular products in double-float on the FP32
  *   pipe (target position and location FP64; the L^-1 blocks computed in FP64
- *   and kept as double-float).
+ *   and kept as double-float).  At y = 2 for spin 1 and 2 FLINTS_FP64 is the
+ *   faster precision, not only the more accurate one (its products run in 64-bit
+ *   fixed point); elsewhere FLINTS_MIXED is.
  *   Builds on `stream` the xi table(s) on [0, min((7 / Nside_c)^2, 4)]
  *   (interval count by the rule of flints_plan), a table of the map pixels'
  *   positions (and frames, spin 1, 2), the stencil table and the L^-1 blocks,
